@@ -48,6 +48,8 @@ struct rlbm_ctx {
   int fused = 0;                 // 1: M1, 2: G1..G6, 3: E5, 4: S2; 0: generic kernel
   int ext = 0;                   // FP32 storage on a compiled stencil: extended moment sums
   std::unique_ptr<FusedParams> fp;
+  int fused64 = 0;               // FP64 storage: compiled kernel of the same stencils (0: generic)
+  std::unique_ptr<Fused64Params> fp64;
   // third-order stencils (eleven groups)
   int order = 2;
   std::unique_ptr<StencilBuildO3> sb3;
@@ -126,6 +128,13 @@ static void fill_params(rlbm_ctx* c, StepParams<CT>* p) {
   fill_pop_table<CT>(c->sb, c->Nx, c->Ny, &p->pt);
 }
 
+static int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 1;
+  return n;
+}
+
 static HL split(double x) {
   HL h;
   h.hi = (float)x;
@@ -133,9 +142,9 @@ static HL split(double x) {
   return h;
 }
 
-// Which stencil-specialised kernel serves this context (0: none).
-static int fused_kind(const rlbm_ctx* c) {
-  if (c->dtype == RLBM_F64) return 0;
+// The compiled second-order stencil of this context (0: none): its groups, in
+// the compiled population order (same storage planes).
+static int stencil_kind(const rlbm_ctx* c) {
   auto same = [&](const int* g) {
     for (int k = 0; k < 6; ++k)
       if (c->sb.groups[k] != g[k]) return false;
@@ -148,15 +157,49 @@ static int fused_kind(const rlbm_ctx* c) {
   else if (same(StencilE5::groups)) kind = 3, F = &StencilE5::F;
   else if (same(StencilS2::groups)) kind = 4, F = &StencilS2::F;
   if (!kind || F->Q != c->Q || F->halo != c->sb.halo) return 0;
-  // the compiled population order must be the host's (same storage planes)
   for (int i = 0; i < F->Q; ++i) {
     const FoldedPop& fp = c->sb.pops[i];
     if (fp.nx != F->nx[i] || fp.ny != F->ny[i] || fp.group != F->grp[i] || fp.mult != F->mult[i]) return 0;
   }
-  const int halo = F->halo;
+  return kind;
+}
+
+// Which stencil-specialised FP32 / BF16 kernel serves this context (0: none).
+static int fused_kind(const rlbm_ctx* c) {
+  if (c->dtype == RLBM_F64) return 0;
+  const int halo = c->sb.halo;
   // the kernels wrap a source coordinate at most once
   if (c->Nx < halo || c->Ny < halo) return 0;
-  return kind;
+  return stencil_kind(c);
+}
+
+// Displacements -6..6 reduced modulo the lattice (any lattice size).
+static void fill_disp(int Nx, int Ny, int (&dxm)[13], int (&dym)[13]) {
+  for (int d = -6; d <= 6; ++d) {
+    dxm[d + 6] = ((d % Nx) + Nx) % Nx;
+    dym[d + 6] = ((d % Ny) + Ny) % Ny;
+  }
+}
+
+static void fill_fused64(rlbm_ctx* c) {
+  Fused64Params& f = *c->fp64;
+  std::memset(&f, 0, sizeof f);
+  f.Nx = c->Nx;
+  f.Ny = c->Ny;
+  f.pitch = c->pitch;
+  f.plane = c->plane;
+  f.inv_tau = 1.0 / c->tau;
+  f.v0 = c->sb.v0;
+  f.sc = c->sb.sc;
+  for (int g = 0; g < 6; ++g) {
+    for (int q = 0; q < 5; ++q) f.gm[g][q] = c->sb.gm[g][q];
+    for (int q = 0; q < 10; ++q) f.gf[g][q] = c->sb.gf[g][q];
+  }
+  fill_disp(c->Nx, c->Ny, f.dxm, f.dym);
+  f.sms = sm_count();
+  f.rt64 = c->d_rt64;
+  f.rt32 = c->d_rt32;
+  f.err = c->d_err;
 }
 
 static void fill_fused(rlbm_ctx* c, double nref) {
@@ -581,6 +624,10 @@ rlbm_status rlbm_create(const rlbm_stencil* st, double m, double tau, int Nx, in
     c->fp.reset(new FusedParams);
     fill_fused(c.get(), 1.0);
   }
+  if (dtype == RLBM_F64 && (c->fused64 = stencil_kind(c.get())) != 0) {
+    c->fp64.reset(new Fused64Params);
+    fill_fused64(c.get());
+  }
   if (dtype == RLBM_BF16_DEV) {
     if (!c->fused) {
       release(c.get());
@@ -692,6 +739,7 @@ rlbm_status rlbm_step(rlbm_ctx* c, int nsteps) {
     if (c->order == 3)
       e = c->fo3 ? launch_fused_o3(c->fused, *c->fo3, fin, fout, c->stream)
                  : launch_step_o3(c->dtype, *c->o3, fin, fout, c->stream);
+    else if (c->fused64) e = launch_fused_f64(c->fused64, *c->fp64, fin, fout, c->stream);
     else if (c->dtype == RLBM_F64) e = launch_step_f64(*c->p64, fin, fout, c->qb, c->stream);
     else if (c->fused) {
       const int mode = fused_mode(c);

@@ -158,6 +158,25 @@ struct FusedParams {
   int doff[kMaxQ2], dcoff[kMaxQ2];
 };
 
+// Stencil-specialised FP64 step (rlbm_fused64.cu): group momenta gm and folded
+// equilibrium constants gf of StencilBuild in FP64; dxm, dym: displacement D
+// at [D + 6], reduced modulo the lattice into [0, N).
+struct Fused64Params {
+  int Nx, Ny;
+  long long pitch, plane;     // elements
+  double inv_tau, v0;
+  SiteConsts sc;
+  double gm[6][5], gf[6][10];
+  int dxm[13], dym[13];
+  int sms;                    // SMs of the device (block size of small lattices)
+  const double* rt64;
+  const float* rt32;
+  unsigned* err;
+};
+
+// kind 1..4: the stencils of rlbm_info.kernel
+cudaError_t launch_fused_f64(int kind, const Fused64Params& p, const void* fin, void* fout, cudaStream_t s);
+
 // One lattice of a persistent batch launch (device memory; rlbm_persist.cuh).
 struct PersistLattice {
   FusedParams p[2];       // step parameters for S_t in buf[0] / buf[1] (BF16 coefficient planes set)
