@@ -22,8 +22,8 @@
 // 504 -> 240 us against step_o3_kernel.
 // The populations are pulled twice (the second pull hits L1/L2) instead of
 // being held in 116 registers: 128 registers, eight blocks of 64 threads an SM
-(65536 sites are 6.7 such blocks an SM; blocks of 128 left the SMs with four of
-them to finish 9 % later).
+// (65536 sites are 6.7 such blocks an SM; blocks of 128 left the SMs with four of
+// them to finish 9 % later).
 #pragma once
 
 #include <utility>
