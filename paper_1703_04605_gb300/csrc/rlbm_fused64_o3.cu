@@ -1,0 +1,157 @@
+// Stencil-specialised FP64 third-order step (storage f_i, all arithmetic FP64;
+// rlbm_fused64.cuh).  Equilibrium f^eq_i = n wr_i + sum_l e_l W_il, e_l = n dmu_l
+// (rlbm_o3.cuh), summed once a reflection orbit over the parity classes of the
+// twenty monomials (as rlbm_fused_o3.cu): 21 FP64 instructions a quartet of
+// populations instead of 84.
+#include "rlbm_fused64.cuh"
+#include "rlbm_o3.cuh"
+
+namespace rlbm {
+namespace {
+
+// Parity classes of the centred monomials (kO3Mono order).
+using EE = std::integer_sequence<int, 0, 1, 6, 7, 9, 10, 11, 17>;   // even in p_x and p_y
+using OE = std::integer_sequence<int, 2, 4, 13, 15, 18>;            // odd in p_x only
+using EO = std::integer_sequence<int, 3, 5, 14, 16, 19>;            // odd in p_y only
+using OO = std::integer_sequence<int, 8, 12>;                       // odd in both
+
+template <int... L>
+__device__ __forceinline__ double sum64(std::integer_sequence<int, L...>, const double* w, const double (&e)[kO3Mono],
+                                        double acc) {
+  ((acc = fma(w[1 + L], e[L], acc)), ...);
+  return acc;
+}
+
+__device__ __forceinline__ void deviations64(const FusedO364Params& p, const Macro<double>& o, double (&e)[kO3Mono]) {
+  o3_deviations<double>(p.sc.mbar, p.c, o.n, o.U0, o.Ux, o.Uy, o.dU, o.dR, o.T - 1.0, o.T, o.R, e, p.sc.inv_m);
+}
+
+template <class Def, int K>
+__device__ __forceinline__ void collide64_orbit(const FusedO364Params& p, const double (&e)[kO3Mono], double n,
+                                                const Pull64& q, const Relax64& rx) {
+  constexpr int kind = Def::O.kind[K];
+  const double* w = p.ow[K];
+  const double E = sum64(EE{}, w, e, w[0] * n);
+  double X = 0.0, Y = 0.0, Z = 0.0;
+  if constexpr (kind == 2 || kind == 4) X = sum64(OE{}, w, e, 0.0);
+  if constexpr (kind == 3 || kind == 4) Y = sum64(EO{}, w, e, 0.0);
+  if constexpr (kind == 4) Z = sum64(OO{}, w, e, 0.0);
+  relax64_orbit<Def, K>(q, rx, E, X, Y, Z);
+}
+
+template <class Def, int... Ks>
+__device__ __forceinline__ void collide64_all(std::integer_sequence<int, Ks...>, const FusedO364Params& p,
+                                              const double (&e)[kO3Mono], double n, const Pull64& q,
+                                              const Relax64& rx) {
+  (collide64_orbit<Def, Ks>(p, e, n, q, rx), ...);
+}
+
+template <class Def>
+__global__ void __launch_bounds__(64, 6) fused_f64_o3_kernel(const __grid_constant__ FusedO364Params p,
+                                                             const double* __restrict__ fin,
+                                                             double* __restrict__ fout) {
+  static_assert(Def::halo <= kMaxDisp && Def::O.K <= kMaxOrbO3, "table sizes");
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned fl = 0;
+  if (s < p.Nx * p.Ny) {
+    int x, y;
+    site_of(s, p.Nx, x, y);
+    const Pull64 q{fin, (size_t)p.plane, (unsigned)p.pitch, x, y, p.Nx, p.Ny, p.dxm, p.dym};
+    using Orb = std::make_integer_sequence<int, Def::O.K>;
+    double M[9];
+    acc64_all<Def>(Orb{}, q, p.gm, M);
+    const Macro<double> o = solve_site_f64_seeded(M, p.sc, p.rt64, p.rt32, fl);
+    double e[kO3Mono];
+    deviations64(p, o, e);
+    const double wv = p.v0 * p.inv_tau;
+    const Relax64 rx{o.U0 * p.inv_tau, wv * o.Ux, wv * o.Uy, fout + ((unsigned)y * (unsigned)p.pitch + (unsigned)x),
+                     (size_t)p.plane};
+    collide64_all<Def>(Orb{}, p, e, o.n, q, rx);
+  }
+  report(fl, p.err);
+}
+
+// Four lanes a site (rlbm_fused64.cuh): the signs of a lane go into the odd e_l.
+template <class Def, int K>
+__device__ __forceinline__ void lane_collide(const FusedO364Params& p, const Lane64& q, const double (&d)[Def::O.K],
+                                             const double (&e)[kO3Mono], double n, double a0, double wx, double wy) {
+  constexpr int kind = Def::O.kind[K], ax = Def::O.ax[K], ay = Def::O.ay[K];
+  const double* w = p.ow[K];
+  double f = sum64(EE{}, w, e, w[0] * n);
+  if constexpr (kind == 4) f = sum64(OO{}, w, e, f);
+  if constexpr (kind == 2 || kind == 4) f = sum64(OE{}, w, e, f);
+  if constexpr (kind == 3 || kind == 4) f = sum64(EO{}, w, e, f);
+  double om = a0;
+  if constexpr (ax != 0) om = fma(-(double)ax, wx, om);
+  if constexpr (ay != 0) om = fma(-(double)ay, wy, om);
+  if (lane_has<Def, K>(q.l)) __stcs(q.out + q.here + lane_plane<Def, K>(q), fma(om, f - d[K], d[K]));
+}
+
+template <class Def, int... Ks>
+__device__ __forceinline__ void lane_collide_all(std::integer_sequence<int, Ks...>, const FusedO364Params& p,
+                                                 const Lane64& q, const double (&d)[Def::O.K],
+                                                 const double (&e)[kO3Mono], double n, double a0, double wx,
+                                                 double wy) {
+  (lane_collide<Def, Ks>(p, q, d, e, n, a0, wx, wy), ...);
+}
+
+template <int... L>
+__device__ __forceinline__ void flip_all(std::integer_sequence<int, L...>, double (&e)[kO3Mono], int negative) {
+  ((e[L] = flip(e[L], negative)), ...);
+}
+
+template <class Def>
+__global__ void __launch_bounds__(32) fused_f64_o3_quad_kernel(const __grid_constant__ FusedO364Params p,
+                                                               const double* __restrict__ fin,
+                                                               double* __restrict__ fout) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int nsite = p.Nx * p.Ny;
+  const bool live = (t >> 2) < nsite;
+  const int site = live ? t >> 2 : nsite - 1;
+  unsigned fl = 0;
+  int x, y;
+  site_of(site, p.Nx, x, y);
+  const Lane64 q{fin, fout, (size_t)p.plane, (unsigned)p.pitch, (unsigned)y * (unsigned)p.pitch + (unsigned)x, x, y,
+                 p.Nx, p.Ny, t & 3, p.dxm, p.dym};
+  using Orb = std::make_integer_sequence<int, Def::O.K>;
+  double d[Def::O.K], M[9];
+  lane_moments_all<Def>(Orb{}, q, d, p.gm, M);
+  const Macro<double> o = solve_site_f64_seeded(M, p.sc, p.rt64, p.rt32, fl);
+  double e[kO3Mono];
+  deviations64(p, o, e);
+  flip_all(OE{}, e, q.l & 1);
+  flip_all(EO{}, e, q.l >> 1);
+  flip_all(OO{}, e, (q.l ^ (q.l >> 1)) & 1);
+  const double wv = p.v0 * p.inv_tau;
+  if (live)
+    lane_collide_all<Def>(Orb{}, p, q, d, e, o.n, o.U0 * p.inv_tau, flip(wv * o.Ux, q.l & 1),
+                          flip(wv * o.Uy, q.l >> 1));
+  report(fl, p.err);
+}
+
+template <class Def>
+cudaError_t launch64(const FusedO364Params& p, const void* fin, void* fout, cudaStream_t s) {
+  const long long nsite = (long long)p.Nx * p.Ny;
+  if (nsite <= kQuadSites * p.sms)
+    fused_f64_o3_quad_kernel<Def><<<(unsigned)((nsite + 7) / 8), 32, 0, s>>>(p, static_cast<const double*>(fin),
+                                                                             static_cast<double*>(fout));
+  else
+    fused_f64_o3_kernel<Def><<<(unsigned)((nsite + 63) / 64), 64, 0, s>>>(p, static_cast<const double*>(fin),
+                                                                          static_cast<double*>(fout));
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_fused_f64_o3(int kind, const FusedO364Params& p, const void* fin, void* fout, cudaStream_t s) {
+  switch (kind) {
+    case 5: return launch64<StencilO3M5>(p, fin, fout, s);
+    case 6: return launch64<StencilO3D>(p, fin, fout, s);
+    case 7: return launch64<StencilO3E>(p, fin, fout, s);
+    case 8: return launch64<StencilO3A>(p, fin, fout, s);
+    case 9: return launch64<StencilO3B>(p, fin, fout, s);
+    default: return launch64<StencilO3C>(p, fin, fout, s);
+  }
+}
+
+}  // namespace rlbm

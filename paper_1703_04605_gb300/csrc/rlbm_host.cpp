@@ -54,6 +54,7 @@ struct rlbm_ctx {
   int order = 2;
   std::unique_ptr<StencilBuildO3> sb3;
   std::unique_ptr<O3Params> o3;
+  std::unique_ptr<FusedO364Params> fo364;   // compiled FP64 third-order kernel (fused64 5..10)
   std::unique_ptr<FusedO3Params> fo3;   // compiled third-order kernel (fused == 5)
   int* d_shift = nullptr;
   long long* d_off = nullptr;
@@ -306,10 +307,9 @@ static bool fused_o3_is(const rlbm_ctx* c) {
   return true;
 }
 
-// Which compiled third-order kernel serves this context (0: none): FP32,
-// compiled groups in the host's population order, Nx, Ny >= halo.
-static int fused_o3_kind(const rlbm_ctx* c) {
-  if (c->dtype != RLBM_F32 || c->Nx < c->sb3->halo || c->Ny < c->sb3->halo) return 0;
+// The compiled third-order stencil of this context (0: none): compiled groups
+// in the host's population order.
+static int stencil_o3_kind(const rlbm_ctx* c) {
   if (fused_o3_is<StencilO3M5>(c)) return 5;
   if (fused_o3_is<StencilO3D>(c)) return 6;
   if (fused_o3_is<StencilO3E>(c)) return 7;
@@ -319,12 +319,56 @@ static int fused_o3_kind(const rlbm_ctx* c) {
   return 0;
 }
 
-template <class D>
-static void fill_orbits_o3(const StencilBuildO3& sb, FusedO3Params& f) {
+// Which compiled FP32 third-order kernel serves this context (0: none): the
+// kernels wrap a source coordinate at most once, so Nx, Ny >= halo.
+static int fused_o3_kind(const rlbm_ctx* c) {
+  if (c->dtype != RLBM_F32 || c->Nx < c->sb3->halo || c->Ny < c->sb3->halo) return 0;
+  return stencil_o3_kind(c);
+}
+
+static void set_const(HL& c, double v) { c = split(v); }
+static void set_const(double& c, double v) { c = v; }
+
+template <class D, class P>
+static void fill_orbits_o3(const StencilBuildO3& sb, P& f) {
   for (int k = 0; k < D::O.K; ++k) {
     const auto& row = sb.rows[D::O.idx[k][0]];
-    for (int l = 0; l <= kO3Mono; ++l) f.ow[k][l] = split(row[9 + l]);
+    for (int l = 0; l <= kO3Mono; ++l) set_const(f.ow[k][l], row[9 + l]);
   }
+}
+
+template <class P>
+static void fill_orbits_o3(int kind, const StencilBuildO3& sb, P& f) {
+  switch (kind) {
+    case 5: fill_orbits_o3<StencilO3M5>(sb, f); break;
+    case 6: fill_orbits_o3<StencilO3D>(sb, f); break;
+    case 7: fill_orbits_o3<StencilO3E>(sb, f); break;
+    case 8: fill_orbits_o3<StencilO3A>(sb, f); break;
+    case 9: fill_orbits_o3<StencilO3B>(sb, f); break;
+    default: fill_orbits_o3<StencilO3C>(sb, f); break;
+  }
+}
+
+static void fill_fused_o364(rlbm_ctx* c) {
+  FusedO364Params& f = *c->fo364;
+  std::memset(&f, 0, sizeof f);
+  const StencilBuildO3& sb = *c->sb3;
+  f.Nx = c->Nx;
+  f.Ny = c->Ny;
+  f.pitch = c->pitch;
+  f.plane = c->plane;
+  f.inv_tau = 1.0 / c->tau;
+  f.v0 = sb.v0;
+  f.c = sb.c;
+  f.sc = sb.sc;
+  for (int g = 0; g < 11; ++g)
+    for (int q = 0; q < 5; ++q) f.gm[g][q] = sb.gm[g][q];
+  fill_orbits_o3(c->fused64, sb, f);
+  fill_disp(c->Nx, c->Ny, f.dxm, f.dym);
+  f.sms = sm_count();
+  f.rt64 = c->d_rt64;
+  f.rt32 = c->d_rt32;
+  f.err = c->d_err;
 }
 
 static void fill_fused_o3(rlbm_ctx* c, double nref) {
@@ -350,14 +394,7 @@ static void fill_fused_o3(rlbm_ctx* c, double nref) {
   f.mb64 = sb.mbar;
   for (int g = 0; g < 11; ++g)
     for (int q = 0; q < 5; ++q) f.gm[g][q] = split(sb.gm[g][q]);
-  switch (c->fused) {
-    case 5: fill_orbits_o3<StencilO3M5>(sb, f); break;
-    case 6: fill_orbits_o3<StencilO3D>(sb, f); break;
-    case 7: fill_orbits_o3<StencilO3E>(sb, f); break;
-    case 8: fill_orbits_o3<StencilO3A>(sb, f); break;
-    case 9: fill_orbits_o3<StencilO3B>(sb, f); break;
-    default: fill_orbits_o3<StencilO3C>(sb, f); break;
-  }
+  fill_orbits_o3(c->fused, sb, f);
   f.rt64 = c->d_rt64;
   f.rt32 = c->d_rt32;
   f.dr64 = c->d_dr64;
@@ -519,6 +556,10 @@ static rlbm_status create_o3(const rlbm_stencil* st, double m, double tau, int N
   if (c->fused) {
     c->fo3.reset(new FusedO3Params);
     fill_fused_o3(c.get(), 1.0);
+  }
+  if (dtype == RLBM_F64 && (c->fused64 = stencil_o3_kind(c.get())) != 0) {
+    c->fo364.reset(new FusedO364Params);
+    fill_fused_o364(c.get());
   }
   *out = c.release();
   return RLBM_OK;
@@ -737,8 +778,9 @@ rlbm_status rlbm_step(rlbm_ctx* c, int nsteps) {
     void* fout = c->buf[1 - c->cur];
     cudaError_t e;
     if (c->order == 3)
-      e = c->fo3 ? launch_fused_o3(c->fused, *c->fo3, fin, fout, c->stream)
-                 : launch_step_o3(c->dtype, *c->o3, fin, fout, c->stream);
+      e = c->fo3     ? launch_fused_o3(c->fused, *c->fo3, fin, fout, c->stream)
+          : c->fo364 ? launch_fused_f64_o3(c->fused64, *c->fo364, fin, fout, c->stream)
+                     : launch_step_o3(c->dtype, *c->o3, fin, fout, c->stream);
     else if (c->fused64) e = launch_fused_f64(c->fused64, *c->fp64, fin, fout, c->stream);
     else if (c->dtype == RLBM_F64) e = launch_step_f64(*c->p64, fin, fout, c->qb, c->stream);
     else if (c->fused) {

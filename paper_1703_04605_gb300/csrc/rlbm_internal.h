@@ -285,6 +285,25 @@ struct FusedO3Params {
   unsigned* err;
 };
 
+// Stencil-specialised FP64 third-order step (rlbm_fused64_o3.cu): ow as
+// FusedO3Params, the rest as Fused64Params.
+struct FusedO364Params {
+  int Nx, Ny;
+  long long pitch, plane;
+  double inv_tau, v0, c;
+  SiteConsts sc;
+  double gm[11][5];
+  double ow[kMaxOrbO3][21];
+  int dxm[13], dym[13];
+  int sms;
+  const double* rt64;
+  const float* rt32;
+  unsigned* err;
+};
+
+// kind 5..10 as launch_fused_o3
+cudaError_t launch_fused_f64_o3(int kind, const FusedO364Params& p, const void* fin, void* fout, cudaStream_t s);
+
 // kind 5, 6, 7: groups {1,2,5,6,7,9,10,11,12,13,15}, {2,3,5,6,7,8,9,10,11,13,15},
 // {1,2,3,6,7,8,9,10,11,13,15}; 8, 9, 10: {8,15,20,24,26,27,28,30,36,37,42},
 // {4,10,15,20,24,26,27,28,30,36,37}, {4,8,14,15,16,17,18,21,22,23,26}

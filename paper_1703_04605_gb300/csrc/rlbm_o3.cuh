@@ -21,10 +21,10 @@ __device__ __forceinline__ float o3_fma(float a, float b, float c) { return fmaf
 __device__ __forceinline__ double o3_rcp(double a) { return 1.0 / a; }
 __device__ __forceinline__ float o3_rcp(float a) { return __fdividef(1.0f, a); }
 
-// e_l = n dmu_l (kO3Mono order); m = m/T_R, c the centring shift of t.
+// e_l = n dmu_l (kO3Mono order); m = m/T_R, c the centring shift of t, im = 1/m.
 template <typename R_t>
 __device__ __forceinline__ void o3_deviations(R_t m, R_t c, R_t n, R_t U0, R_t Ux, R_t Uy, R_t dU, R_t dR,
-                                              R_t dT, R_t T, R_t R, R_t (&e)[kO3Mono]) {
+                                              R_t dT, R_t T, R_t R, R_t (&e)[kO3Mono], R_t im) {
   const R_t h = o3_fma(m, R, R_t(4) * T);
   const R_t dh = o3_fma(m, dR, R_t(4) * dT);
   const R_t Th = T * h;
@@ -32,7 +32,7 @@ __device__ __forceinline__ void o3_deviations(R_t m, R_t c, R_t n, R_t U0, R_t U
   const R_t hU = o3_fma(h, U0, -c);
   const R_t sdev = o3_fma(dT, hU, o3_fma(h, dU, dh));   // T (h U0 - c) - (h_r - c)
   const R_t q = o3_fma(Am, U0, -c * h);
-  const R_t dRm = dR * o3_rcp(m);
+  const R_t dRm = dR * im;
   const R_t Ux2 = Ux * Ux, Uy2 = Uy * Uy, Uxy = Ux * Uy;
   e[0] = n * dRm;                                    // 1
   e[1] = n * o3_fma(-c, dRm, dU);                    // t
@@ -54,6 +54,12 @@ __device__ __forceinline__ void o3_deviations(R_t m, R_t c, R_t n, R_t U0, R_t U
   e[17] = n * sdev;                                  // t pz^2
   e[18] = e[2] * Th;                                 // px pz^2
   e[19] = e[3] * Th;                                 // py pz^2
+}
+
+template <typename R_t>
+__device__ __forceinline__ void o3_deviations(R_t m, R_t c, R_t n, R_t U0, R_t Ux, R_t Uy, R_t dU, R_t dR,
+                                              R_t dT, R_t T, R_t R, R_t (&e)[kO3Mono]) {
+  o3_deviations<R_t>(m, c, n, U0, Ux, Uy, dU, dR, dT, T, R, e, o3_rcp(m));
 }
 
 }  // namespace rlbm
