@@ -298,8 +298,8 @@ rlbm_status rlbm_batch_tuning(rlbm_ctx* const* ctxs, int count, int* steps_per_g
  * The paper's model is three-dimensional (Sec. II-III, App. C); these entry
  * points run it on an Nx x Ny x Nz periodic lattice with the unfolded
  * stencil (every vector of the six Table I orbits, signed n_z), all three
- * velocity components and the 14 polynomials of App. A.  They use generic
- * kernels (any six-group stencil): FP64 storage (f_i), or FP32 storage of
+ * velocity components and the 14 polynomials of App. A (any six-group
+ * stencil): FP64 storage (f_i), or FP32 storage of
  * d_i = f_i - r_i with FP32 accumulation; the site solve (Landau frame by
  * Newton iteration on the three velocities, Eq. 20; EOS, Eq. 28) is FP64.
  * Fields are [Nz][Ny][Nx] arrays, x fastest.  A separate context type. */
@@ -317,15 +317,15 @@ typedef struct {
   int kernel;               /* step kernel: 0 generic; 1..4 compiled for the
                                stencils {5,12,14,17,21,26}, {1..6},
                                {1,14,49,51,60,70}, {3,9,10,14,17,21} (FP32
-                               storage, lattice at least a halo wide)         */
+                               storage, lattice at least a halo wide); 0 for
+                               every third-order stencil                      */
   int order;                /* expansion order of f^eq: 2 or 3 (eleven groups:
-                               the thirty-monomial third-order equilibrium on
-                               the generic kernels)                           */
+                               the thirty-monomial third-order equilibrium)   */
 } rlbm3_info;
 
 /* As rlbm_create, with Nz >= 1 and Nx Ny Nz <= 2^31 - 1; dtype RLBM_F64 or RLBM_F32 (ENOTSUP for
  * BF16).  Six groups: the second-order equilibrium (App. A-B); eleven: the
- * third-order one, exact to the third moment T^abc (generic kernels).  More
+ * third-order one, exact to the third moment T^abc.  More
  * than 160 unfolded populations: ENOTSUP. */
 rlbm_status rlbm3_create(const rlbm_stencil* st, double m, double tau, int Nx, int Ny, int Nz,
                          rlbm_dtype dtype, void* cuda_stream, rlbm_ctx3** out);

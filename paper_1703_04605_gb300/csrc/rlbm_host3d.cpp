@@ -51,6 +51,8 @@ struct rlbm_ctx3 {
   double* d_w64 = nullptr;
   float* d_w32 = nullptr;
   Step3O3Params q{};
+  std::unique_ptr<Fused3O3Params> fo3;   // compiled FP32 third-order kernel
+  std::unique_ptr<StencilBuild3O3> s3;
   DevMem mem;                  // device allocator (rlbm_set_allocator at creation)
   std::string last_error;
 };
@@ -89,9 +91,9 @@ HL split3(double v) {
 // The compiled 3D stencil for these groups, when its population order is the
 // host's (the storage planes) and the lattice is at least a halo wide.
 template <class D>
-bool same_order(const rlbm_ctx3* c) {
-  for (int k = 0; k < 6; ++k)
-    if (c->sb.sb.groups[k] != D::groups[k]) return false;
+bool same_order(const rlbm_ctx3* c, const int* groups) {
+  for (int g : D::groups)
+    if (*groups++ != g) return false;
   if (D::Q != c->Q) return false;
   for (int i = 0; i < D::Q; ++i) {
     const Pop3& q = c->sb.pops[i];
@@ -103,10 +105,10 @@ bool same_order(const rlbm_ctx3* c) {
 
 int fused3_kind(const rlbm_ctx3* c) {
   if (c->dtype != RLBM_F32) return 0;
-  if (same_order<Stencil3M1>(c)) return 1;
-  if (same_order<Stencil3G16>(c)) return 2;
-  if (same_order<Stencil3E5>(c)) return 3;
-  if (same_order<Stencil3S2>(c)) return 4;
+  if (same_order<Stencil3M1>(c, c->sb.sb.groups)) return 1;
+  if (same_order<Stencil3G16>(c, c->sb.sb.groups)) return 2;
+  if (same_order<Stencil3E5>(c, c->sb.sb.groups)) return 3;
+  if (same_order<Stencil3S2>(c, c->sb.sb.groups)) return 4;
   return 0;
 }
 
@@ -146,6 +148,45 @@ void fill_fused3(rlbm_ctx3* c, double nref) {
   f.err = c->d_err;
 }
 
+// Parameters of the compiled third-order kernel at reference density nref.
+void fill_fused3_o3(rlbm_ctx3* c, double nref) {
+  Fused3O3Params& f = *c->fo3;
+  std::memset(&f, 0, sizeof f);
+  const StencilBuild3O3& s3 = *c->s3;
+  const StencilBuild& sb = c->sb.sb;
+  f.Nx = c->Nx;
+  f.Ny = c->Ny;
+  f.Nz = c->Nz;
+  f.pitch = c->pitch;
+  f.zstride = c->pitch * c->Ny;
+  f.plane = c->plane;
+  f.inv_tau = (float)(1.0 / c->tau);
+  f.v0 = (float)sb.v0;
+  f.mb = (float)sb.mbar;
+  f.im = (float)(1.0 / sb.mbar);
+  f.cv_r = (float)sb.cv_r;
+  f.c = (float)s3.c;
+  f.Rr = split3(sb.sc.Rr);
+  const double N0r = nref * c->sb.mref1[0];
+  f.nr = split3(N0r);
+  f.yr = split3(nref * c->sb.mref1[4] / N0r);
+  for (int k = 0; k < 14; ++k) f.mref[k] = split3(nref * c->sb.mref1[k]);
+  f.Rr64 = sb.sc.Rr;
+  f.mb64 = sb.mbar;
+  for (int g = 0; g < 11; ++g)
+    for (int q = 0; q < 5; ++q) f.gm[g][q] = split3(s3.gm[g][q]);
+  using D = Stencil3O3M5;
+  for (int k = 0; k < D::O.K; ++k) {
+    const int i = D::O.idx[k][0];
+    f.ow[k][0] = split3(c->sb.pops[i].c[14]);
+    for (int l = 0; l < kO3Mono3; ++l) f.ow[k][1 + l] = split3(s3.wrows[i][l]);
+  }
+  f.rt64 = c->d_rt64;
+  f.rt32 = c->d_rt32;
+  f.dr64 = c->d_dr64;
+  f.err = c->d_err;
+}
+
 // Reference r_i of the FP32 storage at density nref (FP64 storage: none).
 void set_reference3(rlbm_ctx3* c, double nref) {
   if (c->dtype == RLBM_F64) nref = 0.0;
@@ -153,6 +194,7 @@ void set_reference3(rlbm_ctx3* c, double nref) {
   c->p.b0ref = c->order == 3 ? 0.0 : nref * c->sb.sb.b0ref1;
   for (int k = 0; k < 14; ++k) c->p.mref[k] = nref * c->sb.mref1[k];
   if (c->fused) fill_fused3(c, nref);
+  if (c->fo3) fill_fused3_o3(c, nref);
 }
 
 rlbm_status check_error3(rlbm_ctx3* c) {
@@ -312,6 +354,10 @@ rlbm_status rlbm3_create(const rlbm_stencil* st, double m, double tau, int Nx, i
     c->q.c = s3->c;
     c->q.w64 = c->d_w64;
     c->q.w32 = c->d_w32;
+    if (dtype == RLBM_F32 && same_order<Stencil3O3M5>(c.get(), s3->groups)) {
+      c->fo3.reset(new Fused3O3Params);
+      c->s3 = std::move(s3);
+    }
   }
   set_reference3(c.get(), 1.0);
   *out = c.release();
@@ -362,7 +408,8 @@ rlbm_status rlbm3_step(rlbm_ctx3* c, int nsteps) {
   c->q.b = c->p;
   for (int k = 0; k < nsteps; ++k) {
     cudaError_t e;
-    if (c->order == 3) e = launch_step3d_o3(c->dtype, c->q, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
+    if (c->fo3) e = launch_fused3d_o3(*c->fo3, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
+    else if (c->order == 3) e = launch_step3d_o3(c->dtype, c->q, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
     else if (c->fused) e = launch_fused3d(c->fused, c->fp, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
     else e = launch_step3d(c->dtype, c->p, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
     if (e != cudaSuccess) return cuda_fail3(c, e, "step launch");

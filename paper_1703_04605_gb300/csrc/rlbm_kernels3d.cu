@@ -18,7 +18,7 @@
 #include <utility>
 
 #include "rlbm_kernels.cuh"
-#include "rlbm_o3_3d.h"
+#include "rlbm_o3_3d.cuh"
 
 namespace rlbm {
 namespace {
@@ -425,49 +425,6 @@ __global__ void __launch_bounds__(128) moments3d_kernel(const __grid_constant__ 
 }
 
 // ------------------------------------------------------------ third order
-// Site quantities of the third-order equilibrium (see rlbm_o3_3d.h and the
-// 2D form in rlbm_o3.cuh): with h = m R + 4T, A3 = m^2 + 6 T h, B3 = -T h,
-// the deviations from rest at T_R of the moments (per unit density) of
-// t^a p^s1 ... p^sr are
-//   r = 0:  a = 0: dR/m           a = 1: dU - c dR/m
-//   r = 1:  a = 0: U_s            a = 1: U_s (h U0 - c)
-//   r = 2:  a = 0: h U_s U_s' + d_ss' dT
-//           a = 1: (A3 U0 - c h) U_s U_s' + d_ss' (T (h U0 - c) - (h_r - c))
-//   r = 3:  A3 U_s U_s' U_s'' + T h (d_ss' U_s'' + d_ss'' U_s' + d_s's'' U_s)
-// (Eq. 4-6, 28-29, 43-44; eta^ab = -delta_ab on the spatial indices).
-template <typename R>
-struct O3Site3 {
-  R n, U[4], dU, dR, dT, m, c, h, Th, Am, hU, sdev, q;
-};
-
-template <int A, int I, int J, int K, typename R>
-__device__ __forceinline__ R o3dev3(const O3Site3<R>& s) {
-  constexpr int r = I + J + K;
-  constexpr int i1 = I > 0 ? 1 : (J > 0 ? 2 : 3);
-  constexpr int i2 = I > 1 ? 1 : (I + J > 1 ? 2 : 3);
-  constexpr int i3 = I > 2 ? 1 : (I + J > 2 ? 2 : 3);
-  if constexpr (r == 0) {
-    return A == 0 ? s.n * s.dR / s.m : s.n * (s.dU - s.c * s.dR / s.m);
-  } else if constexpr (r == 1) {
-    return A == 0 ? s.n * s.U[i1] : s.n * s.U[i1] * s.hU;
-  } else if constexpr (r == 2) {
-    const R uu = s.U[i1] * s.U[i2];
-    if constexpr (A == 0) return s.n * (s.h * uu + (i1 == i2 ? s.dT : R(0)));
-    else return s.n * (s.q * uu + (i1 == i2 ? s.sdev : R(0)));
-  } else {
-    R v = s.Am * s.U[i1] * s.U[i2] * s.U[i3];
-    if constexpr (i1 == i2) v += s.Th * s.U[i3];
-    if constexpr (i1 == i3) v += s.Th * s.U[i2];
-    if constexpr (i2 == i3) v += s.Th * s.U[i1];
-    return s.n * v;
-  }
-}
-
-template <typename R, int... L>
-__device__ __forceinline__ void o3_dev3_all(std::integer_sequence<int, L...>, const O3Site3<R>& s, R* e) {
-  ((e[L] = o3dev3<kO3Exp3.e[L][0], kO3Exp3.e[L][1], kO3Exp3.e[L][2], kO3Exp3.e[L][3], R>(s)), ...);
-}
-
 // e_l = n dmu_l of the thirty monomials from the FP64 site macros.
 template <typename R>
 __device__ __forceinline__ void o3_deviations3(const Macro3& o, double Rr, double mbar, double c, R* e) {
@@ -487,9 +444,8 @@ __device__ __forceinline__ void o3_deviations3(const Macro3& o, double Rr, doubl
   s.U[2] = (R)o.Uy;
   s.U[3] = (R)o.Uz;
   s.dU = (R)dU;
-  s.dR = (R)dR;
+  s.dRm = (R)(dR / mbar);
   s.dT = (R)dT;
-  s.m = (R)mbar;
   s.c = (R)c;
   s.h = (R)h;
   s.Th = (R)Th;

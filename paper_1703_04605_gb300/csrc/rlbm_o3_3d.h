@@ -39,6 +39,28 @@ struct Step3O3Params {
   const float* w32;       // [Q][kRowW3] (FP32 storage)
 };
 
+// Compiled FP32 third-order 3D step (rlbm_fused3d_o3.cu): as Fused3Params with
+// eleven groups; ow[K]: rest weight and thirty dual-basis values of the
+// representative (+n_x, +n_y, +n_z) of octant orbit K, as hi/lo pairs.
+constexpr int kMaxOct3 = 40;
+struct Fused3O3Params {
+  int Nx, Ny, Nz;
+  long long pitch, zstride, plane;   // elements; zstride = pitch * Ny
+  float inv_tau, v0;
+  float mb, cv_r, c, im;             // im = 1/m
+  HL Rr, nr, yr;
+  HL mref[14];
+  double Rr64, mb64;
+  HL gm[11][5];
+  HL ow[kMaxOct3][kO3Mono3 + 1];
+  const double* rt64;
+  const float* rt32;
+  const double* dr64;
+  unsigned* err;
+};
+
+cudaError_t launch_fused3d_o3(const Fused3O3Params& p, const void* fin, void* fout, cudaStream_t s);
+
 cudaError_t launch_step3d_o3(rlbm_dtype dt, const Step3O3Params& p, const void* fin, void* fout, cudaStream_t s);
 cudaError_t launch_init3d_o3(rlbm_dtype dt, const Step3O3Params& p, Field3Ptrs f, void* cur, void* prev,
                              cudaStream_t s);

@@ -750,6 +750,7 @@ rlbm_status build_stencil3d_o3(const rlbm_stencil* st, double m, StencilBuild3O3
   for (int k = 0; k < 11; ++k) {
     out->groups[k] = f.groups[k];
     out->w_group[k] = f.w_group[k];
+    for (int q = 0; q < 5; ++q) out->gm[k][q] = f.gm[k][q];
   }
   out->c = f.c;
   StencilBuild& sb = out->base.sb;

@@ -130,6 +130,7 @@ struct StencilBuild3O3 {
   int groups[11];
   double w_group[11];
   double c;                 // centring shift mbar K2/K1(mbar)
+  double gm[11][5];         // per group: P0, P0^2, Pv, P0 Pv, Pv^2
   std::vector<std::array<double, kRowW3>> wrows;
 };
 

@@ -128,13 +128,13 @@ struct Unfolded {
   int grp[kMaxUnfolded], nx[kMaxUnfolded], ny[kMaxUnfolded], nz[kMaxUnfolded];
 };
 
-constexpr Unfolded unfold_stencil(int g0, int g1, int g2, int g3, int g4, int g5) {
+template <int NG>
+constexpr Unfolded unfold_groups(const int (&gs)[NG]) {
   Unfolded U{};
-  const int gs[6] = {g0, g1, g2, g3, g4, g5};
   int perms[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
   U.Q = 0;
   U.halo = 0;
-  for (int g = 0; g < 6; ++g) {
+  for (int g = 0; g < NG; ++g) {
     const int* b = kTableI.v[gs[g] - 1];
     int vec[48][3] = {};
     int nvec = 0;
@@ -176,6 +176,55 @@ constexpr Unfolded unfold_stencil(int g0, int g1, int g2, int g3, int g4, int g5
   return U;
 }
 
+constexpr Unfolded unfold_stencil(int g0, int g1, int g2, int g3, int g4, int g5) {
+  const int gs[6] = {g0, g1, g2, g3, g4, g5};
+  return unfold_groups<6>(gs);
+}
+
+// Octant orbits of an unfolded stencil: the populations (+-a_x, +-a_y, +-a_z)
+// of one group.  Member s (bits 0, 1, 2: x, y, z negative) is population
+// idx[k][s], with the bits of zero components cleared (idx of such an s
+// repeats the cleared one's).
+struct Octants {
+  int K;
+  int grp[kMaxUnfolded], ax[kMaxUnfolded], ay[kMaxUnfolded], az[kMaxUnfolded];
+  int idx[kMaxUnfolded][8];
+};
+
+constexpr Octants make_octants(const Unfolded& U) {
+  Octants O{};
+  O.K = 0;
+  for (int i = 0; i < U.Q; ++i) {
+    if (U.nx[i] < 0 || U.ny[i] < 0 || U.nz[i] < 0) continue;   // (+,+,+) represents the orbit
+    const int k = O.K++;
+    O.grp[k] = U.grp[i];
+    O.ax[k] = U.nx[i];
+    O.ay[k] = U.ny[i];
+    O.az[k] = U.nz[i];
+    for (int s = 0; s < 8; ++s) {
+      const int x = (s & 1) ? -U.nx[i] : U.nx[i], y = (s & 2) ? -U.ny[i] : U.ny[i], z = (s & 4) ? -U.nz[i] : U.nz[i];
+      O.idx[k][s] = -1;
+      for (int j = 0; j < U.Q; ++j)
+        if (U.grp[j] == U.grp[i] && U.nx[j] == x && U.ny[j] == y && U.nz[j] == z) O.idx[k][s] = j;
+    }
+  }
+  return O;
+}
+
+// Every population in exactly one orbit.
+constexpr bool octants_cover(const Unfolded& U, const Octants& O) {
+  int seen[kMaxUnfolded] = {};
+  for (int k = 0; k < O.K; ++k)
+    for (int s = 0; s < 8; ++s) {
+      if (((s & 1) && !O.ax[k]) || ((s & 2) && !O.ay[k]) || ((s & 4) && !O.az[k])) continue;
+      if (O.idx[k][s] < 0) return false;
+      seen[O.idx[k][s]] += 1;
+    }
+  for (int i = 0; i < U.Q; ++i)
+    if (seen[i] != 1) return false;
+  return true;
+}
+
 // Compiled 3D stencils (group ids ascending).
 template <int G0, int G1, int G2, int G3, int G4, int G5>
 struct Stencil3Def {
@@ -188,6 +237,16 @@ using Stencil3M1 = Stencil3Def<5, 12, 14, 17, 21, 26>;
 using Stencil3G16 = Stencil3Def<1, 2, 3, 4, 5, 6>;
 using Stencil3E5 = Stencil3Def<1, 14, 49, 51, 60, 70>;
 using Stencil3S2 = Stencil3Def<3, 9, 10, 14, 17, 21>;
+
+// The third-order 3D stencil (159 populations; the library's other
+// third-order sets have more than the 3D maximum of 160).
+struct Stencil3O3M5 {
+  static constexpr int groups[11] = {1, 2, 5, 6, 7, 9, 10, 11, 12, 13, 15};
+  static constexpr Unfolded U = unfold_groups<11>(groups);
+  static constexpr int Q = U.Q;
+  static constexpr Octants O = make_octants(U);
+  static_assert(octants_cover(U, O), "octant orbits must partition the unfolded stencil");
+};
 
 // Reflection orbits of a folded stencil: the populations of one group with
 // the same |n_x|, |n_y| and n_z^2 under n_x -> -n_x and n_y -> -n_y.  kind 4:
