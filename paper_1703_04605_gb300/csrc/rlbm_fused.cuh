@@ -940,160 +940,14 @@ cudaError_t launch_fused_impl(const FusedParams& p, const void* fin, void* fout,
 
 namespace rlbm {
 
-// ---------------------------------------------------- BF16 init and read-out
-// Group coefficients of f^eq - r at one site from its fields, in FP64 (same
-// definitions as the step kernel: r0..r9 and the folded constants p.gf).
-__device__ __forceinline__ void fp64_group_coeffs(const FusedParams& p, const SiteConsts& sc, double n,
-                                                  double ux, double uy, double T, double (&c)[6][6],
-                                                  unsigned& fl) {
-  const double v2 = ux * ux + uy * uy;
-  const double g = 1.0 / sqrt(1.0 - v2);
-  const double dU = g * g * v2 / (g + 1.0);
-  const double Ux = g * ux, Uy = g * uy;
-  const double R = ratio64(sc.mbar / T, p.rt64, fl);
-  const double dR = R - sc.Rr;
-  const double mr32 = sc.mbar * R + 4.0 * T;
-  const double F = sc.mY * dR + 3.0 * (T - 1.0);
-  const double G = sc.mbar * dR + 4.0 * (T - 1.0);
-  const double r0 = n * R - p.nr64 * sc.Rr;
-  const double r1 = n * (dU - sc.k21 * dR);
-  const double r2 = n * Ux, r3 = n * Uy;
-  const double r4 = n * (F + dU * (2.0 * mr32 + sc.cb00_1) + dU * dU * mr32);
-  const double h = G + mr32 * dU;
-  const double r5 = n * h * Ux, r6 = n * h * Uy;
-  const double r7 = n * mr32 * Uy * Uy, r8 = n * mr32 * (Uy * Uy - 2.0 * Ux * Ux), r9 = n * mr32 * Ux * Uy;
-  for (int k = 0; k < 6; ++k) {
-    double a[10];
-    for (int q = 0; q < 10; ++q) a[q] = (double)p.gf[k][q].hi + (double)p.gf[k][q].lo;
-    c[k][0] = a[0] * r0 + a[1] * r1 + a[2] * r4 + a[3] * r7 + a[4] * r8;
-    c[k][1] = a[5] * r2 + a[6] * r5;
-    c[k][2] = a[5] * r3 + a[6] * r6;
-    c[k][3] = a[7] * (r7 - r8);
-    c[k][4] = a[8] * r7;
-    c[k][5] = a[9] * r9;
-  }
-}
-
-__device__ __forceinline__ uint2 bf_coeffs(const double (&c)[6][6], int g) {
-  uint2 q;
-  q.x = bf_pack((float)c[g][0], (float)c[g][1]);
-  q.y = bf_pack((float)c[g][2], (float)(0.5 * (c[g][3] + c[g][4])));
-  return q;
-}
-
-__device__ __forceinline__ double bf_ref_rt(uint2 c, int nx, int ny, int mult) {
-  return mult * ((double)bf_lo(c.x) + nx * (double)bf_hi(c.x) + ny * (double)bf_lo(c.y) +
-                 (nx * nx + ny * ny) * (double)bf_hi(c.y));
-}
-
-// Init, phase 1: reference coefficients of every site into both buffers.
-template <class Def>
-__global__ void __launch_bounds__(128) bf16_init_coeffs(const __grid_constant__ FusedParams p, SiteConsts sc,
-                                                        FieldPtrs fd, uint2* __restrict__ c0,
-                                                        uint2* __restrict__ c1) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned fl = 0;
-  if (s < p.Nx * p.Ny) {
-    int x, y;
-    site_of(s, p.Nx, x, y);
-    double c[6][6];
-    fp64_group_coeffs(p, sc, fd.n[s], fd.ux[s], fd.uy[s], fd.T[s], c, fl);
-    const long long here = (long long)y * p.pitch + x;
-    for (int g = 0; g < 6; ++g) {
-      const uint2 q = bf_coeffs(c, g);
-      c0[(long long)g * p.plane + here] = q;
-      c1[(long long)g * p.plane + here] = q;
-    }
-  }
-  report(fl, p.err);
-}
-
-// Init, phase 2: S_0 at the site and S_{-1} at x - n_i (see init_kernel).
-template <class Def>
-__global__ void __launch_bounds__(128) bf16_init_pops(const __grid_constant__ FusedParams p, SiteConsts sc,
-                                                      FieldPtrs fd, const uint2* __restrict__ coef,
-                                                      unsigned short* __restrict__ cur,
-                                                      unsigned short* __restrict__ prev) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned fl = 0;
-  if (s < p.Nx * p.Ny) {
-    int x, y;
-    site_of(s, p.Nx, x, y);
-    double c[6][6];
-    fp64_group_coeffs(p, sc, fd.n[s], fd.ux[s], fd.uy[s], fd.T[s], c, fl);
-    const long long here = (long long)y * p.pitch + x;
-    constexpr Folded F = Def::F;   // local copies: indexed at run time below
-    constexpr BfWords B = Def::B;
-    for (int i = 0; i < Def::Q; ++i) {
-      const int g = F.grp[i], nx = F.nx[i], ny = F.ny[i], mult = F.mult[i];
-      const double fr = mult * (c[g][0] + nx * c[g][1] + ny * c[g][2] + nx * nx * c[g][3] + ny * ny * c[g][4] +
-                                nx * ny * c[g][5]);
-      const uint2 own = coef[(long long)g * p.plane + here];
-      cur[2 * ((long long)B.word[i] * p.plane + here) + B.half[i]] =
-          __bfloat16_as_ushort(__double2bfloat16(fr - bf_ref_rt(own, nx, ny, mult)));
-      int xs = x - nx, ys = y - ny;
-      xs = ((xs % p.Nx) + p.Nx) % p.Nx;
-      ys = ((ys % p.Ny) + p.Ny) % p.Ny;
-      const long long there = (long long)ys * p.pitch + xs;
-      const uint2 rem = coef[(long long)g * p.plane + there];
-      prev[2 * ((long long)B.word[i] * p.plane + there) + B.half[i]] =
-          __bfloat16_as_ushort(__double2bfloat16(fr - bf_ref_rt(rem, nx, ny, mult)));
-    }
-  }
-  report(fl, p.err);
-}
-
-// Read-out: decode the pull of S_{t-1} with its coefficients, FP64 solve.
-template <class Def>
-__global__ void __launch_bounds__(128) bf16_moments(const __grid_constant__ StepParams<double> p,
-                                                    const unsigned short* __restrict__ prev,
-                                                    const uint2* __restrict__ cprev, MomentOut mo) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned fl = 0;
-  const long long N = (long long)p.Nx * p.Ny;
-  if (s < N) {
-    int x, y;
-    site_of(s, p.Nx, x, y);
-    double m[9];
-    for (int k = 0; k < 9; ++k) m[k] = 0.0;
-    constexpr Folded F = Def::F;   // local copies: indexed at run time below
-    constexpr BfWords B = Def::B;
-    for (int i = 0; i < Def::Q; ++i) {
-      const int g = F.grp[i], nx = F.nx[i], ny = F.ny[i], mult = F.mult[i];
-      const int xs = wrap_sub(x, p.pt.dxm[i], p.Nx);
-      const int ys = wrap_sub(y, p.pt.dym[i], p.Ny);
-      const long long there = (long long)ys * p.pitch + xs;
-      const unsigned short h = prev[2 * ((long long)B.word[i] * p.plane + there) + B.half[i]];
-      const double f = (double)__uint_as_float((unsigned)h << 16) +
-                       bf_ref_rt(cprev[(long long)g * p.plane + there], nx, ny, mult);
-      for (int k = 0; k < 9; ++k) m[k] = fma(f, p.pt.mom[k][i], m[k]);
-    }
-    for (int k = 0; k < 9; ++k) m[k] += p.mref[k];
-    const Macro<double> md = solve_site_f64(m, p.sc, p.rt64, fl);
-    double* out = mo.out;
-    int plane = 0;
-    if (mo.mask & RLBM_M_N) out[(plane++) * N + s] = md.n;
-    if (mo.mask & RLBM_M_UX) out[(plane++) * N + s] = md.Ux / md.U0;
-    if (mo.mask & RLBM_M_UY) out[(plane++) * N + s] = md.Uy / md.U0;
-    if (mo.mask & RLBM_M_T) out[(plane++) * N + s] = md.T;
-    if (mo.mask & RLBM_M_E) out[(plane++) * N + s] = m[3] - m[4] * (md.Ux / md.U0) - m[5] * (md.Uy / md.U0);
-    if (mo.mask & RLBM_M_NVEC)
-      for (int k = 0; k < 3; ++k) out[(plane++) * N + s] = m[k];
-    if (mo.mask & RLBM_M_TMN)
-      for (int k = 3; k < 9; ++k) out[(plane++) * N + s] = m[k];
-  }
-  report(fl, p.err);
-}
-
 // ---------------------------------------------------- FP32 init and read-out
 // Init of FP32 storage on a compiled stencil: per site the step kernel's own
 // equilibrium of the given fields (split site state with the FP64 dR(Td)
 // table, FP32 projections and group coefficients, FP32 group polynomials),
-// written to S_0 at the site and to S_{-1} at x - n_i (see init_kernel).
-template <class Def, bool PREV, int... Is>
+// written to S_0 at the site.
+template <class Def, int... Is>
 __device__ __forceinline__ void f32_init_pops(std::integer_sequence<int, Is...>, const float (&c)[6][6],
-                                              float* __restrict__ cur, float* __restrict__ prev,
-                                              long long plane, long long pitch, int x, int y, int Nx, int Ny) {
+                                              float* __restrict__ cur, long long plane, long long pitch, int x, int y) {
   // 32-bit element indices (a plane holds fewer than 2^32 elements)
   const unsigned here = (unsigned)y * (unsigned)pitch + (unsigned)x;
   const size_t pl = (unsigned)plane;
@@ -1109,23 +963,15 @@ __device__ __forceinline__ void f32_init_pops(std::integer_sequence<int, Is...>,
         if constexpr (nx != 0 && ny != 0) e = fmaf((float)(nx * ny), c[g][5], e);
         if constexpr (mult != 1) e *= (float)mult;
         cur[here + pl * i] = e;
-        if constexpr (PREV) {
-          // population i of S_{-1} sits at x - n_i: the first pull brings it back
-          const unsigned xs = (unsigned)wrap_c<nx>(x, Nx), ys = (unsigned)wrap_c<ny>(y, Ny);
-          prev[ys * (unsigned)pitch + xs + pl * i] = e;
-        }
       }(),
       ...);
 }
 
-// PREV: also write S_{-1} (the copy whose pull is the initial state) into
-// prev; without it the read-out of the freshly initialised state reads cur
-// in place (f32_moments_kernel<Def, false>) and the first step overwrites
-// prev anyway.
-template <class Def, bool PREV>
-__global__ void __launch_bounds__(128) f32_init_kernel(const __grid_constant__ FusedParams p, SiteConsts sc,
-                                                       FieldPtrs fd, float* __restrict__ cur,
-                                                       float* __restrict__ prev) {
+// S_{-1} is not written: the read-out of the freshly initialised state reads
+// S_0 in place (f32_moments_kernel<Def, false>).
+template <class Def>
+__global__ void __launch_bounds__(128) f32_init_kernel(const __grid_constant__ FusedParams p, FieldPtrs fd,
+                                                       float* __restrict__ cur) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned fl = 0;
   if (s < p.Nx * p.Ny) {
@@ -1154,9 +1000,7 @@ __global__ void __launch_bounds__(128) f32_init_kernel(const __grid_constant__ F
     ss.R = p.Rr.hi + (p.Rr.lo + ss.dR);
     float c[6][6];
     fused_coeffs(p, ss, c);
-    (void)sc;
-    f32_init_pops<Def, PREV>(std::make_integer_sequence<int, Def::Q>{}, c, cur, prev, p.plane, p.pitch, x, y, p.Nx,
-                       p.Ny);
+    f32_init_pops<Def>(std::make_integer_sequence<int, Def::Q>{}, c, cur, p.plane, p.pitch, x, y);
   }
   report(fl, p.err);
 }
@@ -1168,7 +1012,7 @@ __global__ void __launch_bounds__(128) f32_init_kernel(const __grid_constant__ F
 // carry FP32 rounding of their deviations from the reference only.  The
 // moment planes are assembled in FP64 from the float-float sums.
 // PULL: the state at t is the pull of S_{t-1} in prev; otherwise (right
-// after f32_init_kernel<Def, false>) it is S_0 in prev read in place.
+// after f32_init_kernel) it is S_0 in prev read in place.
 template <class Def, bool PULL>
 __global__ void __launch_bounds__(128) f32_moments_kernel(const __grid_constant__ FusedParams fp,
                                                           const __grid_constant__ StepParams<double> p,
@@ -1234,32 +1078,17 @@ __global__ void __launch_bounds__(128) f32_moments_kernel(const __grid_constant_
   report(fl, p.err);
 }
 
-// what: 0 BF16 init, 1 BF16 read-out, 2 FP32 init, 3 FP32 read-out.
+// what: 0 init of S_0 into buf, 1 read-out of the pull of buf, 2 read-out of
+// S_0 in buf, in place.
 template <class Def>
-cudaError_t launch_bf16_io_impl(int what, const FusedParams& fp, const StepParams<double>& p, FieldPtrs fd,
-                                void* cur, void* prev, void* ccur, void* cprev, MomentOut mo, cudaStream_t s) {
+cudaError_t launch_f32_io_impl(int what, const FusedParams& fp, const StepParams<double>& p, FieldPtrs fd, void* buf,
+                               MomentOut mo, cudaStream_t s) {
   const long long nsite = (long long)p.Nx * p.Ny;
   const unsigned grid = (unsigned)((nsite + 127) / 128);
-  if (what == 2) {
-    f32_init_kernel<Def, false><<<grid, 128, 0, s>>>(fp, p.sc, fd, static_cast<float*>(cur), static_cast<float*>(prev));
-    return cudaGetLastError();
-  }
-  if (what == 3) {
-    f32_moments_kernel<Def, true><<<grid, 128, 0, s>>>(fp, p, static_cast<const float*>(prev), mo);
-    return cudaGetLastError();
-  }
-  if (what == 4) {
-    f32_moments_kernel<Def, false><<<grid, 128, 0, s>>>(fp, p, static_cast<const float*>(prev), mo);
-    return cudaGetLastError();
-  }
-  if (what == 0) {
-    bf16_init_coeffs<Def><<<grid, 128, 0, s>>>(fp, p.sc, fd, static_cast<uint2*>(ccur), static_cast<uint2*>(cprev));
-    bf16_init_pops<Def><<<grid, 128, 0, s>>>(fp, p.sc, fd, static_cast<const uint2*>(ccur),
-                                             static_cast<unsigned short*>(cur), static_cast<unsigned short*>(prev));
-  } else {
-    bf16_moments<Def><<<grid, 128, 0, s>>>(p, static_cast<const unsigned short*>(prev),
-                                           static_cast<const uint2*>(cprev), mo);
-  }
+  float* b = static_cast<float*>(buf);
+  if (what == 0) f32_init_kernel<Def><<<grid, 128, 0, s>>>(fp, fd, b);
+  else if (what == 1) f32_moments_kernel<Def, true><<<grid, 128, 0, s>>>(fp, p, b, mo);
+  else f32_moments_kernel<Def, false><<<grid, 128, 0, s>>>(fp, p, b, mo);
   return cudaGetLastError();
 }
 

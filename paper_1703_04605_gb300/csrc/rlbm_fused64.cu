@@ -8,33 +8,6 @@
 namespace rlbm {
 namespace {
 
-// Equilibrium coefficients of one group from the projections r.
-__device__ __forceinline__ void group_coeffs64(const double* a, const double (&r)[10], double (&c)[6]) {
-  c[0] = fma(a[0], r[0], fma(a[1], r[1], fma(a[2], r[4], fma(a[3], r[7], a[4] * r[8]))));
-  c[1] = fma(a[5], r[2], a[6] * r[5]);
-  c[2] = fma(a[5], r[3], a[6] * r[6]);
-  c[3] = a[7] * (r[7] - r[8]);
-  c[4] = a[8] * r[7];
-  c[5] = a[9] * r[9];
-}
-
-// n times the projections of App. B without their normalisations (in gf).
-__device__ __forceinline__ void projections64(const SiteConsts& sc, const Macro<double>& o, double (&r)[10]) {
-  const double n = o.n, mr32 = fma(sc.mbar, o.R, 4.0 * o.T);
-  const double nm = n * mr32, h = n * fma(mr32, o.dU, o.G);
-  const double yy = nm * o.Uy * o.Uy;
-  r[0] = n * o.R;
-  r[1] = n * (o.dU - sc.k21 * o.dR);
-  r[2] = n * o.Ux;
-  r[3] = n * o.Uy;
-  r[4] = n * (o.F + o.dU * (fma(2.0, mr32, sc.cb00_1) + o.dU * mr32));
-  r[5] = h * o.Ux;
-  r[6] = h * o.Uy;
-  r[7] = yy;
-  r[8] = fma(-2.0 * nm * o.Ux, o.Ux, yy);
-  r[9] = nm * o.Ux * o.Uy;
-}
-
 template <class Def, int K>
 __device__ __forceinline__ void collide64_orbit(const Fused64Params& p, const double (&r)[10], double (&c)[6],
                                                 const Pull64& q, const Relax64& rx) {
@@ -71,7 +44,7 @@ __global__ void __launch_bounds__(64, 8) fused_f64_kernel(const __grid_constant_
     acc64_all<Def>(Orb{}, q, p.gm, M);
     const Macro<double> o = solve_site_f64_seeded(M, p.sc, p.rt64, p.rt32, fl);
     double r[10];
-    projections64(p.sc, o, r);
+    projections64(p.sc, o, 0.0, r);
     const double wv = p.v0 * p.inv_tau;
     const Relax64 rx{o.U0 * p.inv_tau, wv * o.Ux, wv * o.Uy, fout + ((unsigned)y * (unsigned)p.pitch + (unsigned)x),
                      (size_t)p.plane};
@@ -131,7 +104,7 @@ __global__ void __launch_bounds__(32) fused_f64_quad_kernel(const __grid_constan
   lane_moments_all<Def>(Orb{}, q, d, p.gm, M);
   const Macro<double> o = solve_site_f64_seeded(M, p.sc, p.rt64, p.rt32, fl);
   double r[10];
-  projections64(p.sc, o, r);
+  projections64(p.sc, o, 0.0, r);
   const double wv = p.v0 * p.inv_tau;
   if (live)
     lane_collide_all<Def>(Orb{}, p, q, d, r, o.U0 * p.inv_tau, flip(wv * o.Ux, q.l & 1), flip(wv * o.Uy, q.l >> 1));

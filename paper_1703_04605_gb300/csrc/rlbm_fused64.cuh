@@ -48,6 +48,57 @@ static __device__ __noinline__ void solve_site_f64_cold(const double* m, const S
   *o = solve_site_f64(m, *sc, rt64, *fl);
 }
 
+// T and R = K1/K2(m/T) of 3 T + m R(m/T) = y (Eq. 28): FP32 Newton, then FP64
+// corrections; iT = 1/T nearly.  False where it did not settle.
+__device__ __forceinline__ bool eos_seeded(double y, const SiteConsts& sc, const double* __restrict__ rt64,
+                                           const float* __restrict__ rt32, double& T, double& iT, double& R) {
+  const double mb = sc.mbar;
+  const double w = y - mb;
+  bool ok = w > 1e-30 && w < 1e30;
+  float last = 1.0f;
+  {
+    const float mbf = (float)mb, yf = (float)y;
+    float Tf = __fdividef((float)w, 3.0f - 1.5f * __fdividef(mbf * mbf, yf * yf));
+    unsigned fz = 0;
+#pragma unroll 1
+    for (int it = 0; it < 12; ++it) {
+      const float z = __fdividef(mbf, Tf);
+      const float Rf = ratio32(z, rt32, fz);
+      const float dT = __fdividef(3.0f * Tf + mbf * (Rf - 1.0f) - (float)w, eos_slope<float>(Rf, z));
+      if (!(Tf - dT > 0.0f)) break;
+      Tf -= dT;
+      // a step this short leaves an error of its square
+      if (fabsf(dT) < 3e-4f * Tf) break;
+    }
+    ok = ok && Tf > 1e-30f && Tf < 1e30f;
+    T = (double)Tf;
+    float fiT = __frcp_rn(Tf);
+    iT = (double)fiT;
+    float dR = 0.0f, z32 = 0.0f;
+#pragma unroll 1
+    for (int it = 0; it < 4; ++it) {
+      // iT is off by 1e-7 (the seed's rounding or the last step): two steps
+      iT = fma(iT, fma(-T, iT, 1.0), iT);
+      iT = fma(iT, fma(-T, iT, 1.0), iT);
+      const double z = mb * iT;
+      R = ratio64(z, rt64, fz);
+      const double slope = eos_slope<double>(R, z);
+      const float dT = (float)(fma(3.0, T, fma(mb, R, -y))) * __frcp_rn((float)slope);
+      T -= (double)dT;
+      last = fabsf(dT) * (float)iT;
+      z32 = (float)z;
+      // d R = R' dz, dz = z dT / T (T falls by dT), R' = (3 - slope) / z^2
+      dR = (3.0f - (float)slope) * __frcp_rn(z32) * (dT * (float)iT);
+      // the correction's slope is exact to FP32 rounding, so what is left is
+      // 1e-7 of this step (and its square)
+      if (last < 1e-9f) break;
+    }
+    R += (double)dR;
+    ok = ok && last < 1e-9f && fz == 0;
+  }
+  return ok;
+}
+
 // Site solve of FP64 storage: m = N0 Nx Ny T00 T0x T0y Txx Txy Tyy.
 __device__ __forceinline__ Macro<double> solve_site_f64_seeded(const double (&m)[9], const SiteConsts& sc,
                                                                const double* __restrict__ rt64,
@@ -58,7 +109,9 @@ __device__ __forceinline__ Macro<double> solve_site_f64_seeded(const double (&m)
   double t[6];
 #pragma unroll
   for (int k = 0; k < 6; ++k) t[k] = m[3 + k] * scale;   // T00 T0x T0y Txx Txy Tyy
-  bool ok = ex > 0 && ex < 2046;
+  // 2^-465 .. 2^465, where the products of the all-FP64 Landau step neither
+  // overflow nor underflow; it decides about states beyond
+  bool ok = ex > 1023 - 465 && ex < 1023 + 465;
   float vx, vy, j11, j12, j21, j22;   // iterate, inverse Jacobian
   {
     float f[6];
@@ -120,51 +173,8 @@ __device__ __forceinline__ Macro<double> solve_site_f64_seeded(const double (&m)
   const double rn = rcp64(ns);
   double y = e * rn;
   y = fma(rn, fma(-ns, y, e), y);            // e/n
-  // T: FP32 Newton on 3 T + m R(m/T) = y, then FP64 corrections
-  const double w = y - mb;
-  ok = ok && w > 1e-30 && w < 1e30;
   double T, iT, R;
-  float last = 1.0f;
-  {
-    const float mbf = (float)mb, yf = (float)y;
-    float Tf = __fdividef((float)w, 3.0f - 1.5f * __fdividef(mbf * mbf, yf * yf));
-    unsigned fz = 0;
-#pragma unroll 1
-    for (int it = 0; it < 12; ++it) {
-      const float z = __fdividef(mbf, Tf);
-      const float Rf = ratio32(z, rt32, fz);
-      const float dT = __fdividef(3.0f * Tf + mbf * (Rf - 1.0f) - (float)w, eos_slope<float>(Rf, z));
-      if (!(Tf - dT > 0.0f)) break;
-      Tf -= dT;
-      // a step this short leaves an error of its square
-      if (fabsf(dT) < 3e-4f * Tf) break;
-    }
-    ok = ok && Tf > 1e-30f && Tf < 1e30f;
-    T = (double)Tf;
-    float fiT = __frcp_rn(Tf);
-    iT = (double)fiT;
-    float dR = 0.0f, z32 = 0.0f;
-#pragma unroll 1
-    for (int it = 0; it < 4; ++it) {
-      // iT is off by 1e-7 (the seed's rounding or the last step): two steps
-      iT = fma(iT, fma(-T, iT, 1.0), iT);
-      iT = fma(iT, fma(-T, iT, 1.0), iT);
-      const double z = mb * iT;
-      R = ratio64(z, rt64, fz);
-      const double slope = eos_slope<double>(R, z);
-      const float dT = (float)(fma(3.0, T, fma(mb, R, -y))) * __frcp_rn((float)slope);
-      T -= (double)dT;
-      last = fabsf(dT) * (float)iT;
-      z32 = (float)z;
-      // d R = R' dz, dz = z dT / T (T falls by dT), R' = (3 - slope) / z^2
-      dR = (3.0f - (float)slope) * __frcp_rn(z32) * (dT * (float)iT);
-      // the correction's slope is exact to FP32 rounding, so what is left is
-      // 1e-7 of this step (and its square)
-      if (last < 1e-9f) break;
-    }
-    R += (double)dR;
-    ok = ok && last < 1e-9f && fz == 0;
-  }
+  ok = eos_seeded(y, sc, rt64, rt32, T, iT, R) && ok;
   if (!ok) {
     // copies: passing the addresses of m or o would move them to local memory
     double mm[9];
@@ -214,11 +224,26 @@ __device__ __forceinline__ double pull64(const Pull64& q) {
   return __ldg(q.fin + (ys * q.pitch + xs) + q.plane * I);
 }
 
+// FP32 planes, as FP64 values.
+struct Pull32 {
+  const float* fin;
+  size_t plane;
+  unsigned pitch;
+  int x, y, Nx, Ny;
+  const int *dxm, *dym;
+};
+template <class Def, int I>
+__device__ __forceinline__ double pull64(const Pull32& q) {
+  const unsigned xs = (unsigned)wrap_sub(q.x, q.dxm[Def::F.nx[I] + kMaxDisp], q.Nx);
+  const unsigned ys = (unsigned)wrap_sub(q.y, q.dym[Def::F.ny[I] + kMaxDisp], q.Ny);
+  return (double)__ldg(q.fin + (ys * q.pitch + xs) + q.plane * I);
+}
+
 // Sums of the current group, 1, n_x, n_y, n_x^2, n_x n_y, n_y^2, over one
 // reflection orbit; at the end of a group they go into the moments with the
 // group's momenta gm = P0, P0^2, Pv, P0 Pv, Pv^2.
-template <class Def, int K>
-__device__ __forceinline__ void acc64_orbit(const Pull64& q, const double (*gmt)[5], double (&s)[6], double (&M)[9]) {
+template <class Def, int K, class Pull>
+__device__ __forceinline__ void acc64_orbit(const Pull& q, const double (*gmt)[5], double (&s)[6], double (&M)[9]) {
   constexpr int kind = Def::O.kind[K], g = Def::O.grp[K], ax = Def::O.ax[K], ay = Def::O.ay[K];
   constexpr int i0 = Def::O.idx[K][0], i1 = Def::O.idx[K][1], i2 = Def::O.idx[K][2], i3 = Def::O.idx[K][3];
   if constexpr (orbit_starts_group<Def, K>()) {
@@ -264,8 +289,8 @@ __device__ __forceinline__ void acc64_orbit(const Pull64& q, const double (*gmt)
   }
 }
 
-template <class Def, int... Ks>
-__device__ __forceinline__ void acc64_all(std::integer_sequence<int, Ks...>, const Pull64& q, const double (*gmt)[5],
+template <class Def, class Pull, int... Ks>
+__device__ __forceinline__ void acc64_all(std::integer_sequence<int, Ks...>, const Pull& q, const double (*gmt)[5],
                                           double (&M)[9]) {
   double s[6];
 #pragma unroll
@@ -311,6 +336,35 @@ __device__ __forceinline__ void relax64_orbit(const Pull64& q, const Relax64& r,
 }
 
 // ------------------------------------------------------ four lanes a site
+// Equilibrium coefficients of one group from the projections r.
+__device__ __forceinline__ void group_coeffs64(const double* a, const double (&r)[10], double (&c)[6]) {
+  c[0] = fma(a[0], r[0], fma(a[1], r[1], fma(a[2], r[4], fma(a[3], r[7], a[4] * r[8]))));
+  c[1] = fma(a[5], r[2], a[6] * r[5]);
+  c[2] = fma(a[5], r[3], a[6] * r[6]);
+  c[3] = a[7] * (r[7] - r[8]);
+  c[4] = a[8] * r[7];
+  c[5] = a[9] * r[9];
+}
+
+// n times the projections of App. B without their normalisations (in gf); ref:
+// n R of the reference state that the storage subtracts (0: none).
+__device__ __forceinline__ void projections64(const SiteConsts& sc, const Macro<double>& o, double ref,
+                                              double (&r)[10]) {
+  const double n = o.n, mr32 = fma(sc.mbar, o.R, 4.0 * o.T);
+  const double nm = n * mr32, h = n * fma(mr32, o.dU, o.G);
+  const double yy = nm * o.Uy * o.Uy;
+  r[0] = n * o.R - ref;
+  r[1] = n * (o.dU - sc.k21 * o.dR);
+  r[2] = n * o.Ux;
+  r[3] = n * o.Uy;
+  r[4] = n * (o.F + o.dU * (fma(2.0, mr32, sc.cb00_1) + o.dU * mr32));
+  r[5] = h * o.Ux;
+  r[6] = h * o.Uy;
+  r[7] = yy;
+  r[8] = fma(-2.0 * nm * o.Ux, o.Ux, yy);
+  r[9] = nm * o.Ux * o.Uy;
+}
+
 // The members (+,+), (-,+), (+,-), (-,-) of the reflection orbits on four
 // neighbouring lanes: lane l holds the population with signs sx (bit 0 of l)
 // and sy (bit 1), so all lanes run the same code with the signs in data, each

@@ -3,39 +3,16 @@
 // (rlbm_o3.cuh), summed once a reflection orbit over the parity classes of the
 // twenty monomials (as rlbm_fused_o3.cu): 21 FP64 instructions a quartet of
 // populations instead of 84.
-#include "rlbm_fused64.cuh"
-#include "rlbm_o3.cuh"
+#include "rlbm_fused64_o3.cuh"
 
 namespace rlbm {
 namespace {
 
-// Parity classes of the centred monomials (kO3Mono order).
-using EE = std::integer_sequence<int, 0, 1, 6, 7, 9, 10, 11, 17>;   // even in p_x and p_y
-using OE = std::integer_sequence<int, 2, 4, 13, 15, 18>;            // odd in p_x only
-using EO = std::integer_sequence<int, 3, 5, 14, 16, 19>;            // odd in p_y only
-using OO = std::integer_sequence<int, 8, 12>;                       // odd in both
-
-template <int... L>
-__device__ __forceinline__ double sum64(std::integer_sequence<int, L...>, const double* w, const double (&e)[kO3Mono],
-                                        double acc) {
-  ((acc = fma(w[1 + L], e[L], acc)), ...);
-  return acc;
-}
-
-__device__ __forceinline__ void deviations64(const FusedO364Params& p, const Macro<double>& o, double (&e)[kO3Mono]) {
-  o3_deviations<double>(p.sc.mbar, p.c, o.n, o.U0, o.Ux, o.Uy, o.dU, o.dR, o.T - 1.0, o.T, o.R, e, p.sc.inv_m);
-}
-
 template <class Def, int K>
 __device__ __forceinline__ void collide64_orbit(const FusedO364Params& p, const double (&e)[kO3Mono], double n,
                                                 const Pull64& q, const Relax64& rx) {
-  constexpr int kind = Def::O.kind[K];
-  const double* w = p.ow[K];
-  const double E = sum64(EE{}, w, e, w[0] * n);
-  double X = 0.0, Y = 0.0, Z = 0.0;
-  if constexpr (kind == 2 || kind == 4) X = sum64(OE{}, w, e, 0.0);
-  if constexpr (kind == 3 || kind == 4) Y = sum64(EO{}, w, e, 0.0);
-  if constexpr (kind == 4) Z = sum64(OO{}, w, e, 0.0);
+  double E, X, Y, Z;
+  orbit_equilibrium_o3<Def, K>(p.ow[K], e, n, E, X, Y, Z);
   relax64_orbit<Def, K>(q, rx, E, X, Y, Z);
 }
 
@@ -77,10 +54,10 @@ __device__ __forceinline__ void lane_collide(const FusedO364Params& p, const Lan
                                              const double (&e)[kO3Mono], double n, double a0, double wx, double wy) {
   constexpr int kind = Def::O.kind[K], ax = Def::O.ax[K], ay = Def::O.ay[K];
   const double* w = p.ow[K];
-  double f = sum64(EE{}, w, e, w[0] * n);
-  if constexpr (kind == 4) f = sum64(OO{}, w, e, f);
-  if constexpr (kind == 2 || kind == 4) f = sum64(OE{}, w, e, f);
-  if constexpr (kind == 3 || kind == 4) f = sum64(EO{}, w, e, f);
+  double f = sum64(O3EE{}, w, e, w[0] * n);
+  if constexpr (kind == 4) f = sum64(O3OO{}, w, e, f);
+  if constexpr (kind == 2 || kind == 4) f = sum64(O3OE{}, w, e, f);
+  if constexpr (kind == 3 || kind == 4) f = sum64(O3EO{}, w, e, f);
   double om = a0;
   if constexpr (ax != 0) om = fma(-(double)ax, wx, om);
   if constexpr (ay != 0) om = fma(-(double)ay, wy, om);
@@ -119,9 +96,9 @@ __global__ void __launch_bounds__(32) fused_f64_o3_quad_kernel(const __grid_cons
   const Macro<double> o = solve_site_f64_seeded(M, p.sc, p.rt64, p.rt32, fl);
   double e[kO3Mono];
   deviations64(p, o, e);
-  flip_all(OE{}, e, q.l & 1);
-  flip_all(EO{}, e, q.l >> 1);
-  flip_all(OO{}, e, (q.l ^ (q.l >> 1)) & 1);
+  flip_all(O3OE{}, e, q.l & 1);
+  flip_all(O3EO{}, e, q.l >> 1);
+  flip_all(O3OO{}, e, (q.l ^ (q.l >> 1)) & 1);
   const double wv = p.v0 * p.inv_tau;
   if (live)
     lane_collide_all<Def>(Orb{}, p, q, d, e, o.n, o.U0 * p.inv_tau, flip(wv * o.Ux, q.l & 1),

@@ -48,21 +48,19 @@ const void* persist_kernel_fn<StencilS2>(int);
 // fin, float* fout), for graph kernel nodes; grid (Nx Ny + 127)/128, block
 // 128, no dynamic shared memory (rlbm_fused_o3.cu).
 const void* fused_o3_kernel_fn(int kind);
-// Init and read-out on a compiled stencil.  BF16 deviation storage: what = 0
-// init (fields -> coefficients, S_0, S_{-1}), what = 1 read-out of the pull of
-// prev; FP32 storage: what = 2 init of S_0 into cur only, what = 3 read-out
-// of the pull of prev, what = 4 read-out of S_0 in prev (pass cur) right after
-// what = 2, before any step (ccur, cprev unused).
+// Init and read-out of FP32 storage on a compiled stencil: what = 0 init of S_0
+// into buf, 1 read-out of the pull of buf, 2 read-out of S_0 in buf in place
+// (right after the init).  BF16-deviation storage: rlbm_io2.cu.
 template <class Def>
-cudaError_t launch_bf16_io(int what, const FusedParams& fp, const StepParams<double>& p, FieldPtrs fd,
-                           void* cur, void* prev, void* ccur, void* cprev, MomentOut mo, cudaStream_t s);
-#define RLBM_DECL_BF16_IO(S)                                                                              \
-  template <>                                                                                            \
-  cudaError_t launch_bf16_io<S>(int, const FusedParams&, const StepParams<double>&, FieldPtrs, void*, void*, \
-                                void*, void*, MomentOut, cudaStream_t);
-RLBM_DECL_BF16_IO(StencilM1)
-RLBM_DECL_BF16_IO(StencilG16)
-RLBM_DECL_BF16_IO(StencilE5)
-RLBM_DECL_BF16_IO(StencilS2)
-#undef RLBM_DECL_BF16_IO
+cudaError_t launch_f32_io(int what, const FusedParams& fp, const StepParams<double>& p, FieldPtrs fd, void* buf,
+                          MomentOut mo, cudaStream_t s);
+#define RLBM_DECL_F32_IO(S)                                                                                \
+  template <>                                                                                              \
+  cudaError_t launch_f32_io<S>(int, const FusedParams&, const StepParams<double>&, FieldPtrs, void*, MomentOut, \
+                               cudaStream_t);
+RLBM_DECL_F32_IO(StencilM1)
+RLBM_DECL_F32_IO(StencilG16)
+RLBM_DECL_F32_IO(StencilE5)
+RLBM_DECL_F32_IO(StencilS2)
+#undef RLBM_DECL_F32_IO
 }  // namespace rlbm

@@ -42,19 +42,20 @@ struct rlbm_ctx {
   size_t device_bytes = 0;
   bool initialised = false;
   bool host_init = false;   // rlbm_init in progress (it sets the reference itself)
-  bool fresh = false;       // FP32 compiled path: S_0 written in place by the init, not stepped yet
+  bool fresh = false;       // compiled init: S_0 written in place, not stepped yet (S_{-1} not written)
   std::unique_ptr<StepParams<double>> p64;
   std::unique_ptr<StepParams<float>> p32;
   int fused = 0;                 // 1: M1, 2: G1..G6, 3: E5, 4: S2; 0: generic kernel
   int ext = 0;                   // FP32 storage on a compiled stencil: extended moment sums
   std::unique_ptr<FusedParams> fp;
-  int fused64 = 0;               // FP64 storage: compiled kernel of the same stencils (0: generic)
-  std::unique_ptr<Fused64Params> fp64;
+  int kind64 = 0;                // compiled stencil (1..4, 5..10; 0: none) of the FP64 step and of the
+                                 // FP64-arithmetic init and read-out, whatever the lattice's size
+  std::unique_ptr<Io2Params> io2;
   // third-order stencils (eleven groups)
   int order = 2;
   std::unique_ptr<StencilBuildO3> sb3;
   std::unique_ptr<O3Params> o3;
-  std::unique_ptr<FusedO364Params> fo364;   // compiled FP64 third-order kernel (fused64 5..10)
+  std::unique_ptr<IoO3Params> io3;
   std::unique_ptr<FusedO3Params> fo3;   // compiled third-order kernel (fused == 5)
   int* d_shift = nullptr;
   long long* d_off = nullptr;
@@ -183,8 +184,8 @@ static void fill_disp(int Nx, int Ny, int (&dxm)[13], int (&dym)[13]) {
 }
 
 static void fill_fused64(rlbm_ctx* c) {
-  Fused64Params& f = *c->fp64;
-  std::memset(&f, 0, sizeof f);
+  std::memset(c->io2.get(), 0, sizeof(Io2Params));
+  Fused64Params& f = c->io2->b;
   f.Nx = c->Nx;
   f.Ny = c->Ny;
   f.pitch = c->pitch;
@@ -350,8 +351,8 @@ static void fill_orbits_o3(int kind, const StencilBuildO3& sb, P& f) {
 }
 
 static void fill_fused_o364(rlbm_ctx* c) {
-  FusedO364Params& f = *c->fo364;
-  std::memset(&f, 0, sizeof f);
+  std::memset(c->io3.get(), 0, sizeof(IoO3Params));
+  FusedO364Params& f = c->io3->b;
   const StencilBuildO3& sb = *c->sb3;
   f.Nx = c->Nx;
   f.Ny = c->Ny;
@@ -363,7 +364,7 @@ static void fill_fused_o364(rlbm_ctx* c) {
   f.sc = sb.sc;
   for (int g = 0; g < 11; ++g)
     for (int q = 0; q < 5; ++q) f.gm[g][q] = sb.gm[g][q];
-  fill_orbits_o3(c->fused64, sb, f);
+  fill_orbits_o3(c->kind64, sb, f);
   fill_disp(c->Nx, c->Ny, f.dxm, f.dym);
   f.sms = sm_count();
   f.rt64 = c->d_rt64;
@@ -408,6 +409,10 @@ static void set_reference(rlbm_ctx* c, double nref) {
     c->o3->nref = nref;
     for (int k = 0; k < 9; ++k) c->o3->mref[k] = nref * c->sb3->mref1[k];
     if (c->fo3) fill_fused_o3(c, nref);
+    if (c->io3) {
+      c->io3->nref = nref;
+      for (int k = 0; k < 9; ++k) c->io3->mref[k] = c->o3->mref[k];
+    }
     return;
   }
   for (StepParams<double>* p : {c->p64.get()}) {
@@ -420,6 +425,10 @@ static void set_reference(rlbm_ctx* c, double nref) {
   q->b0ref = nref * c->sb.b0ref1;
   for (int k = 0; k < 9; ++k) q->mref[k] = nref * c->sb.mref1[k];
   if (c->fused) fill_fused(c, nref);
+  if (c->io2) {
+    c->io2->ref = nref * c->sb.mref1[0] * c->sb.sc.Rr;
+    for (int k = 0; k < 9; ++k) c->io2->mref[k] = c->p64->mref[k];
+  }
 }
 
 static rlbm_status check_device_error(rlbm_ctx* c) {
@@ -442,6 +451,17 @@ static rlbm_status check_device_error(rlbm_ctx* c) {
     return fail(c, RLBM_ENONPHYS, msg);
   }
   return RLBM_OK;
+}
+
+// The read-out parameters with the displacements that pull the state (or none).
+template <class P>
+static P in_place(const P& p, bool fresh) {
+  P q = p;
+  if (fresh) {
+    std::memset(q.b.dxm, 0, sizeof q.b.dxm);
+    std::memset(q.b.dym, 0, sizeof q.b.dym);
+  }
+  return q;
 }
 
 // Context of a third-order (eleven-group) stencil: FP64 or FP32 storage,
@@ -557,8 +577,8 @@ static rlbm_status create_o3(const rlbm_stencil* st, double m, double tau, int N
     c->fo3.reset(new FusedO3Params);
     fill_fused_o3(c.get(), 1.0);
   }
-  if (dtype == RLBM_F64 && (c->fused64 = stencil_o3_kind(c.get())) != 0) {
-    c->fo364.reset(new FusedO364Params);
+  if ((c->kind64 = stencil_o3_kind(c.get())) != 0) {
+    c->io3.reset(new IoO3Params);
     fill_fused_o364(c.get());
   }
   *out = c.release();
@@ -665,8 +685,8 @@ rlbm_status rlbm_create(const rlbm_stencil* st, double m, double tau, int Nx, in
     c->fp.reset(new FusedParams);
     fill_fused(c.get(), 1.0);
   }
-  if (dtype == RLBM_F64 && (c->fused64 = stencil_kind(c.get())) != 0) {
-    c->fp64.reset(new Fused64Params);
+  if (dtype != RLBM_F32 && (c->kind64 = stencil_kind(c.get())) != 0) {
+    c->io2.reset(new Io2Params);
     fill_fused64(c.get());
   }
   if (dtype == RLBM_BF16_DEV) {
@@ -698,20 +718,18 @@ rlbm_status rlbm_init_device(rlbm_ctx* c, const double* n, const double* ux, con
   batch_forget(c);   // its parameters change below
   if (!c->host_init) set_reference(c, 1.0);
   cudaError_t e;
-  if (c->order == 3) {
+  if (c->io3) {
+    e = launch_init_o3c(c->kind64, c->dtype == RLBM_F64, *c->io3, fp, c->buf[0], c->stream);
+  } else if (c->order == 3) {
     e = launch_init_o3(c->dtype, *c->o3, fp, c->buf[0], c->buf[1], c->stream);
-  } else if (c->dtype == RLBM_BF16_DEV) {
-    MomentOut none{nullptr, 0};
-    if (c->fused == 1) e = launch_bf16_io<StencilM1>(0, *c->fp, *c->p64, fp, c->buf[0], c->buf[1], c->coef[0], c->coef[1], none, c->stream);
-    else if (c->fused == 2) e = launch_bf16_io<StencilG16>(0, *c->fp, *c->p64, fp, c->buf[0], c->buf[1], c->coef[0], c->coef[1], none, c->stream);
-    else if (c->fused == 3) e = launch_bf16_io<StencilE5>(0, *c->fp, *c->p64, fp, c->buf[0], c->buf[1], c->coef[0], c->coef[1], none, c->stream);
-    else e = launch_bf16_io<StencilS2>(0, *c->fp, *c->p64, fp, c->buf[0], c->buf[1], c->coef[0], c->coef[1], none, c->stream);
+  } else if (c->io2) {
+    e = launch_init2(c->kind64, c->dtype == RLBM_BF16_DEV, *c->io2, fp, c->buf[0], c->coef[0], c->stream);
   } else if (c->dtype == RLBM_F32 && c->fused) {
     MomentOut none{nullptr, 0};
-    if (c->fused == 1) e = launch_bf16_io<StencilM1>(2, *c->fp, *c->p64, fp, c->buf[0], c->buf[1], nullptr, nullptr, none, c->stream);
-    else if (c->fused == 2) e = launch_bf16_io<StencilG16>(2, *c->fp, *c->p64, fp, c->buf[0], c->buf[1], nullptr, nullptr, none, c->stream);
-    else if (c->fused == 3) e = launch_bf16_io<StencilE5>(2, *c->fp, *c->p64, fp, c->buf[0], c->buf[1], nullptr, nullptr, none, c->stream);
-    else e = launch_bf16_io<StencilS2>(2, *c->fp, *c->p64, fp, c->buf[0], c->buf[1], nullptr, nullptr, none, c->stream);
+    if (c->fused == 1) e = launch_f32_io<StencilM1>(0, *c->fp, *c->p64, fp, c->buf[0], none, c->stream);
+    else if (c->fused == 2) e = launch_f32_io<StencilG16>(0, *c->fp, *c->p64, fp, c->buf[0], none, c->stream);
+    else if (c->fused == 3) e = launch_f32_io<StencilE5>(0, *c->fp, *c->p64, fp, c->buf[0], none, c->stream);
+    else e = launch_f32_io<StencilS2>(0, *c->fp, *c->p64, fp, c->buf[0], none, c->stream);
   } else {
     e = launch_init(c->dtype, *c->p64, fp, c->buf[0], c->buf[1], c->stream);
   }
@@ -719,7 +737,7 @@ rlbm_status rlbm_init_device(rlbm_ctx* c, const double* n, const double* ux, con
   c->cur = 0;
   c->t = 0;
   c->initialised = true;
-  c->fresh = c->order == 2 && c->dtype == RLBM_F32 && c->fused;
+  c->fresh = c->io2 || c->io3 || (c->order == 2 && c->dtype == RLBM_F32 && c->fused);
   return RLBM_OK;
 }
 
@@ -779,9 +797,9 @@ rlbm_status rlbm_step(rlbm_ctx* c, int nsteps) {
     cudaError_t e;
     if (c->order == 3)
       e = c->fo3     ? launch_fused_o3(c->fused, *c->fo3, fin, fout, c->stream)
-          : c->fo364 ? launch_fused_f64_o3(c->fused64, *c->fo364, fin, fout, c->stream)
+          : c->io3 && c->dtype == RLBM_F64 ? launch_fused_f64_o3(c->kind64, c->io3->b, fin, fout, c->stream)
                      : launch_step_o3(c->dtype, *c->o3, fin, fout, c->stream);
-    else if (c->fused64) e = launch_fused_f64(c->fused64, *c->fp64, fin, fout, c->stream);
+    else if (c->dtype == RLBM_F64 && c->io2) e = launch_fused_f64(c->kind64, c->io2->b, fin, fout, c->stream);
     else if (c->dtype == RLBM_F64) e = launch_step_f64(*c->p64, fin, fout, c->qb, c->stream);
     else if (c->fused) {
       const int mode = fused_mode(c);
@@ -830,27 +848,25 @@ rlbm_status rlbm_moments(rlbm_ctx* c, double* out, unsigned mask) {
   }
   MomentOut mo{direct ? direct : c->d_out, mask};
   cudaError_t e;
-  if (c->order == 3) {
-    e = launch_moments_o3(c->dtype, *c->o3, c->buf[1 - c->cur], mo, c->stream);
-  } else if (c->dtype == RLBM_BF16_DEV) {
-    FieldPtrs none{nullptr, nullptr, nullptr, nullptr};
-    void* pv = c->buf[1 - c->cur];
-    void* cp = c->coef[1 - c->cur];
-    if (c->fused == 1) e = launch_bf16_io<StencilM1>(1, *c->fp, *c->p64, none, nullptr, pv, nullptr, cp, mo, c->stream);
-    else if (c->fused == 2) e = launch_bf16_io<StencilG16>(1, *c->fp, *c->p64, none, nullptr, pv, nullptr, cp, mo, c->stream);
-    else if (c->fused == 3) e = launch_bf16_io<StencilE5>(1, *c->fp, *c->p64, none, nullptr, pv, nullptr, cp, mo, c->stream);
-    else e = launch_bf16_io<StencilS2>(1, *c->fp, *c->p64, none, nullptr, pv, nullptr, cp, mo, c->stream);
+  // the state at t is the pull of S_{t-1}; right after a compiled init, S_0 read in place
+  const void* src = c->fresh ? c->buf[c->cur] : c->buf[1 - c->cur];
+  if (c->io3) {
+    e = launch_moments_o3c(c->kind64, c->dtype == RLBM_F64, in_place(*c->io3, c->fresh), src, mo, c->stream);
+  } else if (c->order == 3) {
+    e = launch_moments_o3(c->dtype, *c->o3, src, mo, c->stream);
+  } else if (c->io2) {
+    e = launch_moments2(c->kind64, c->dtype == RLBM_BF16_DEV, in_place(*c->io2, c->fresh), src,
+                        c->fresh ? c->coef[c->cur] : c->coef[1 - c->cur], mo, c->stream);
   } else if (c->dtype == RLBM_F32 && c->fused) {
-    // the state at t is the pull of S_{t-1}; right after the init, S_0 read in place
     FieldPtrs none{nullptr, nullptr, nullptr, nullptr};
-    void* pv = c->fresh ? c->buf[c->cur] : c->buf[1 - c->cur];
-    const int what = c->fresh ? 4 : 3;
-    if (c->fused == 1) e = launch_bf16_io<StencilM1>(what, *c->fp, *c->p64, none, nullptr, pv, nullptr, nullptr, mo, c->stream);
-    else if (c->fused == 2) e = launch_bf16_io<StencilG16>(what, *c->fp, *c->p64, none, nullptr, pv, nullptr, nullptr, mo, c->stream);
-    else if (c->fused == 3) e = launch_bf16_io<StencilE5>(what, *c->fp, *c->p64, none, nullptr, pv, nullptr, nullptr, mo, c->stream);
-    else e = launch_bf16_io<StencilS2>(what, *c->fp, *c->p64, none, nullptr, pv, nullptr, nullptr, mo, c->stream);
+    void* pv = const_cast<void*>(src);
+    const int what = c->fresh ? 2 : 1;
+    if (c->fused == 1) e = launch_f32_io<StencilM1>(what, *c->fp, *c->p64, none, pv, mo, c->stream);
+    else if (c->fused == 2) e = launch_f32_io<StencilG16>(what, *c->fp, *c->p64, none, pv, mo, c->stream);
+    else if (c->fused == 3) e = launch_f32_io<StencilE5>(what, *c->fp, *c->p64, none, pv, mo, c->stream);
+    else e = launch_f32_io<StencilS2>(what, *c->fp, *c->p64, none, pv, mo, c->stream);
   } else {
-    e = launch_moments(c->dtype, *c->p64, c->buf[1 - c->cur], mo, c->stream);
+    e = launch_moments(c->dtype, *c->p64, src, mo, c->stream);
   }
   if (e != cudaSuccess) return cuda_fail(c, e, "moments launch");
   if (!direct) {

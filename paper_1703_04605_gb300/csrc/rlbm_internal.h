@@ -158,6 +158,20 @@ struct FusedParams {
   int doff[kMaxQ2], dcoff[kMaxQ2];
 };
 
+// Fields read by the init kernel and written by the moments kernel.
+struct FieldPtrs {
+  const double* n;
+  const double* ux;
+  const double* uy;
+  const double* T;
+};
+
+struct MomentOut {
+  double* out;           // device-accessible buffer (device memory or mapped
+                         // page-locked host memory), planes of Nx*Ny doubles
+  unsigned mask;
+};
+
 // Stencil-specialised FP64 step (rlbm_fused64.cu): group momenta gm and folded
 // equilibrium constants gf of StencilBuild in FP64; dxm, dym: displacement D
 // at [D + 6], reduced modulo the lattice into [0, N).
@@ -176,6 +190,19 @@ struct Fused64Params {
 
 // kind 1..4: the stencils of rlbm_info.kernel
 cudaError_t launch_fused_f64(int kind, const Fused64Params& p, const void* fin, void* fout, cudaStream_t s);
+
+// Init and read-out of compiled second-order stencils in FP64 and
+// BF16-deviation storage (rlbm_io2.cu): the FP64 step's parameters (dxm, dym all
+// zero: read in place), n R and the moments of the reference state that the
+// storage subtracts (zero for FP64 storage).
+struct Io2Params {
+  Fused64Params b;
+  double ref;
+  double mref[9];
+};
+cudaError_t launch_init2(int kind, bool bf, const Io2Params& p, FieldPtrs f, void* cur, void* ccur, cudaStream_t s);
+cudaError_t launch_moments2(int kind, bool bf, const Io2Params& p, const void* prev, const void* cprev, MomentOut mo,
+                            cudaStream_t s);
 
 // One lattice of a persistent batch launch (device memory; rlbm_persist.cuh).
 struct PersistLattice {
@@ -207,20 +234,6 @@ enum : unsigned {
   ERR_EOS = 4u,      // e/n <= m or T <= 0 or non-finite
   ERR_ZETA = 8u,     // zeta outside the tabulated range
   ERR_TIMEOUT = 16u, // a bounded device-side wait ran out (persistent batch)
-};
-
-// Fields read by the init kernel and written by the moments kernel.
-struct FieldPtrs {
-  const double* n;
-  const double* ux;
-  const double* uy;
-  const double* T;
-};
-
-struct MomentOut {
-  double* out;           // device-accessible buffer (device memory or mapped
-                         // page-locked host memory), planes of Nx*Ny doubles
-  unsigned mask;
 };
 
 // Validation of uploaded initial fields (rlbm_init, rlbm3_init), on the
@@ -303,6 +316,17 @@ struct FusedO364Params {
 
 // kind 5..10 as launch_fused_o3
 cudaError_t launch_fused_f64_o3(int kind, const FusedO364Params& p, const void* fin, void* fout, cudaStream_t s);
+
+// Init and read-out of compiled third-order stencils (rlbm_io_o3.cu), as
+// Io2Params: nref and mref are zero for FP64 storage.
+struct IoO3Params {
+  FusedO364Params b;
+  double nref;
+  double mref[9];
+};
+cudaError_t launch_init_o3c(int kind, bool f64, const IoO3Params& p, FieldPtrs f, void* cur, cudaStream_t s);
+cudaError_t launch_moments_o3c(int kind, bool f64, const IoO3Params& p, const void* prev, MomentOut mo,
+                               cudaStream_t s);
 
 // kind 5, 6, 7: groups {1,2,5,6,7,9,10,11,12,13,15}, {2,3,5,6,7,8,9,10,11,13,15},
 // {1,2,3,6,7,8,9,10,11,13,15}; 8, 9, 10: {8,15,20,24,26,27,28,30,36,37,42},

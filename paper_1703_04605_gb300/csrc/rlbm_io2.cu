@@ -1,0 +1,185 @@
+// Init and read-out of the compiled second-order stencils, FP64 and
+// BF16-deviation storage (rlbm_io.cuh; FP32 storage: rlbm_fused.cuh).
+#include "rlbm_fused.cuh"
+#include "rlbm_io.cuh"
+
+namespace rlbm {
+namespace {
+
+// BF16-deviation storage: the values f - r = d + ref of a source site, ref from
+// its coefficient word (bf_ref of rlbm_fused.cuh).  Every term is exact in FP32,
+// and their sum is carried as an FP32 number and its rounding error.
+struct PullBF {
+  const unsigned short* fin;
+  const uint2* cin;
+  size_t plane;
+  unsigned pitch;
+  int x, y, Nx, Ny;
+  const int *dxm, *dym;
+};
+
+template <class Def, int I>
+__device__ __forceinline__ double pull64(const PullBF& q) {
+  constexpr int nx = Def::F.nx[I], ny = Def::F.ny[I], g = Def::F.grp[I], mult = Def::F.mult[I];
+  constexpr int word = Def::B.word[I], half = Def::B.half[I];
+  const unsigned xs = (unsigned)wrap_sub(q.x, q.dxm[nx + kMaxDisp], q.Nx);
+  const unsigned ys = (unsigned)wrap_sub(q.y, q.dym[ny + kMaxDisp], q.Ny);
+  const unsigned idx = ys * q.pitch + xs;
+  const uint2 c = __ldg(q.cin + idx + q.plane * g);
+  const unsigned h = __ldg(q.fin + 2 * (size_t)idx + half + 2 * q.plane * word);
+  float s = (float)mult * bf_lo(c.x), e = 0.0f, t;
+  if constexpr (nx * nx + ny * ny != 0) {
+    s = ex_two_sum(s, (float)(mult * (nx * nx + ny * ny)) * bf_hi(c.y), t);
+    e += t;
+  }
+  if constexpr (ny != 0) {
+    s = ex_two_sum(s, (float)(mult * ny) * bf_lo(c.y), t);
+    e += t;
+  }
+  if constexpr (nx != 0) {
+    s = ex_two_sum(s, (float)(mult * nx) * bf_hi(c.x), t);
+    e += t;
+  }
+  s = ex_two_sum(s, __uint_as_float(h << 16), t);
+  e += t;
+  return (double)s + (double)e;
+}
+
+// Puts an equilibrium value as its deviation from the site's own reference.
+struct PutBF {
+  unsigned* out;   // the site's word of word plane 0
+  size_t plane;
+  uint2 cq;        // coefficient word of the current group
+  template <class Def, int I>
+  __device__ __forceinline__ float dev(double v) const {
+    constexpr int nx = Def::F.nx[I], ny = Def::F.ny[I], mult = Def::F.mult[I];
+    return (float)(v - (double)bf_ref<nx, ny, mult>(cq));
+  }
+  template <class Def, int I>
+  __device__ __forceinline__ void one(double v) const {
+    constexpr int word = Def::B.word[I], half = Def::B.half[I];
+    unsigned short* w = reinterpret_cast<unsigned short*>(out + plane * word);
+    __stcs(w + half, __bfloat16_as_ushort(__float2bfloat16_rn(dev<Def, I>(v))));
+  }
+  template <class Def, int I, int J>
+  __device__ __forceinline__ void pair(double a, double b) const {
+    static_assert(Def::B.word[I] == Def::B.word[J] && Def::B.half[I] == 0, "orbit partners share a word");
+    constexpr int word = Def::B.word[I];
+    __stcs(out + plane * word, bf_pack(dev<Def, I>(a), dev<Def, J>(b)));
+  }
+};
+
+template <class Def, int K, class Put>
+__device__ __forceinline__ void init_orbit(const Io2Params& p, const double (&r)[10], double (&c)[6], Put& put,
+                                           uint2* cout) {
+  constexpr int g = Def::O.grp[K], ax = Def::O.ax[K], ay = Def::O.ay[K];
+  constexpr double m = (double)Def::O.mult[K];
+  if constexpr (orbit_starts_group<Def, K>()) {
+    group_coeffs64(p.b.gf[g], r, c);
+    if constexpr (std::is_same<Put, PutBF>::value) {
+      put.cq.x = bf_pack((float)c[0], (float)c[1]);
+      put.cq.y = bf_pack((float)c[2], (float)(0.5 * (c[3] + c[4])));
+      __stcs(cout + put.plane * g, put.cq);
+    }
+  }
+  double E = m == 1.0 ? c[0] : m * c[0];
+  if constexpr (ax != 0) E = fma(m * (double)(ax * ax), c[3], E);
+  if constexpr (ay != 0) E = fma(m * (double)(ay * ay), c[4], E);
+  emit_orbit<Def, K>(put, E, (m * (double)ax) * c[1], (m * (double)ay) * c[2], (m * (double)(ax * ay)) * c[5]);
+}
+
+template <class Def, class Put, int... Ks>
+__device__ __forceinline__ void init_all(std::integer_sequence<int, Ks...>, const Io2Params& p, const double (&r)[10],
+                                         Put& put, uint2* cout) {
+  double c[6];
+  (init_orbit<Def, Ks>(p, r, c, put, cout), ...);
+}
+
+template <class Def, bool BF>
+__global__ void __launch_bounds__(128) init2_kernel(const __grid_constant__ Io2Params p, FieldPtrs fd,
+                                                    void* __restrict__ cur, uint2* __restrict__ ccur) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned fl = 0;
+  if (s < p.b.Nx * p.b.Ny) {
+    int x, y;
+    site_of(s, p.b.Nx, x, y);
+    const Macro<double> o = macro_of_fields64(fd.n[s], fd.ux[s], fd.uy[s], fd.T[s], p.b.sc, p.b.rt64, fl);
+    double r[10];
+    projections64(p.b.sc, o, p.ref, r);
+    const unsigned here = (unsigned)y * (unsigned)p.b.pitch + (unsigned)x;
+    using Orb = std::make_integer_sequence<int, Def::O.K>;
+    if constexpr (BF) {
+      PutBF put{static_cast<unsigned*>(cur) + here, (size_t)p.b.plane, make_uint2(0u, 0u)};
+      init_all<Def>(Orb{}, p, r, put, ccur + here);
+    } else {
+      PutPlain<double> put{static_cast<double*>(cur) + here, (size_t)p.b.plane};
+      init_all<Def>(Orb{}, p, r, put, nullptr);
+    }
+  }
+  report(fl, p.b.err);
+}
+
+template <class Def, bool BF>
+__global__ void __launch_bounds__(64, 8) moments2_kernel(const __grid_constant__ Io2Params p,
+                                                         const void* __restrict__ prev,
+                                                         const uint2* __restrict__ cprev, MomentOut mo) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned fl = 0;
+  const long long N = (long long)p.b.Nx * p.b.Ny;
+  if (s < N) {
+    int x, y;
+    site_of(s, p.b.Nx, x, y);
+    double m[9];
+    using Orb = std::make_integer_sequence<int, Def::O.K>;
+    if constexpr (BF)
+      acc64_all<Def>(Orb{},
+                     PullBF{static_cast<const unsigned short*>(prev), cprev, (size_t)p.b.plane, (unsigned)p.b.pitch, x,
+                            y, p.b.Nx, p.b.Ny, p.b.dxm, p.b.dym},
+                     p.b.gm, m);
+    else
+      acc64_all<Def>(Orb{},
+                     Pull64{static_cast<const double*>(prev), (size_t)p.b.plane, (unsigned)p.b.pitch, x, y, p.b.Nx,
+                            p.b.Ny, p.b.dxm, p.b.dym},
+                     p.b.gm, m);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) m[k] += p.mref[k];
+    const Macro<double> o = solve_site_f64_seeded(m, p.b.sc, p.b.rt64, p.b.rt32, fl);
+    write_planes64(mo, N, s, m, o);
+  }
+  report(fl, p.b.err);
+}
+
+template <class Def>
+cudaError_t init2(bool bf, const Io2Params& p, FieldPtrs f, void* cur, void* ccur, cudaStream_t s) {
+  const unsigned grid = (unsigned)(((long long)p.b.Nx * p.b.Ny + 127) / 128);
+  if (bf) init2_kernel<Def, true><<<grid, 128, 0, s>>>(p, f, cur, static_cast<uint2*>(ccur));
+  else init2_kernel<Def, false><<<grid, 128, 0, s>>>(p, f, cur, nullptr);
+  return cudaGetLastError();
+}
+
+template <class Def>
+cudaError_t moments2(bool bf, const Io2Params& p, const void* prev, const void* cprev, MomentOut mo, cudaStream_t s) {
+  const unsigned grid = (unsigned)(((long long)p.b.Nx * p.b.Ny + 63) / 64);
+  if (bf) moments2_kernel<Def, true><<<grid, 64, 0, s>>>(p, prev, static_cast<const uint2*>(cprev), mo);
+  else moments2_kernel<Def, false><<<grid, 64, 0, s>>>(p, prev, nullptr, mo);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_init2(int kind, bool bf, const Io2Params& p, FieldPtrs f, void* cur, void* ccur, cudaStream_t s) {
+  if (kind == 1) return init2<StencilM1>(bf, p, f, cur, ccur, s);
+  if (kind == 2) return init2<StencilG16>(bf, p, f, cur, ccur, s);
+  if (kind == 3) return init2<StencilE5>(bf, p, f, cur, ccur, s);
+  return init2<StencilS2>(bf, p, f, cur, ccur, s);
+}
+
+cudaError_t launch_moments2(int kind, bool bf, const Io2Params& p, const void* prev, const void* cprev, MomentOut mo,
+                            cudaStream_t s) {
+  if (kind == 1) return moments2<StencilM1>(bf, p, prev, cprev, mo, s);
+  if (kind == 2) return moments2<StencilG16>(bf, p, prev, cprev, mo, s);
+  if (kind == 3) return moments2<StencilE5>(bf, p, prev, cprev, mo, s);
+  return moments2<StencilS2>(bf, p, prev, cprev, mo, s);
+}
+
+}  // namespace rlbm

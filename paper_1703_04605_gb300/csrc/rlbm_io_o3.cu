@@ -1,0 +1,112 @@
+// Init and read-out of the compiled third-order stencils on 2D lattices, FP64 and
+// FP32 storage (rlbm_io.cuh).
+#include "rlbm_fused64_o3.cuh"
+#include "rlbm_io.cuh"
+
+namespace rlbm {
+namespace {
+
+template <class Def, int K, class Put>
+__device__ __forceinline__ void init_orbit(const IoO3Params& p, const double (&e)[kO3Mono], double dn, const Put& put) {
+  double E, X, Y, Z;
+  orbit_equilibrium_o3<Def, K>(p.b.ow[K], e, dn, E, X, Y, Z);
+  emit_orbit<Def, K>(put, E, X, Y, Z);
+}
+
+template <class Def, class Put, int... Ks>
+__device__ __forceinline__ void init_all(std::integer_sequence<int, Ks...>, const IoO3Params& p,
+                                         const double (&e)[kO3Mono], double dn, const Put& put) {
+  (init_orbit<Def, Ks>(p, e, dn, put), ...);
+}
+
+template <class Def, typename S>
+__global__ void __launch_bounds__(128) init_o3c_kernel(const __grid_constant__ IoO3Params p, FieldPtrs fd,
+                                                       S* __restrict__ cur) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned fl = 0;
+  if (s < p.b.Nx * p.b.Ny) {
+    int x, y;
+    site_of(s, p.b.Nx, x, y);
+    const Macro<double> o = macro_of_fields64(fd.n[s], fd.ux[s], fd.uy[s], fd.T[s], p.b.sc, p.b.rt64, fl);
+    double e[kO3Mono];
+    deviations64(p.b, o, e);
+    const PutPlain<S> put{cur + ((unsigned)y * (unsigned)p.b.pitch + (unsigned)x), (size_t)p.b.plane};
+    init_all<Def>(std::make_integer_sequence<int, Def::O.K>{}, p, e, o.n - p.nref, put);
+  }
+  report(fl, p.b.err);
+}
+
+template <typename S>
+struct PullOf;
+template <>
+struct PullOf<double> {
+  using type = Pull64;
+};
+template <>
+struct PullOf<float> {
+  using type = Pull32;
+};
+
+template <class Def, typename S>
+__global__ void __launch_bounds__(64, 8) moments_o3c_kernel(const __grid_constant__ IoO3Params p,
+                                                            const S* __restrict__ prev, MomentOut mo) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned fl = 0;
+  const long long N = (long long)p.b.Nx * p.b.Ny;
+  if (s < N) {
+    int x, y;
+    site_of(s, p.b.Nx, x, y);
+    double m[9];
+    const typename PullOf<S>::type q{prev, (size_t)p.b.plane, (unsigned)p.b.pitch, x, y, p.b.Nx, p.b.Ny, p.b.dxm,
+                                     p.b.dym};
+    acc64_all<Def>(std::make_integer_sequence<int, Def::O.K>{}, q, p.b.gm, m);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) m[k] += p.mref[k];
+    const Macro<double> o = solve_site_f64_seeded(m, p.b.sc, p.b.rt64, p.b.rt32, fl);
+    write_planes64(mo, N, s, m, o);
+  }
+  report(fl, p.b.err);
+}
+
+template <class Def>
+cudaError_t init3(bool f64, const IoO3Params& p, FieldPtrs f, void* cur, cudaStream_t s) {
+  const unsigned grid = (unsigned)(((long long)p.b.Nx * p.b.Ny + 127) / 128);
+  if (f64) init_o3c_kernel<Def, double><<<grid, 128, 0, s>>>(p, f, static_cast<double*>(cur));
+  else init_o3c_kernel<Def, float><<<grid, 128, 0, s>>>(p, f, static_cast<float*>(cur));
+  return cudaGetLastError();
+}
+
+template <class Def>
+cudaError_t moments3(bool f64, const IoO3Params& p, const void* prev, MomentOut mo, cudaStream_t s) {
+  const unsigned grid = (unsigned)(((long long)p.b.Nx * p.b.Ny + 63) / 64);
+  if (f64) moments_o3c_kernel<Def, double><<<grid, 64, 0, s>>>(p, static_cast<const double*>(prev), mo);
+  else moments_o3c_kernel<Def, float><<<grid, 64, 0, s>>>(p, static_cast<const float*>(prev), mo);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_init_o3c(int kind, bool f64, const IoO3Params& p, FieldPtrs f, void* cur, cudaStream_t s) {
+  switch (kind) {
+    case 5: return init3<StencilO3M5>(f64, p, f, cur, s);
+    case 6: return init3<StencilO3D>(f64, p, f, cur, s);
+    case 7: return init3<StencilO3E>(f64, p, f, cur, s);
+    case 8: return init3<StencilO3A>(f64, p, f, cur, s);
+    case 9: return init3<StencilO3B>(f64, p, f, cur, s);
+    default: return init3<StencilO3C>(f64, p, f, cur, s);
+  }
+}
+
+cudaError_t launch_moments_o3c(int kind, bool f64, const IoO3Params& p, const void* prev, MomentOut mo,
+                               cudaStream_t s) {
+  switch (kind) {
+    case 5: return moments3<StencilO3M5>(f64, p, prev, mo, s);
+    case 6: return moments3<StencilO3D>(f64, p, prev, mo, s);
+    case 7: return moments3<StencilO3E>(f64, p, prev, mo, s);
+    case 8: return moments3<StencilO3A>(f64, p, prev, mo, s);
+    case 9: return moments3<StencilO3B>(f64, p, prev, mo, s);
+    default: return moments3<StencilO3C>(f64, p, prev, mo, s);
+  }
+}
+
+}  // namespace rlbm
