@@ -52,6 +52,11 @@ struct rlbm_ctx3 {
   float* d_w32 = nullptr;
   Step3O3Params q{};
   std::unique_ptr<Fused3O3Params> fo3;   // compiled FP32 third-order kernel
+  // compiled stencil, whatever the lattice's size: FP64 step, init, read-out
+  int kind = 0;                          // second order: 1..4
+  std::unique_ptr<C3Params2> c2;
+  std::unique_ptr<C3Params3> c3;
+  bool fresh = false;                    // S_0 written in place by such an init, not stepped yet
   std::unique_ptr<StencilBuild3O3> s3;
   DevMem mem;                  // device allocator (rlbm_set_allocator at creation)
   std::string last_error;
@@ -88,8 +93,8 @@ HL split3(double v) {
   return h;
 }
 
-// The compiled 3D stencil for these groups, when its population order is the
-// host's (the storage planes) and the lattice is at least a halo wide.
+// Whether the context's stencil is the compiled one, in the compiled population
+// order (the storage planes).
 template <class D>
 bool same_order(const rlbm_ctx3* c, const int* groups) {
   for (int g : D::groups)
@@ -99,17 +104,88 @@ bool same_order(const rlbm_ctx3* c, const int* groups) {
     const Pop3& q = c->sb.pops[i];
     if (q.group != D::U.grp[i] || q.nx != D::U.nx[i] || q.ny != D::U.ny[i] || q.nz != D::U.nz[i]) return false;
   }
-  const int h = D::U.halo;
+  return true;
+}
+
+int stencil3_kind(const rlbm_ctx3* c) {
+  const int* g = c->sb.sb.groups;
+  if (same_order<Stencil3M1>(c, g)) return 1;
+  if (same_order<Stencil3G16>(c, g)) return 2;
+  if (same_order<Stencil3E5>(c, g)) return 3;
+  if (same_order<Stencil3S2>(c, g)) return 4;
+  return 0;
+}
+
+// The compiled FP32 kernels wrap a source coordinate at most once.
+bool halo_wide(const rlbm_ctx3* c) {
+  const int h = c->sb.halo;
   return c->Nx >= h && c->Ny >= h && c->Nz >= h;
 }
 
-int fused3_kind(const rlbm_ctx3* c) {
-  if (c->dtype != RLBM_F32) return 0;
-  if (same_order<Stencil3M1>(c, c->sb.sb.groups)) return 1;
-  if (same_order<Stencil3G16>(c, c->sb.sb.groups)) return 2;
-  if (same_order<Stencil3E5>(c, c->sb.sb.groups)) return 3;
-  if (same_order<Stencil3S2>(c, c->sb.sb.groups)) return 4;
-  return 0;
+// Fields that the compiled FP64-arithmetic kernels of both orders share.
+void fill_c3(const rlbm_ctx3* c, C3Params& f) {
+  f.Nx = c->Nx;
+  f.Ny = c->Ny;
+  f.Nz = c->Nz;
+  f.pitch = c->pitch;
+  f.zstride = c->pitch * c->Ny;
+  f.plane = c->plane;
+  f.inv_tau = 1.0 / c->tau;
+  f.v0 = c->sb.sb.v0;
+  f.sc = c->sb.sb.sc;
+  for (int d = -6; d <= 6; ++d) {
+    f.dxm[d + 6] = ((d % c->Nx) + c->Nx) % c->Nx;
+    f.dym[d + 6] = ((d % c->Ny) + c->Ny) % c->Ny;
+    f.dzm[d + 6] = ((d % c->Nz) + c->Nz) % c->Nz;
+  }
+  f.rt64 = c->d_rt64;
+  f.rt32 = c->d_rt32;
+  f.err = c->d_err;
+}
+
+void fill_c2(rlbm_ctx3* c) {
+  C3Params2& f = *c->c2;
+  std::memset(&f, 0, sizeof f);
+  fill_c3(c, f);
+  for (int g = 0; g < 6; ++g) {
+    for (int q = 0; q < 5; ++q) f.gm[g][q] = c->sb.sb.gm[g][q];
+    for (int q = 0; q < 10; ++q) f.gf[g][q] = c->sb.gf3[g][q];
+  }
+}
+
+void fill_c3o3(rlbm_ctx3* c, const StencilBuild3O3& s3) {
+  C3Params3& f = *c->c3;
+  std::memset(&f, 0, sizeof f);
+  fill_c3(c, f);
+  f.c = s3.c;
+  for (int g = 0; g < 11; ++g)
+    for (int q = 0; q < 5; ++q) f.gm[g][q] = s3.gm[g][q];
+  using D = Stencil3O3M5;
+  for (int k = 0; k < D::O.K; ++k) {
+    const int i = D::O.idx[k][0];
+    f.ow[k][0] = c->sb.pops[i].c[14];
+    for (int l = 0; l < kO3Mono3; ++l) f.ow[k][1 + l] = s3.wrows[i][l];
+  }
+}
+
+// The reference state of the FP32 storage, and the displacements of a read-out.
+template <class P>
+void set_reference_c3(const rlbm_ctx3* c, P* f) {
+  if (!f) return;
+  f->nref = c->p.nref;
+  f->ref = c->p.nref * c->sb.mref1[0] * c->sb.sb.sc.Rr;
+  for (int k = 0; k < 14; ++k) f->mref[k] = c->p.mref[k];
+}
+
+template <class P>
+P in_place3(const P& p, bool fresh) {
+  P q = p;
+  if (fresh) {
+    std::memset(q.dxm, 0, sizeof q.dxm);
+    std::memset(q.dym, 0, sizeof q.dym);
+    std::memset(q.dzm, 0, sizeof q.dzm);
+  }
+  return q;
 }
 
 // Parameters of the stencil-specialised 3D kernel at reference density nref.
@@ -195,6 +271,8 @@ void set_reference3(rlbm_ctx3* c, double nref) {
   for (int k = 0; k < 14; ++k) c->p.mref[k] = nref * c->sb.mref1[k];
   if (c->fused) fill_fused3(c, nref);
   if (c->fo3) fill_fused3_o3(c, nref);
+  set_reference_c3(c, c->c2.get());
+  set_reference_c3(c, c->c3.get());
 }
 
 rlbm_status check_error3(rlbm_ctx3* c) {
@@ -349,15 +427,22 @@ rlbm_status rlbm3_create(const rlbm_stencil* st, double m, double tau, int Nx, i
   p.tab64 = c->d_tab64;
   p.tab32 = c->d_tab32;
   p.err = c->d_err;
-  c->fused = c->order == 3 ? 0 : fused3_kind(c.get());
   if (c->order == 3) {
     c->q.c = s3->c;
     c->q.w64 = c->d_w64;
     c->q.w32 = c->d_w32;
-    if (dtype == RLBM_F32 && same_order<Stencil3O3M5>(c.get(), s3->groups)) {
-      c->fo3.reset(new Fused3O3Params);
-      c->s3 = std::move(s3);
+    if (same_order<Stencil3O3M5>(c.get(), s3->groups)) {
+      c->c3.reset(new C3Params3);
+      fill_c3o3(c.get(), *s3);
+      if (dtype == RLBM_F32 && halo_wide(c.get())) {
+        c->fo3.reset(new Fused3O3Params);
+        c->s3 = std::move(s3);
+      }
     }
+  } else if ((c->kind = stencil3_kind(c.get())) != 0) {
+    c->c2.reset(new C3Params2);
+    fill_c2(c.get());
+    if (dtype == RLBM_F32 && halo_wide(c.get())) c->fused = c->kind;
   }
   set_reference3(c.get(), 1.0);
   *out = c.release();
@@ -392,12 +477,16 @@ rlbm_status rlbm3_init(rlbm_ctx3* c, const double* n, const double* ux, const do
   set_reference3(c, fs.nsum / (double)N);
   Field3Ptrs fp{c->d_fields, c->d_fields + N, c->d_fields + 2 * N, c->d_fields + 3 * N, c->d_fields + 4 * N};
   c->q.b = c->p;
-  cudaError_t e = c->order == 3 ? launch_init3d_o3(c->dtype, c->q, fp, c->buf[0], c->buf[1], c->stream)
-                                : launch_init3d(c->dtype, c->p, fp, c->buf[0], c->buf[1], c->stream);
+  const bool f64 = c->dtype == RLBM_F64;
+  cudaError_t e = c->c2           ? launch_init3c(c->kind, f64, *c->c2, fp, c->buf[0], c->stream)
+                  : c->c3         ? launch_init3c(f64, *c->c3, fp, c->buf[0], c->stream)
+                  : c->order == 3 ? launch_init3d_o3(c->dtype, c->q, fp, c->buf[0], c->buf[1], c->stream)
+                                  : launch_init3d(c->dtype, c->p, fp, c->buf[0], c->buf[1], c->stream);
   if (e != cudaSuccess) return cuda_fail3(c, e, "init launch");
   c->cur = 0;
   c->t = 0;
   c->initialised = true;
+  c->fresh = c->c2 || c->c3;
   return check_error3(c);
 }
 
@@ -409,12 +498,15 @@ rlbm_status rlbm3_step(rlbm_ctx3* c, int nsteps) {
   for (int k = 0; k < nsteps; ++k) {
     cudaError_t e;
     if (c->fo3) e = launch_fused3d_o3(*c->fo3, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
+    else if (c->c3 && c->dtype == RLBM_F64) e = launch_step3c(*c->c3, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
+    else if (c->c2 && c->dtype == RLBM_F64) e = launch_step3c(c->kind, *c->c2, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
     else if (c->order == 3) e = launch_step3d_o3(c->dtype, c->q, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
     else if (c->fused) e = launch_fused3d(c->fused, c->fp, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
     else e = launch_step3d(c->dtype, c->p, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
     if (e != cudaSuccess) return cuda_fail3(c, e, "step launch");
     c->cur = 1 - c->cur;
     ++c->t;
+    c->fresh = false;
   }
   return RLBM_OK;
 }
@@ -447,8 +539,13 @@ rlbm_status rlbm3_moments(rlbm_ctx3* c, double* out, unsigned mask) {
     c->out_cap = need;
   }
   MomentOut mo{direct ? direct : c->d_out, mask};
-  // the pre-collision state at t is the pull of S_{t-1}, the buffer the last step read
-  cudaError_t e = launch_moments3d(c->dtype, c->p, c->buf[1 - c->cur], mo, c->stream);
+  // the pre-collision state at t is the pull of S_{t-1}, the buffer the last step
+  // read; right after a compiled init, S_0 read in place
+  const void* src = c->fresh ? c->buf[c->cur] : c->buf[1 - c->cur];
+  const bool f64 = c->dtype == RLBM_F64;
+  cudaError_t e = c->c2   ? launch_moments3c(c->kind, f64, in_place3(*c->c2, c->fresh), src, mo, c->stream)
+                  : c->c3 ? launch_moments3c(f64, in_place3(*c->c3, c->fresh), src, mo, c->stream)
+                          : launch_moments3d(c->dtype, c->p, src, mo, c->stream);
   if (e == cudaSuccess && !direct)
     e = cudaMemcpyAsync(out, c->d_out, need * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
   if (e != cudaSuccess) return cuda_fail3(c, e, "read-out");

@@ -61,6 +61,37 @@ struct Fused3O3Params {
 
 cudaError_t launch_fused3d_o3(const Fused3O3Params& p, const void* fin, void* fout, cudaStream_t s);
 
+// FP64 arithmetic of the compiled 3D stencils (rlbm_fused64_3d.cu): the FP64
+// step, and init and read-out of both storages.  dxm, dym, dzm: displacement D at
+// [D + 6] reduced modulo the lattice (all zero: read in place); mref, ref (n R)
+// and nref: the reference state that FP32 storage subtracts.
+struct C3Params {
+  int Nx, Ny, Nz;
+  long long pitch, zstride, plane;   // elements; zstride = pitch * Ny
+  double inv_tau, v0;
+  SiteConsts sc;
+  double nref, ref;
+  double mref[14];
+  int dxm[13], dym[13], dzm[13];
+  const double* rt64;
+  const float* rt32;
+  unsigned* err;
+};
+struct C3Params2 : C3Params {   // second order: group momenta and the constants gf3
+  double gm[6][5], gf[6][10];
+};
+struct C3Params3 : C3Params {   // third order: dual basis of the octant representatives
+  double c;
+  double gm[11][5];
+  double ow[kMaxOct3][kO3Mono3 + 1];
+};
+cudaError_t launch_step3c(int kind, const C3Params2& p, const void* fin, void* fout, cudaStream_t s);
+cudaError_t launch_step3c(const C3Params3& p, const void* fin, void* fout, cudaStream_t s);
+cudaError_t launch_init3c(int kind, bool f64, const C3Params2& p, Field3Ptrs f, void* cur, cudaStream_t s);
+cudaError_t launch_init3c(bool f64, const C3Params3& p, Field3Ptrs f, void* cur, cudaStream_t s);
+cudaError_t launch_moments3c(int kind, bool f64, const C3Params2& p, const void* prev, MomentOut mo, cudaStream_t s);
+cudaError_t launch_moments3c(bool f64, const C3Params3& p, const void* prev, MomentOut mo, cudaStream_t s);
+
 cudaError_t launch_step3d_o3(rlbm_dtype dt, const Step3O3Params& p, const void* fin, void* fout, cudaStream_t s);
 cudaError_t launch_init3d_o3(rlbm_dtype dt, const Step3O3Params& p, Field3Ptrs f, void* cur, void* prev,
                              cudaStream_t s);

@@ -231,6 +231,8 @@ struct Stencil3Def {
   static constexpr int groups[6] = {G0, G1, G2, G3, G4, G5};
   static constexpr Unfolded U = unfold_stencil(G0, G1, G2, G3, G4, G5);
   static constexpr int Q = U.Q;
+  static constexpr Octants O = make_octants(U);
+  static_assert(octants_cover(U, O), "octant orbits must partition the unfolded stencil");
 };
 
 using Stencil3M1 = Stencil3Def<5, 12, 14, 17, 21, 26>;
