@@ -53,6 +53,7 @@
 #include <utility>
 
 #include "rlbm_kernels.cuh"
+#include "rlbm_pdl.cuh"
 #include "rlbm_stencils.h"
 
 namespace rlbm {
@@ -126,11 +127,15 @@ __device__ __forceinline__ float bf_ref(uint2 c) {
   return r;
 }
 
-// CG: loads through L2 only (ld.global.cg), for kernels that read data other
-// blocks of the same launch wrote (the read-only path may hold stale lines).
-template <bool CG, class T>
+// How populations are loaded: read-only path; L2 only (ld.global.cg), for
+// kernels that read data other blocks of the same launch wrote (L1 may hold
+// stale lines); coherently, for a step launched while the previous one ends
+// (rlbm_pdl.cuh).
+enum PopLoad { LD_RO = 0, LD_CG = 1, LD_CHAIN = 2 };
+template <int LD, class T>
 __device__ __forceinline__ T fused_ld(const T* p) {
-  if constexpr (CG) return __ldcg(p);
+  if constexpr (LD == LD_CG) return __ldcg(p);
+  else if constexpr (LD == LD_CHAIN) return ld_pop(p);
   else return __ldg(p);
 }
 
@@ -139,7 +144,7 @@ __device__ __forceinline__ T fused_ld(const T* p) {
 // a plane offset I plane are formed in 32-bit arithmetic; the address is then
 // one wide multiply-add from the base, where 64-bit index arithmetic costs
 // several integer instructions a population.
-template <class Def, bool BF, int I, bool CG = false>
+template <class Def, bool BF, int I, int LD = LD_RO>
 __device__ __forceinline__ void fused_load(float (&d)[Def::Q], const void* __restrict__ fin,
                                            const uint2* __restrict__ cin, long long plane, long long pitch,
                                            int x, int y, int Nx, int Ny) {
@@ -151,11 +156,11 @@ __device__ __forceinline__ void fused_load(float (&d)[Def::Q], const void* __res
   if constexpr (BF) {
     constexpr int g = Def::F.grp[I], mult = Def::F.mult[I], w = Def::B.word[I], hf = Def::B.half[I];
     const unsigned short h =
-        fused_ld<CG>(static_cast<const unsigned short*>(fin) + 2 * (size_t)idx + hf + 2 * pl * w);
-    const uint2 c = fused_ld<CG>(cin + idx + pl * g);
+        fused_ld<LD>(static_cast<const unsigned short*>(fin) + 2 * (size_t)idx + hf + 2 * pl * w);
+    const uint2 c = fused_ld<LD>(cin + idx + pl * g);
     d[I] = add_bf(h, bf_ref<DX, DY, mult>(c));
   } else {
-    d[I] = fused_ld<CG>(static_cast<const float*>(fin) + idx + pl * I);
+    d[I] = fused_ld<LD>(static_cast<const float*>(fin) + idx + pl * I);
   }
 }
 
@@ -163,12 +168,12 @@ __device__ __forceinline__ void fused_load(float (&d)[Def::Q], const void* __res
 // the value and its coefficient word sit at fixed offsets from the site's
 // own elements (fh: its half-word slot 0 of word plane 0, ch: its
 // coefficient word of group 0), which takes the index arithmetic off the path.
-template <class Def, int I, bool CG = false>
+template <class Def, int I, int LD = LD_RO>
 __device__ __forceinline__ void fused_load_inner(float (&d)[Def::Q], const unsigned short* __restrict__ fh,
                                                  const uint2* __restrict__ ch, const FusedParams& p) {
   constexpr int DX = Def::F.nx[I], DY = Def::F.ny[I], mult = Def::F.mult[I];
-  const unsigned short h = fused_ld<CG>(fh + p.doff[I]);
-  const uint2 c = fused_ld<CG>(ch + p.dcoff[I]);
+  const unsigned short h = fused_ld<LD>(fh + p.doff[I]);
+  const uint2 c = fused_ld<LD>(ch + p.dcoff[I]);
   d[I] = add_bf(h, bf_ref<DX, DY, mult>(c));
 }
 
@@ -498,19 +503,19 @@ __device__ __forceinline__ void fused_collide_orbit(const float (&d)[Def::Q], co
   }
 }
 
-template <class Def, bool CG = false, int... Is>
+template <class Def, int LD = LD_RO, int... Is>
 __device__ __forceinline__ void fused_load_inner_all(std::integer_sequence<int, Is...>, float (&d)[Def::Q],
                                                      const unsigned short* __restrict__ fh,
                                                      const uint2* __restrict__ ch, const FusedParams& p) {
   static_assert(Def::Q <= kMaxQ2, "offset tables hold kMaxQ2 populations");
-  (fused_load_inner<Def, Is, CG>(d, fh, ch, p), ...);
+  (fused_load_inner<Def, Is, LD>(d, fh, ch, p), ...);
 }
 
-template <class Def, bool BF, bool CG = false, int... Is>
+template <class Def, bool BF, int LD = LD_RO, int... Is>
 __device__ __forceinline__ void fused_load_all(std::integer_sequence<int, Is...>, float (&d)[Def::Q],
                                                const void* __restrict__ fin, const uint2* __restrict__ cin,
                                                long long plane, long long pitch, int x, int y, int Nx, int Ny) {
-  (fused_load<Def, BF, Is, CG>(d, fin, cin, plane, pitch, x, y, Nx, Ny), ...);
+  (fused_load<Def, BF, Is, LD>(d, fin, cin, plane, pitch, x, y, Nx, Ny), ...);
 }
 
 template <class Def, int... Ks>
@@ -790,7 +795,7 @@ __device__ __forceinline__ void fused_coeffs(const FusedParams& p, const SplitSi
 }
 
 // One site update (see the header comment); p describes the lattice.
-template <class Def, bool BF, int EXL = 0, bool CG = false>
+template <class Def, bool BF, int EXL = 0, int LD = LD_RO>
 __device__ __forceinline__ void fused_site(const FusedParams& p, const void* __restrict__ fin,
                                            void* __restrict__ fout, int site, unsigned& fl) {
   static_assert(!(BF && EXL), "extended moment sums are for FP32 storage");
@@ -810,13 +815,13 @@ __device__ __forceinline__ void fused_site(const FusedParams& p, const void* __r
     if constexpr (BF) {
       constexpr int H = Def::halo;
       if ((unsigned)(x - H) < (unsigned)p.inner_nx && (unsigned)(y - H) < (unsigned)p.inner_ny)
-        fused_load_inner_all<Def, CG>(Seq{}, d, static_cast<const unsigned short*>(fin) + 2 * (size_t)here,
+        fused_load_inner_all<Def, LD>(Seq{}, d, static_cast<const unsigned short*>(fin) + 2 * (size_t)here,
                                       static_cast<const uint2*>(p.cin) + here, p);
       else
-        fused_load_all<Def, true, CG>(Seq{}, d, fin, static_cast<const uint2*>(p.cin), p.plane, p.pitch, x, y,
+        fused_load_all<Def, true, LD>(Seq{}, d, fin, static_cast<const uint2*>(p.cin), p.plane, p.pitch, x, y,
                                       p.Nx, p.Ny);
     } else {
-      fused_load_all<Def, BF, CG>(Seq{}, d, fin, static_cast<const uint2*>(p.cin), p.plane, p.pitch, x, y, p.Nx,
+      fused_load_all<Def, BF, LD>(Seq{}, d, fin, static_cast<const uint2*>(p.cin), p.plane, p.pitch, x, y, p.Nx,
                                   p.Ny);
     }
     using Orb = std::make_integer_sequence<int, Def::O.K>;
@@ -903,16 +908,24 @@ constexpr int fused_min_blocks() {
   return Def::Q <= 40 ? ((BF || EXL) ? 5 : 6) : ((Def::Q <= 64 && !BF && EXL < 2) ? 5 : 4);
 }
 
-template <class Def, bool BF, int EXL = 0>
+// CHAIN: launched by launch_pdl (rlbm_pdl.cuh).
+template <class Def, bool BF, int EXL = 0, bool CHAIN = true>
 __global__ void __launch_bounds__(128, fused_min_blocks<Def, BF, EXL>()) fused_f32_kernel(const __grid_constant__ FusedParams p,
                                                         const void* __restrict__ fin,
                                                         void* __restrict__ fout) {
   const int site = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned fl = 0;
-  if (site < p.Nx * p.Ny) fused_site<Def, BF, EXL>(p, fin, fout, site, fl);
+  if constexpr (CHAIN) pdl_wait();
+  if (site < p.Nx * p.Ny) fused_site<Def, BF, EXL, CHAIN ? LD_CHAIN : LD_RO>(p, fin, fout, site, fl);
   report(fl, p.err);
 }
 
+// Steps of one lattice are chained, measured (us a step, chained against not):
+// 512^2 M1 FP32 22.0 / 24.6, BF16 29.8 / 31.5, G1-G6 15.4 / 18.3, S2 19.0 / 20.7;
+// 2048^2 M1 297 / 301, S2 BF16 334 / 349; 4096^2 M1 1179 / 1191.  The one kernel
+// that loses on large lattices is E5's FP32 one, which is at the bandwidth and
+// whose loads are slower off the read-only path (2048^2 403 / 391, 512^2
+// 29.9 / 32.8): chained up to 2^20 sites, where the launch saved still counts.
 // Entry point of the step kernel of a stencil, for CUDA graph kernel nodes
 // (rlbm_batch_step); the node's grid is (Nx Ny + 127)/128 blocks of 128.
 // mode: 0 FP32, 1 BF16 deviation, 2 / 3 FP32 with extended moment sums of
@@ -922,18 +935,23 @@ const void* fused_kernel_fn_impl(int mode) {
   return mode == 1 ? (const void*)&fused_f32_kernel<Def, true>
          : mode == 2 ? (const void*)&fused_f32_kernel<Def, false, 1>
          : mode == 3 ? (const void*)&fused_f32_kernel<Def, false, 2>
-                     : (const void*)&fused_f32_kernel<Def, false>;
+                     : (const void*)&fused_f32_kernel<Def, false, 0, Def::Q != 73>;
 }
 
 template <class Def>
 cudaError_t launch_fused_impl(const FusedParams& p, const void* fin, void* fout, int mode, cudaStream_t s) {
   const long long nsite = (long long)p.Nx * p.Ny;
   const unsigned grid = (unsigned)((nsite + 127) / 128);
-  if (mode == 1) fused_f32_kernel<Def, true><<<grid, 128, 0, s>>>(p, fin, fout);
-  else if (mode == 2) fused_f32_kernel<Def, false, 1><<<grid, 128, 0, s>>>(p, fin, fout);
-  else if (mode == 3) fused_f32_kernel<Def, false, 2><<<grid, 128, 0, s>>>(p, fin, fout);
-  else fused_f32_kernel<Def, false><<<grid, 128, 0, s>>>(p, fin, fout);
-  return cudaGetLastError();
+  if (mode == 1) return launch_pdl(fused_f32_kernel<Def, true>, grid, 128, s, p, fin, fout);
+  if (mode == 2) return launch_pdl(fused_f32_kernel<Def, false, 1>, grid, 128, s, p, fin, fout);
+  if (mode == 3) return launch_pdl(fused_f32_kernel<Def, false, 2>, grid, 128, s, p, fin, fout);
+  if constexpr (Def::Q == 73) {
+    if (nsite > (1LL << 20)) {
+      fused_f32_kernel<Def, false, 0, false><<<grid, 128, 0, s>>>(p, fin, fout);
+      return cudaGetLastError();
+    }
+  }
+  return launch_pdl(fused_f32_kernel<Def, false>, grid, 128, s, p, fin, fout);
 }
 
 }  // namespace rlbm

@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(128, fused_min_blocks<Def, BF, EXL>())
     unsigned fl = 0;
     for (int j = 0; j < pp.spt; ++j) {
       const int site = (tile * pp.spt + j) * 128 + (int)threadIdx.x;
-      if (site < L.nsite) fused_site<Def, BF, EXL, true>(sp, fin, fout, site, fl);
+      if (site < L.nsite) fused_site<Def, BF, EXL, LD_CG>(sp, fin, fout, site, fl);
     }
     report(fl, sp.err);
     __syncthreads();   // every store of the unit is issued
