@@ -53,74 +53,11 @@ __global__ void __launch_bounds__(64, 8) fused_f64_kernel(const __grid_constant_
   report(fl, p.err);
 }
 
-// ------------------------------------------------------ four lanes a site
-template <class Def, int K>
-__device__ __forceinline__ void lane_collide(const Fused64Params& p, const Lane64& q, const double (&d)[Def::O.K],
-                                             const double (&r)[10], double (&c)[6], double a0, double wx, double wy) {
-  constexpr int g = Def::O.grp[K], ax = Def::O.ax[K], ay = Def::O.ay[K];
-  constexpr double m = (double)Def::O.mult[K];
-  if constexpr (orbit_starts_group<Def, K>()) {
-    group_coeffs64(p.gf[g], r, c);
-    c[1] = flip(c[1], q.l & 1);
-    c[2] = flip(c[2], q.l >> 1);
-    c[5] = flip(c[5], (q.l ^ (q.l >> 1)) & 1);
-  }
-  double e = m == 1.0 ? c[0] : m * c[0];
-  if constexpr (ax != 0) e = fma(m * (double)(ax * ax), c[3], e);
-  if constexpr (ay != 0) e = fma(m * (double)(ay * ay), c[4], e);
-  if constexpr (ax != 0 && ay != 0) e = fma(m * (double)(ax * ay), c[5], e);
-  if constexpr (ax != 0) e = fma(m * (double)ax, c[1], e);
-  if constexpr (ay != 0) e = fma(m * (double)ay, c[2], e);
-  double om = a0;
-  if constexpr (ax != 0) om = fma(-(double)ax, wx, om);
-  if constexpr (ay != 0) om = fma(-(double)ay, wy, om);
-  if (lane_has<Def, K>(q.l)) __stcs(q.out + q.here + lane_plane<Def, K>(q), fma(om, e - d[K], d[K]));
-}
-
-template <class Def, int... Ks>
-__device__ __forceinline__ void lane_collide_all(std::integer_sequence<int, Ks...>, const Fused64Params& p,
-                                                 const Lane64& q, const double (&d)[Def::O.K], const double (&r)[10],
-                                                 double a0, double wx, double wy) {
-  double c[6];
-  (lane_collide<Def, Ks>(p, q, d, r, c, a0, wx, wy), ...);
-}
-
-template <class Def>
-__global__ void __launch_bounds__(32) fused_f64_quad_kernel(const __grid_constant__ Fused64Params p,
-                                                            const double* __restrict__ fin, double* __restrict__ fout) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nsite = p.Nx * p.Ny;
-  // lanes past the end repeat the last site without storing, so that every
-  // lane takes part in the sums over lanes
-  const bool live = (t >> 2) < nsite;
-  const int site = live ? t >> 2 : nsite - 1;
-  unsigned fl = 0;
-  int x, y;
-  site_of(site, p.Nx, x, y);
-  const Lane64 q{fin, fout, (size_t)p.plane, (unsigned)p.pitch, (unsigned)y * (unsigned)p.pitch + (unsigned)x, x, y,
-                 p.Nx, p.Ny, t & 3, p.dxm, p.dym};
-  using Orb = std::make_integer_sequence<int, Def::O.K>;
-  double d[Def::O.K], M[9];
-  lane_moments_all<Def>(Orb{}, q, d, p.gm, M);
-  const Macro<double> o = solve_site_f64_seeded(M, p.sc, p.rt64, p.rt32, fl);
-  double r[10];
-  projections64(p.sc, o, 0.0, r);
-  const double wv = p.v0 * p.inv_tau;
-  if (live)
-    lane_collide_all<Def>(Orb{}, p, q, d, r, o.U0 * p.inv_tau, flip(wv * o.Ux, q.l & 1), flip(wv * o.Uy, q.l >> 1));
-  report(fl, p.err);
-}
-
 template <class Def>
 cudaError_t launch64(const Fused64Params& p, const void* fin, void* fout, cudaStream_t s) {
   const long long nsite = (long long)p.Nx * p.Ny;
-  if (nsite <= kQuadSites * p.sms) {
-    fused_f64_quad_kernel<Def><<<(unsigned)((nsite + 7) / 8), 32, 0, s>>>(p, static_cast<const double*>(fin),
-                                                                          static_cast<double*>(fout));
-  } else {
-    fused_f64_kernel<Def><<<(unsigned)((nsite + 63) / 64), 64, 0, s>>>(p, static_cast<const double*>(fin),
-                                                                       static_cast<double*>(fout));
-  }
+  fused_f64_kernel<Def><<<(unsigned)((nsite + 63) / 64), 64, 0, s>>>(p, static_cast<const double*>(fin),
+                                                                     static_cast<double*>(fout));
   return cudaGetLastError();
 }
 

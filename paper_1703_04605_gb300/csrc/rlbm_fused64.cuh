@@ -16,10 +16,10 @@
 //    to the all-FP64 iterations of solve_site_f64, so every state is treated,
 //    and every error bit set, as there.
 //
-// Measured (M1, FP64): 256^2 272 -> 107 us a step, 800 x 1 77 -> 22.6 us (31 us
-// without the four-lane form below), against the table-driven step_f64_kernel,
-// which other six-group stencils still take.  Third order (Q = 100), 256^2:
-// 504 -> 240 us against step_o3_kernel.
+// Measured (M1, FP64): 256^2 272 -> 107 us a step against the table-driven
+// step_f64_kernel, which other six-group stencils still take; third order
+// (Q = 100) 504 -> 240 us against step_o3_kernel.  Lattices of few warps:
+// rlbm_lanes64.cu.
 // The populations are pulled twice (the second pull hits L1/L2) instead of
 // being held in 116 registers: 128 registers, eight blocks of 64 threads an SM
 // (65536 sites are 6.7 such blocks an SM; blocks of 128 left the SMs with four of
@@ -363,111 +363,6 @@ __device__ __forceinline__ void projections64(const SiteConsts& sc, const Macro<
   r[7] = yy;
   r[8] = fma(-2.0 * nm * o.Ux, o.Ux, yy);
   r[9] = nm * o.Ux * o.Uy;
-}
-
-// The members (+,+), (-,+), (+,-), (-,-) of the reflection orbits on four
-// neighbouring lanes: lane l holds the population with signs sx (bit 0 of l)
-// and sy (bit 1), so all lanes run the same code with the signs in data, each
-// population is pulled once and held, and the moments are summed over the four
-// lanes.  One warp of the kernel above runs 5400 instructions one after the
-// other, about 12 cycles each, and a lattice of few warps waits for exactly
-// that; here a warp runs a third of them on eight sites.
-//
-// Used up to kQuadSites sites an SM: an SM's one or two warps of the kernel
-// above take about 30 us whatever they hold, and the four-lane form, with two
-// and a half times the FP64 instructions a site, catches up with that there.
-constexpr long long kQuadSites = 48;
-struct Lane64 {
-  const double* fin;
-  double* out;
-  size_t plane;
-  unsigned pitch, here;
-  int x, y, Nx, Ny, l;
-  const int *dxm, *dym;
-};
-
-__device__ __forceinline__ double flip(double v, int negative) {
-  return __longlong_as_double(__double_as_longlong(v) ^ ((long long)negative << 63));
-}
-
-// Does lane l hold a member of orbit K (kind 2: l = 0, 1; 3: 0, 2; 1: 0)?
-template <class Def, int K>
-__device__ __forceinline__ bool lane_has(int l) {
-  constexpr int kind = Def::O.kind[K];
-  if constexpr (kind == 4) return true;
-  else if constexpr (kind == 2) return l < 2;
-  else if constexpr (kind == 3) return (l & 1) == 0;
-  else return l == 0;
-}
-
-template <class Def, int K>
-__device__ __forceinline__ size_t lane_plane(const Lane64& q) {
-  constexpr int kind = Def::O.kind[K];
-  constexpr int i0 = Def::O.idx[K][0], i1 = Def::O.idx[K][1], i2 = Def::O.idx[K][2], i3 = Def::O.idx[K][3];
-  unsigned i = i0;
-  if constexpr (kind == 4) i = (q.l & 2) ? ((q.l & 1) ? i3 : i2) : ((q.l & 1) ? i1 : i0);
-  else if constexpr (kind == 2) i = (q.l & 1) ? i1 : i0;
-  else if constexpr (kind == 3) i = (q.l & 2) ? i2 : i0;
-  return q.plane * i;
-}
-
-template <class Def, int K>
-__device__ __forceinline__ void lane_load(const Lane64& q, double (&d)[Def::O.K]) {
-  constexpr int ax = Def::O.ax[K], ay = Def::O.ay[K];
-  const unsigned xs = (unsigned)wrap_sub(q.x, (q.l & 1) ? q.dxm[kMaxDisp - ax] : q.dxm[kMaxDisp + ax], q.Nx);
-  const unsigned ys = (unsigned)wrap_sub(q.y, (q.l & 2) ? q.dym[kMaxDisp - ay] : q.dym[kMaxDisp + ay], q.Ny);
-  const double* src = q.fin + (ys * q.pitch + xs) + lane_plane<Def, K>(q);
-  d[K] = lane_has<Def, K>(q.l) ? __ldg(src) : 0.0;
-}
-
-template <class Def, int K>
-__device__ __forceinline__ void lane_acc(const double (&d)[Def::O.K], const double (*gmt)[5], double (&s)[6],
-                                         double (&M)[9]) {
-  constexpr int g = Def::O.grp[K], ax = Def::O.ax[K], ay = Def::O.ay[K];
-  if constexpr (orbit_starts_group<Def, K>()) {
-#pragma unroll
-    for (int k = 0; k < 6; ++k) s[k] = 0.0;
-  }
-  const double v = d[K];
-  s[0] += v;
-  if constexpr (ax != 0) s[1] = fma((double)ax, v, s[1]);
-  if constexpr (ay != 0) s[2] = fma((double)ay, v, s[2]);
-  if constexpr (ax != 0) s[3] = fma((double)(ax * ax), v, s[3]);
-  if constexpr (ax != 0 && ay != 0) s[4] = fma((double)(ax * ay), v, s[4]);
-  if constexpr (ay != 0) s[5] = fma((double)(ay * ay), v, s[5]);
-  if constexpr (orbit_ends_group<Def, K>()) {
-    const double* gm = gmt[g];
-    M[0] = fma(gm[0], s[0], M[0]);
-    M[3] = fma(gm[1], s[0], M[3]);
-    M[1] = fma(gm[2], s[1], M[1]);
-    M[2] = fma(gm[2], s[2], M[2]);
-    M[4] = fma(gm[3], s[1], M[4]);
-    M[5] = fma(gm[3], s[2], M[5]);
-    M[6] = fma(gm[4], s[3], M[6]);
-    M[7] = fma(gm[4], s[4], M[7]);
-    M[8] = fma(gm[4], s[5], M[8]);
-  }
-}
-
-template <class Def, int... Ks>
-__device__ __forceinline__ void lane_moments_all(std::integer_sequence<int, Ks...>, const Lane64& q,
-                                                 double (&d)[Def::O.K], const double (*gmt)[5], double (&M)[9]) {
-  (lane_load<Def, Ks>(q, d), ...);
-  double s[6];
-#pragma unroll
-  for (int k = 0; k < 9; ++k) M[k] = 0.0;
-  (lane_acc<Def, Ks>(d, gmt, s, M), ...);
-  // signs of the odd moments N^x, N^y, T^0x, T^0y, T^xy, then the lanes' sum
-  M[1] = flip(M[1], q.l & 1);
-  M[4] = flip(M[4], q.l & 1);
-  M[2] = flip(M[2], q.l >> 1);
-  M[5] = flip(M[5], q.l >> 1);
-  M[7] = flip(M[7], (q.l ^ (q.l >> 1)) & 1);
-#pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    M[k] += __shfl_xor_sync(0xffffffffu, M[k], 1);
-    M[k] += __shfl_xor_sync(0xffffffffu, M[k], 2);
-  }
 }
 
 }  // namespace rlbm

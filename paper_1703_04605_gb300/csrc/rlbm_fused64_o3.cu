@@ -48,73 +48,11 @@ __global__ void __launch_bounds__(64, 6) fused_f64_o3_kernel(const __grid_consta
   report(fl, p.err);
 }
 
-// Four lanes a site (rlbm_fused64.cuh): the signs of a lane go into the odd e_l.
-template <class Def, int K>
-__device__ __forceinline__ void lane_collide(const FusedO364Params& p, const Lane64& q, const double (&d)[Def::O.K],
-                                             const double (&e)[kO3Mono], double n, double a0, double wx, double wy) {
-  constexpr int kind = Def::O.kind[K], ax = Def::O.ax[K], ay = Def::O.ay[K];
-  const double* w = p.ow[K];
-  double f = sum64(O3EE{}, w, e, w[0] * n);
-  if constexpr (kind == 4) f = sum64(O3OO{}, w, e, f);
-  if constexpr (kind == 2 || kind == 4) f = sum64(O3OE{}, w, e, f);
-  if constexpr (kind == 3 || kind == 4) f = sum64(O3EO{}, w, e, f);
-  double om = a0;
-  if constexpr (ax != 0) om = fma(-(double)ax, wx, om);
-  if constexpr (ay != 0) om = fma(-(double)ay, wy, om);
-  if (lane_has<Def, K>(q.l)) __stcs(q.out + q.here + lane_plane<Def, K>(q), fma(om, f - d[K], d[K]));
-}
-
-template <class Def, int... Ks>
-__device__ __forceinline__ void lane_collide_all(std::integer_sequence<int, Ks...>, const FusedO364Params& p,
-                                                 const Lane64& q, const double (&d)[Def::O.K],
-                                                 const double (&e)[kO3Mono], double n, double a0, double wx,
-                                                 double wy) {
-  (lane_collide<Def, Ks>(p, q, d, e, n, a0, wx, wy), ...);
-}
-
-template <int... L>
-__device__ __forceinline__ void flip_all(std::integer_sequence<int, L...>, double (&e)[kO3Mono], int negative) {
-  ((e[L] = flip(e[L], negative)), ...);
-}
-
-template <class Def>
-__global__ void __launch_bounds__(32) fused_f64_o3_quad_kernel(const __grid_constant__ FusedO364Params p,
-                                                               const double* __restrict__ fin,
-                                                               double* __restrict__ fout) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nsite = p.Nx * p.Ny;
-  const bool live = (t >> 2) < nsite;
-  const int site = live ? t >> 2 : nsite - 1;
-  unsigned fl = 0;
-  int x, y;
-  site_of(site, p.Nx, x, y);
-  const Lane64 q{fin, fout, (size_t)p.plane, (unsigned)p.pitch, (unsigned)y * (unsigned)p.pitch + (unsigned)x, x, y,
-                 p.Nx, p.Ny, t & 3, p.dxm, p.dym};
-  using Orb = std::make_integer_sequence<int, Def::O.K>;
-  double d[Def::O.K], M[9];
-  lane_moments_all<Def>(Orb{}, q, d, p.gm, M);
-  const Macro<double> o = solve_site_f64_seeded(M, p.sc, p.rt64, p.rt32, fl);
-  double e[kO3Mono];
-  deviations64(p, o, e);
-  flip_all(O3OE{}, e, q.l & 1);
-  flip_all(O3EO{}, e, q.l >> 1);
-  flip_all(O3OO{}, e, (q.l ^ (q.l >> 1)) & 1);
-  const double wv = p.v0 * p.inv_tau;
-  if (live)
-    lane_collide_all<Def>(Orb{}, p, q, d, e, o.n, o.U0 * p.inv_tau, flip(wv * o.Ux, q.l & 1),
-                          flip(wv * o.Uy, q.l >> 1));
-  report(fl, p.err);
-}
-
 template <class Def>
 cudaError_t launch64(const FusedO364Params& p, const void* fin, void* fout, cudaStream_t s) {
   const long long nsite = (long long)p.Nx * p.Ny;
-  if (nsite <= kQuadSites * p.sms)
-    fused_f64_o3_quad_kernel<Def><<<(unsigned)((nsite + 7) / 8), 32, 0, s>>>(p, static_cast<const double*>(fin),
-                                                                             static_cast<double*>(fout));
-  else
-    fused_f64_o3_kernel<Def><<<(unsigned)((nsite + 63) / 64), 64, 0, s>>>(p, static_cast<const double*>(fin),
-                                                                          static_cast<double*>(fout));
+  fused_f64_o3_kernel<Def><<<(unsigned)((nsite + 63) / 64), 64, 0, s>>>(p, static_cast<const double*>(fin),
+                                                                        static_cast<double*>(fout));
   return cudaGetLastError();
 }
 

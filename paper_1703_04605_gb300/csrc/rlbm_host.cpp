@@ -51,6 +51,8 @@ struct rlbm_ctx {
   int kind64 = 0;                // compiled stencil (1..4, 5..10; 0: none) of the FP64 step and of the
                                  // FP64-arithmetic init and read-out, whatever the lattice's size
   std::unique_ptr<Io2Params> io2;
+  int lanes = 0;                 // small FP64 lattices: lanes a site (0: one thread a site)
+  std::unique_ptr<LanesParams> lp;
   // third-order stencils (eleven groups)
   int order = 2;
   std::unique_ptr<StencilBuildO3> sb3;
@@ -198,7 +200,6 @@ static void fill_fused64(rlbm_ctx* c) {
     for (int q = 0; q < 10; ++q) f.gf[g][q] = c->sb.gf[g][q];
   }
   fill_disp(c->Nx, c->Ny, f.dxm, f.dym);
-  f.sms = sm_count();
   f.rt64 = c->d_rt64;
   f.rt32 = c->d_rt32;
   f.err = c->d_err;
@@ -366,7 +367,6 @@ static void fill_fused_o364(rlbm_ctx* c) {
     for (int q = 0; q < 5; ++q) f.gm[g][q] = sb.gm[g][q];
   fill_orbits_o3(c->kind64, sb, f);
   fill_disp(c->Nx, c->Ny, f.dxm, f.dym);
-  f.sms = sm_count();
   f.rt64 = c->d_rt64;
   f.rt32 = c->d_rt32;
   f.err = c->d_err;
@@ -451,6 +451,34 @@ static rlbm_status check_device_error(rlbm_ctx* c) {
     return fail(c, RLBM_ENONPHYS, msg);
   }
   return RLBM_OK;
+}
+
+// Lanes a site of the FP64 step of a small lattice: the most that give no more
+// warps than the GPU has SM sub-partitions (four an SM), or 0.
+static int lanes64_for(long long nsite) {
+  for (int L = 32; L >= 4; L /= 2)
+    if (nsite * L <= 32LL * 4 * sm_count()) return L;
+  return 0;
+}
+
+static void fill_lanes(rlbm_ctx* c) {
+  c->lp.reset(new LanesParams);
+  LanesParams& f = *c->lp;
+  std::memset(&f, 0, sizeof f);
+  f.Nx = c->Nx;
+  f.Ny = c->Ny;
+  f.Q = c->Q;
+  f.third = c->order == 3;
+  f.pitch = c->pitch;
+  f.plane = c->plane;
+  f.inv_tau = 1.0 / c->tau;
+  f.c = f.third ? c->sb3->c : 0.0;
+  f.sc = f.third ? c->sb3->sc : c->sb.sc;
+  f.tab = c->d_tab64;
+  f.shift = c->d_shift;
+  f.rt64 = c->d_rt64;
+  f.rt32 = c->d_rt32;
+  f.err = c->d_err;
 }
 
 // The read-out parameters with the displacements that pull the state (or none).
@@ -581,6 +609,7 @@ static rlbm_status create_o3(const rlbm_stencil* st, double m, double tau, int N
     c->io3.reset(new IoO3Params);
     fill_fused_o364(c.get());
   }
+  if (dtype == RLBM_F64 && (c->lanes = lanes64_for((long long)Nx * Ny)) != 0) fill_lanes(c.get());
   *out = c.release();
   return RLBM_OK;
 }
@@ -689,6 +718,36 @@ rlbm_status rlbm_create(const rlbm_stencil* st, double m, double tau, int Nx, in
     c->io2.reset(new Io2Params);
     fill_fused64(c.get());
   }
+  if (dtype == RLBM_F64 && (c->lanes = lanes64_for((long long)Nx * Ny)) != 0) {
+    // table rows and displacements of the several-lanes kernel
+    const int Q = c->Q;
+    std::vector<double> tab((size_t)Q * kRowLanes2, 0.0);
+    std::vector<int> shift(2 * Q);
+    const PopTable<double>& pt = c->p64->pt;
+    for (int i = 0; i < Q; ++i) {
+      double* row = &tab[(size_t)i * kRowLanes2];
+      for (int k = 0; k < 9; ++k) row[k] = pt.mom[k][i];
+      for (int k = 0; k < NJ; ++k) row[10 + k] = pt.cj[k][i];
+      row[20] = pt.vx[i];
+      row[21] = pt.vy[i];
+      shift[i] = pt.dxm[i];
+      shift[Q + i] = pt.dym[i];
+    }
+    if (c->mem.get(&c->d_tab64, tab.size() * sizeof(double)) != cudaSuccess ||
+        c->mem.get(&c->d_shift, shift.size() * sizeof(int)) != cudaSuccess) {
+      release(c.get());
+      return fail(nullptr, RLBM_ENOMEM, "device allocation failed");
+    }
+    e = cudaMemcpy(c->d_tab64, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(c->d_shift, shift.data(), shift.size() * sizeof(int), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+    if (e != cudaSuccess) {
+      release(c.get());
+      return fail(nullptr, RLBM_ECUDA, std::string("upload: ") + cudaGetErrorString(e));
+    }
+    c->device_bytes += tab.size() * 8 + shift.size() * 4;
+    fill_lanes(c.get());
+  }
   if (dtype == RLBM_BF16_DEV) {
     if (!c->fused) {
       release(c.get());
@@ -795,7 +854,8 @@ rlbm_status rlbm_step(rlbm_ctx* c, int nsteps) {
     const void* fin = c->buf[c->cur];
     void* fout = c->buf[1 - c->cur];
     cudaError_t e;
-    if (c->order == 3)
+    if (c->lanes) e = launch_lanes64(*c->lp, c->lanes, fin, fout, c->stream);
+    else if (c->order == 3)
       e = c->fo3     ? launch_fused_o3(c->fused, *c->fo3, fin, fout, c->stream)
           : c->io3 && c->dtype == RLBM_F64 ? launch_fused_f64_o3(c->kind64, c->io3->b, fin, fout, c->stream)
                      : launch_step_o3(c->dtype, *c->o3, fin, fout, c->stream);

@@ -182,7 +182,6 @@ struct Fused64Params {
   SiteConsts sc;
   double gm[6][5], gf[6][10];
   int dxm[13], dym[13];
-  int sms;                    // SMs of the device (block size of small lattices)
   const double* rt64;
   const float* rt32;
   unsigned* err;
@@ -203,6 +202,23 @@ struct Io2Params {
 cudaError_t launch_init2(int kind, bool bf, const Io2Params& p, FieldPtrs f, void* cur, void* ccur, cudaStream_t s);
 cudaError_t launch_moments2(int kind, bool bf, const Io2Params& p, const void* prev, const void* cprev, MomentOut mo,
                             cudaStream_t s);
+
+// FP64 step of small lattices, several lanes a site (rlbm_lanes64.cu).  tab:
+// second order rows of kRowLanes2 (0..8 momentum products, 10..19 w_i J_k,
+// 20, 21 p^a/p^0), third order rows of kRowO3; shift: n_x, n_y modulo the lattice.
+constexpr int kRowLanes2 = 22;
+struct LanesParams {
+  int Nx, Ny, Q, third;
+  long long pitch, plane;
+  double inv_tau, c;
+  SiteConsts sc;
+  const double* tab;
+  const int* shift;           // [2][Q]
+  const double* rt64;
+  const float* rt32;
+  unsigned* err;
+};
+cudaError_t launch_lanes64(const LanesParams& p, int L, const void* fin, void* fout, cudaStream_t s);
 
 // One lattice of a persistent batch launch (device memory; rlbm_persist.cuh).
 struct PersistLattice {
@@ -308,7 +324,6 @@ struct FusedO364Params {
   double gm[11][5];
   double ow[kMaxOrbO3][21];
   int dxm[13], dym[13];
-  int sms;
   const double* rt64;
   const float* rt32;
   unsigned* err;

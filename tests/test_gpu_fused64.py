@@ -1,5 +1,6 @@
 """Compiled FP64 kernels against the FP64 oracle where they can go wrong:
-lattices smaller than a halo, one warp, block-size and tile edges, and states
+lattices smaller than a halo, one warp, block-size and tile edges (the limits of
+the several-lanes kernel are 608, 1216, 2432 and 4864 sites on 152 SMs), and states
 far from the reference (extreme densities, cold and hot gas), where the site
 solve leaves its FP32-seeded path.  Tolerance: the FP64 path's 1e-12."""
 import numpy as np
@@ -60,3 +61,13 @@ def test_nonphysical_state_is_reported():
         lat.step(2)
         with pytest.raises(RLBMError):
             lat.sync()
+
+
+# at most and just above 608, 1216, 2432 and 4864 sites
+@pytest.mark.parametrize("shape", [(19, 32), (87, 7), (64, 19), (1217, 1), (64, 38), (811, 3), (64, 76), (695, 7)])
+def test_lane_counts(shape):
+    st = W.STENCIL_S2
+    f = smooth_fields(shape[0], shape[1], seed=shape[0], du=0.2)
+    got, _ = run_gpu(st, 0.8, f, "f64", 2)
+    e = errors(got, run_oracle(st, 0.8, f, 2))
+    assert max(e.values()) < 1e-12, e

@@ -1,6 +1,6 @@
 """Compiled FP64 third-order kernels against the oracle at the edges of their
-forms: lattices smaller than a halo, both sides of the four-lane threshold
-(48 sites an SM: 7296 on 152 SMs), blocks with a tail.  Tolerance: the FP64
+forms: lattices smaller than a halo, small lattices on several lanes a site (up
+to 4864 sites on 152 SMs), blocks with a tail.  Tolerance: the FP64
 path's 1e-12."""
 import pytest
 
