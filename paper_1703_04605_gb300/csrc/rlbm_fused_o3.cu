@@ -90,6 +90,7 @@ __device__ __forceinline__ void o3_acc_orbit(const float (&d)[Def::Q], float (&s
 // the pulled values of the collision pass: kept in registers since the
 // moment pass, or pulled again (two-pass form; L1/L2 hits)
 struct O3Repull {
+  const float* keep;   // the thread's column of kept values
   const float* fin;
   long long plane, pitch;
   int x, y, Nx, Ny;
@@ -98,8 +99,40 @@ template <class Def, int I>
 __device__ __forceinline__ float o3_pop(const float (&d)[Def::Q]) {
   return d[I];
 }
+// Populations that stay in shared memory between the passes: o3_keep of those
+// with n_x and n_y nonzero (their addresses cost most), the others are pulled
+// again.  Slot of population i, -1: pulled again.
+template <class Def>
+__host__ __device__ constexpr int o3_keep() {
+  return Def::Q <= 104 ? 44 : 80;
+}
+template <class Def>
+__host__ __device__ constexpr int o3_slot(int i) {
+  auto cand = [](int j) { return Def::F.nx[j] != 0 && Def::F.ny[j] != 0; };
+  if (!cand(i)) return -1;
+  int n = 0;
+  for (int j = 0; j < i; ++j) n += cand(j) ? 1 : 0;
+  return n < o3_keep<Def>() ? n : -1;
+}
+template <class Def>
+__host__ __device__ constexpr int o3_slots() {
+  int n = 0;
+  for (int j = 0; j < Def::Q; ++j) n += o3_slot<Def>(j) >= 0 ? 1 : 0;
+  return n;
+}
+template <class Def, int... Is>
+__device__ __forceinline__ void o3_keep_all(std::integer_sequence<int, Is...>, const float (&d)[Def::Q], float* col) {
+  (
+      [&] {
+        constexpr int slot = o3_slot<Def>(Is);
+        if constexpr (slot >= 0) col[slot * 128] = d[Is];
+      }(),
+      ...);
+}
 template <class Def, int I>
 __device__ __forceinline__ float o3_pop(const O3Repull& r) {
+  constexpr int slot = o3_slot<Def>(I);
+  if constexpr (slot >= 0) return r.keep[slot * 128];
   constexpr int DX = Def::F.nx[I], DY = Def::F.ny[I];
   const unsigned idx = (unsigned)wrap_c<DY>(r.y, r.Ny) * (unsigned)r.pitch + (unsigned)wrap_c<DX>(r.x, r.Nx);
   return __ldg(r.fin + idx + (size_t)(unsigned)r.plane * I);
@@ -183,21 +216,23 @@ __device__ __forceinline__ void o3_collide_all(std::integer_sequence<int, Ks...>
   (o3_collide_orbit<Def, Ks, Pops>(d, e, nd, a0, ax, ay, out, plane, p), ...);
 }
 
-// Two passes over the populations: the moment pass pulls each value and
-// folds it into the group sums, the collision pass pulls it again (an L1/L2
-// hit: the block read the same lines moments earlier, 1 % extra DRAM reads)
-// instead of keeping Q values in registers across the site solve.  Resident
-// blocks of 128 threads per SM: four (128 registers, no spills) up to Q = 104,
-// three (168 registers, at most 16 bytes spilled) for the Q = 133-149 sets.
-// Measured on GB300 against one pass: 4 % faster at Q <= 104 (one pass at
-// four blocks spilled 70-90 bytes; at three blocks of 168 registers it was
-// 11 % slower), 8-21 % faster for the larger sets (one pass at two blocks
-// of 255 registers).  Results are the same bit for bit.
+// Two passes over the populations: the moment pass pulls each value and folds it
+// into the group sums; the collision pass takes some from shared memory (o3_keep)
+// and pulls the others again (an L1/L2 hit: the block read the same lines moments
+// earlier), so that few values live across the site solve.  Resident blocks of 128
+// threads per SM: five (96 registers) up to Q = 104, four (128) for the
+// Q = 133-149 sets.  Measured, 2048^2 us a step, kept values x blocks:
+//   Q = 100: 0 x 4 795; 28 x 5 758; 40 x 5 731; 56 x 5 748; 56 x 6 780; 56 x 4 886
+//   Q = 99:  0 x 4 803; 40 x 5 724; 48 x 5 717; 56 x 5 729
+//   Q = 133: 0 x 3 1238; 60 x 4 1045; 80 x 4 1048; 96 x 4 1057; 80 x 5 1270
+//   Q = 149: 0 x 3 1271; 60 x 4 1187; 80 x 4 1147; 96 x 4 1137; 80 x 5 1460
+// One pass (all values in registers, four blocks, 70-90 bytes spilled) was 4 %
+// slower than 0 x 4.  Results are the same bit for bit.
 constexpr bool O3_TWO_PASS = true;
 
 template <class Def>
 constexpr int o3_min_blocks() {
-  return Def::Q <= 104 ? 4 : 3;
+  return Def::Q <= 104 ? 5 : 4;
 }
 
 template <class Def>
@@ -206,6 +241,7 @@ __global__ void __launch_bounds__(128, o3_min_blocks<Def>()) fused_o3_kernel(con
   static_assert(Def::O.K <= kMaxOrbO3, "orbit constants exceed FusedO3Params::ow");
   const int site = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned fl = 0;
+  __shared__ float kept[o3_slots<Def>() * 128];
   if (site < p.Nx * p.Ny) {
     int x, y;
     site_of(site, p.Nx, x, y);
@@ -219,6 +255,7 @@ __global__ void __launch_bounds__(128, o3_min_blocks<Def>()) fused_o3_kernel(con
     if constexpr (two_pass) {
       float dd[Def::Q];
       o3_load_all<Def>(std::make_integer_sequence<int, Def::Q>{}, dd, fin, p.plane, p.pitch, x, y, p.Nx, p.Ny);
+      o3_keep_all<Def>(std::make_integer_sequence<int, Def::Q>{}, dd, kept + threadIdx.x);
       o3_acc_all<Def>(Orb{}, dd, s, M, p);
     } else {
       o3_load_all<Def>(std::make_integer_sequence<int, Def::Q>{}, d, fin, p.plane, p.pitch, x, y, p.Nx, p.Ny);
@@ -228,11 +265,12 @@ __global__ void __launch_bounds__(128, o3_min_blocks<Def>()) fused_o3_kernel(con
     // e_l = n dmu_l in the small quantities dU, dT, dR, U_x, U_y (no cancellation)
     float e[kO3Mono];
     o3_deviations<float>(p.mb, p.c, ss.n, ss.U0, ss.Ux, ss.Uy, ss.dg, ss.dR, ss.Td, ss.T, ss.R, e);
+    asm volatile("" : "+r"(x), "+r"(y) : : "memory");
     const float Ux = ss.Ux, Uy = ss.Uy;
     const float a0 = ss.U0 * p.inv_tau, ax = p.v0 * Ux * p.inv_tau, ay = p.v0 * Uy * p.inv_tau;
     float* out = fout + (long long)y * p.pitch + x;
     if constexpr (two_pass)
-      o3_collide_all<Def>(Orb{}, O3Repull{fin, p.plane, p.pitch, x, y, p.Nx, p.Ny}, e, ss.nd, a0, ax, ay, out,
+      o3_collide_all<Def>(Orb{}, O3Repull{kept + threadIdx.x, fin, p.plane, p.pitch, x, y, p.Nx, p.Ny}, e, ss.nd, a0, ax, ay, out,
                           p.plane, p);
     else o3_collide_all<Def>(Orb{}, d, e, ss.nd, a0, ax, ay, out, p.plane, p);
   }
