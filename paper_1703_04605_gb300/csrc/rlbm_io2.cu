@@ -45,54 +45,70 @@ __device__ __forceinline__ double pull64(const PullBF& q) {
   return (double)s + (double)e;
 }
 
-// Puts an equilibrium value as its deviation from the site's own reference.
+// Puts deviations from the site's own reference.
 struct PutBF {
   unsigned* out;   // the site's word of word plane 0
   size_t plane;
-  uint2 cq;        // coefficient word of the current group
   template <class Def, int I>
-  __device__ __forceinline__ float dev(double v) const {
-    constexpr int nx = Def::F.nx[I], ny = Def::F.ny[I], mult = Def::F.mult[I];
-    return (float)(v - (double)bf_ref<nx, ny, mult>(cq));
-  }
-  template <class Def, int I>
-  __device__ __forceinline__ void one(double v) const {
+  __device__ __forceinline__ void one(float v) const {
     constexpr int word = Def::B.word[I], half = Def::B.half[I];
     unsigned short* w = reinterpret_cast<unsigned short*>(out + plane * word);
-    __stcs(w + half, __bfloat16_as_ushort(__float2bfloat16_rn(dev<Def, I>(v))));
+    __stcs(w + half, __bfloat16_as_ushort(__float2bfloat16_rn(v)));
   }
   template <class Def, int I, int J>
-  __device__ __forceinline__ void pair(double a, double b) const {
+  __device__ __forceinline__ void pair(float a, float b) const {
     static_assert(Def::B.word[I] == Def::B.word[J] && Def::B.half[I] == 0, "orbit partners share a word");
     constexpr int word = Def::B.word[I];
-    __stcs(out + plane * word, bf_pack(dev<Def, I>(a), dev<Def, J>(b)));
+    __stcs(out + plane * word, bf_pack(a, b));
   }
 };
 
+// c: the group's equilibrium coefficients; BF16-deviation storage also e: their
+// deviations from the reference's (rounded) coefficients, formed in FP64, from
+// which the deviations of the populations follow without cancellation in FP32.
+struct GroupCoeffs {
+  double c[6];
+  float e[6];
+};
+
 template <class Def, int K, class Put>
-__device__ __forceinline__ void init_orbit(const Io2Params& p, const double (&r)[10], double (&c)[6], Put& put,
+__device__ __forceinline__ void init_orbit(const Io2Params& p, const double (&r)[10], GroupCoeffs& u, const Put& put,
                                            uint2* cout) {
   constexpr int g = Def::O.grp[K], ax = Def::O.ax[K], ay = Def::O.ay[K];
-  constexpr double m = (double)Def::O.mult[K];
+  constexpr bool BF = std::is_same<Put, PutBF>::value;
+  using T = typename std::conditional<BF, float, double>::type;
+  constexpr T m = (T)Def::O.mult[K];
   if constexpr (orbit_starts_group<Def, K>()) {
+    double(&c)[6] = u.c;
     group_coeffs64(p.b.gf[g], r, c);
-    if constexpr (std::is_same<Put, PutBF>::value) {
-      put.cq.x = bf_pack((float)c[0], (float)c[1]);
-      put.cq.y = bf_pack((float)c[2], (float)(0.5 * (c[3] + c[4])));
-      __stcs(cout + put.plane * g, put.cq);
+    if constexpr (BF) {
+      uint2 cq;
+      cq.x = bf_pack((float)c[0], (float)c[1]);
+      cq.y = bf_pack((float)c[2], (float)(0.5 * (c[3] + c[4])));
+      __stcs(cout + put.plane * g, cq);
+      const double q = (double)bf_hi(cq.y);
+      u.e[0] = (float)(c[0] - (double)bf_lo(cq.x));
+      u.e[1] = (float)(c[1] - (double)bf_hi(cq.x));
+      u.e[2] = (float)(c[2] - (double)bf_lo(cq.y));
+      u.e[3] = (float)(c[3] - q);
+      u.e[4] = (float)(c[4] - q);
+      u.e[5] = (float)c[5];
     }
   }
-  double E = m == 1.0 ? c[0] : m * c[0];
-  if constexpr (ax != 0) E = fma(m * (double)(ax * ax), c[3], E);
-  if constexpr (ay != 0) E = fma(m * (double)(ay * ay), c[4], E);
-  emit_orbit<Def, K>(put, E, (m * (double)ax) * c[1], (m * (double)ay) * c[2], (m * (double)(ax * ay)) * c[5]);
+  const T* c;
+  if constexpr (BF) c = u.e;
+  else c = u.c;
+  T E = m * c[0];
+  if constexpr (ax != 0) E += m * (T)(ax * ax) * c[3];
+  if constexpr (ay != 0) E += m * (T)(ay * ay) * c[4];
+  emit_orbit<Def, K, Put, T>(put, E, (m * (T)ax) * c[1], (m * (T)ay) * c[2], (m * (T)(ax * ay)) * c[5]);
 }
 
 template <class Def, class Put, int... Ks>
 __device__ __forceinline__ void init_all(std::integer_sequence<int, Ks...>, const Io2Params& p, const double (&r)[10],
-                                         Put& put, uint2* cout) {
-  double c[6];
-  (init_orbit<Def, Ks>(p, r, c, put, cout), ...);
+                                         const Put& put, uint2* cout) {
+  GroupCoeffs u;
+  (init_orbit<Def, Ks>(p, r, u, put, cout), ...);
 }
 
 template <class Def, bool BF>
@@ -109,10 +125,10 @@ __global__ void __launch_bounds__(128) init2_kernel(const __grid_constant__ Io2P
     const unsigned here = (unsigned)y * (unsigned)p.b.pitch + (unsigned)x;
     using Orb = std::make_integer_sequence<int, Def::O.K>;
     if constexpr (BF) {
-      PutBF put{static_cast<unsigned*>(cur) + here, (size_t)p.b.plane, make_uint2(0u, 0u)};
+      const PutBF put{static_cast<unsigned*>(cur) + here, (size_t)p.b.plane};
       init_all<Def>(Orb{}, p, r, put, ccur + here);
     } else {
-      PutPlain<double> put{static_cast<double*>(cur) + here, (size_t)p.b.plane};
+      const PutPlain<double> put{static_cast<double*>(cur) + here, (size_t)p.b.plane};
       init_all<Def>(Orb{}, p, r, put, nullptr);
     }
   }
