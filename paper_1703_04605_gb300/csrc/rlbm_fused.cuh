@@ -366,9 +366,9 @@ __device__ __forceinline__ void ex_acc_all(std::integer_sequence<int, Ks...>, co
 
 // Relaxation and store of population I with equilibrium value e (f^eq - r).
 template <class Def, bool BF, int I>
-__device__ __forceinline__ void fused_relax(const float (&d)[Def::Q], float e, const uint2 (&cq)[6], float a0,
+__device__ __forceinline__ void fused_relax(const float (&d)[Def::Q], float e, uint2 cq, float a0,
                                             float ax, float ay, void* __restrict__ out, long long plane) {
-  constexpr int g = Def::F.grp[I], nx = Def::F.nx[I], ny = Def::F.ny[I], mult = Def::F.mult[I];
+  constexpr int nx = Def::F.nx[I], ny = Def::F.ny[I], mult = Def::F.mult[I];
   // weight p_i.U/(p_i^0 tau) = (U0 - v0 (nx Ux + ny Uy))/tau
   float om = a0;
   if constexpr (nx != 0) om = fmaf(-(float)nx, ax, om);
@@ -379,7 +379,7 @@ __device__ __forceinline__ void fused_relax(const float (&d)[Def::Q], float e, c
   if constexpr (BF) {
     // a population without an orbit partner: its own half of its word
     constexpr int w = Def::B.word[I], hf = Def::B.half[I];
-    const float dv = vn - bf_ref<nx, ny, mult>(cq[g]);
+    const float dv = vn - bf_ref<nx, ny, mult>(cq);
     __stcs(static_cast<unsigned short*>(out) + 2 * pl * w + hf, __bfloat16_as_ushort(__float2bfloat16_rn(dv)));
   } else {
     __stcs(static_cast<float*>(out) + pl * I, vn);
@@ -390,10 +390,10 @@ __device__ __forceinline__ void fused_relax(const float (&d)[Def::Q], float e, c
 // half) and one conversion and store of the pair; R2: the arithmetic as
 // packed pairs (each lane the scalar operations)
 template <class Def, int I, int J, bool R2>
-__device__ __forceinline__ void bf_relax_pair(const float (&d)[Def::Q], float eI, float eJ, const uint2 (&cq)[6],
+__device__ __forceinline__ void bf_relax_pair(const float (&d)[Def::Q], float eI, float eJ, uint2 cq,
                                               float a0, float ax, float ay, void* __restrict__ out,
                                               long long plane) {
-  constexpr int g = Def::F.grp[I], nxI = Def::F.nx[I], nyI = Def::F.ny[I], nxJ = Def::F.nx[J],
+  constexpr int nxI = Def::F.nx[I], nyI = Def::F.ny[I], nxJ = Def::F.nx[J],
                 nyJ = Def::F.ny[J], mult = Def::F.mult[I];
   static_assert(Def::B.word[I] == Def::B.word[J] && Def::B.half[I] == 0 && Def::B.half[J] == 1,
                 "orbit partners share a word, the first in its low half");
@@ -402,7 +402,7 @@ __device__ __forceinline__ void bf_relax_pair(const float (&d)[Def::Q], float eI
   if constexpr (nyI != 0) omI = fmaf(-(float)nyI, ay, omI);
   if constexpr (nxJ != 0) omJ = fmaf(-(float)nxJ, ax, omJ);
   if constexpr (nyJ != 0) omJ = fmaf(-(float)nyJ, ay, omJ);
-  const float rI = bf_ref<nxI, nyI, mult>(cq[g]), rJ = bf_ref<nxJ, nyJ, mult>(cq[g]);
+  const float rI = bf_ref<nxI, nyI, mult>(cq), rJ = bf_ref<nxJ, nyJ, mult>(cq);
   float2 dv;
   if constexpr (R2) {
     const float2 v = make_float2(d[I], d[J]);
@@ -422,10 +422,10 @@ __device__ __forceinline__ void bf_relax_pair(const float (&d)[Def::Q], float eI
 // Relaxation of two members I, J of an orbit as packed pairs (each lane the
 // scalar fused_relax's operations)
 template <class Def, bool BF, int I, int J>
-__device__ __forceinline__ void fused_relax2(const float (&d)[Def::Q], float eI, float eJ, const uint2 (&cq)[6],
+__device__ __forceinline__ void fused_relax2(const float (&d)[Def::Q], float eI, float eJ, uint2 cq,
                                              float a0, float ax, float ay, void* __restrict__ out,
                                              long long plane) {
-  constexpr int g = Def::F.grp[I], nxI = Def::F.nx[I], nyI = Def::F.ny[I], nxJ = Def::F.nx[J],
+  constexpr int nxI = Def::F.nx[I], nyI = Def::F.ny[I], nxJ = Def::F.nx[J],
                 nyJ = Def::F.ny[J], mult = Def::F.mult[I];
   float omI = a0, omJ = a0;
   if constexpr (nxI != 0) omI = fmaf(-(float)nxI, ax, omI);
@@ -438,7 +438,6 @@ __device__ __forceinline__ void fused_relax2(const float (&d)[Def::Q], float eI,
   static_assert(!BF, "BF16 pairs go through bf_relax_pair");
   (void)cq;
   (void)mult;
-  (void)g;
   const size_t pl = (unsigned)plane;
   __stcs(static_cast<float*>(out) + pl * I, vn.x);
   __stcs(static_cast<float*>(out) + pl * J, vn.y);
@@ -448,31 +447,31 @@ __device__ __forceinline__ void fused_relax2(const float (&d)[Def::Q], float eI,
 // mult (c0 + c1 n_x + c2 n_y + c3 n_x^2 + c4 n_y^2 + c5 n_x n_y) split into the
 // part even in both n_x and n_y and the odd terms the members share.
 template <class Def, bool BF, int K, bool R2 = false>
-__device__ __forceinline__ void fused_collide_orbit(const float (&d)[Def::Q], const float (&c)[6][6],
-                                                    const uint2 (&cq)[6], float a0, float ax_, float ay_,
+__device__ __forceinline__ void fused_collide_orbit(const float (&d)[Def::Q], const float (&c)[6], uint2 cq,
+                                                    float a0, float ax_, float ay_,
                                                     void* __restrict__ out, long long plane) {
-  constexpr int kind = Def::O.kind[K], g = Def::O.grp[K], ax = Def::O.ax[K], ay = Def::O.ay[K];
+  constexpr int kind = Def::O.kind[K], ax = Def::O.ax[K], ay = Def::O.ay[K];
   constexpr int i0 = Def::O.idx[K][0], i1 = Def::O.idx[K][1], i2 = Def::O.idx[K][2], i3 = Def::O.idx[K][3];
   constexpr float m = (float)Def::O.mult[K];
-  float E0 = m * c[g][0];
-  if constexpr (ax != 0) E0 = fmaf(m * (float)(ax * ax), c[g][3], E0);
-  if constexpr (ay != 0) E0 = fmaf(m * (float)(ay * ay), c[g][4], E0);
+  float E0 = m * c[0];
+  if constexpr (ax != 0) E0 = fmaf(m * (float)(ax * ax), c[3], E0);
+  if constexpr (ay != 0) E0 = fmaf(m * (float)(ay * ay), c[4], E0);
   if constexpr (kind == 1) {
     fused_relax<Def, BF, i0>(d, E0, cq, a0, ax_, ay_, out, plane);
   } else if constexpr (BF && kind == 2) {
-    const float X = (m * (float)ax) * c[g][1];
+    const float X = (m * (float)ax) * c[1];
     bf_relax_pair<Def, i0, i1, R2>(d, E0 + X, E0 - X, cq, a0, ax_, ay_, out, plane);
   } else if constexpr (BF && kind == 3) {
-    const float Y = (m * (float)ay) * c[g][2];
+    const float Y = (m * (float)ay) * c[2];
     bf_relax_pair<Def, i0, i2, R2>(d, E0 + Y, E0 - Y, cq, a0, ax_, ay_, out, plane);
   } else if constexpr (BF) {
-    const float X = (m * (float)ax) * c[g][1], Y = (m * (float)ay) * c[g][2];
-    const float Z = (m * (float)(ax * ay)) * c[g][5];
+    const float X = (m * (float)ax) * c[1], Y = (m * (float)ay) * c[2];
+    const float Z = (m * (float)(ax * ay)) * c[5];
     const float EP = E0 + Z, EM = E0 - Z, XP = X + Y, XM = X - Y;
     bf_relax_pair<Def, i0, i3, R2>(d, EP + XP, EP - XP, cq, a0, ax_, ay_, out, plane);
     bf_relax_pair<Def, i1, i2, R2>(d, EM - XM, EM + XM, cq, a0, ax_, ay_, out, plane);
   } else if constexpr (kind == 2) {
-    const float X = (m * (float)ax) * c[g][1];
+    const float X = (m * (float)ax) * c[1];
     if constexpr (R2) {
       fused_relax2<Def, BF, i0, i1>(d, E0 + X, E0 - X, cq, a0, ax_, ay_, out, plane);
     } else {
@@ -480,7 +479,7 @@ __device__ __forceinline__ void fused_collide_orbit(const float (&d)[Def::Q], co
       fused_relax<Def, BF, i1>(d, E0 - X, cq, a0, ax_, ay_, out, plane);
     }
   } else if constexpr (kind == 3) {
-    const float Y = (m * (float)ay) * c[g][2];
+    const float Y = (m * (float)ay) * c[2];
     if constexpr (R2) {
       fused_relax2<Def, BF, i0, i2>(d, E0 + Y, E0 - Y, cq, a0, ax_, ay_, out, plane);
     } else {
@@ -488,8 +487,8 @@ __device__ __forceinline__ void fused_collide_orbit(const float (&d)[Def::Q], co
       fused_relax<Def, BF, i2>(d, E0 - Y, cq, a0, ax_, ay_, out, plane);
     }
   } else {
-    const float X = (m * (float)ax) * c[g][1], Y = (m * (float)ay) * c[g][2];
-    const float Z = (m * (float)(ax * ay)) * c[g][5];
+    const float X = (m * (float)ax) * c[1], Y = (m * (float)ay) * c[2];
+    const float Z = (m * (float)(ax * ay)) * c[5];
     const float EP = E0 + Z, EM = E0 - Z, XP = X + Y, XM = X - Y;
     if constexpr (R2) {
       fused_relax2<Def, BF, i0, i3>(d, EP + XP, EP - XP, cq, a0, ax_, ay_, out, plane);
@@ -524,11 +523,22 @@ __device__ __forceinline__ void fused_acc_all(std::integer_sequence<int, Ks...>,
   (fused_acc_orbit<Def, Ks>(d, s), ...);
 }
 
+template <class Def, int K>
+__host__ __device__ constexpr int orbit_group() {
+  return Def::O.grp[K];
+}
+template <class Def, int I>
+__host__ __device__ constexpr int pop_group() {
+  return Def::F.grp[I];
+}
+
 template <class Def, bool BF, bool R2, int... Ks>
 __device__ __forceinline__ void fused_collide_all(std::integer_sequence<int, Ks...>, const float (&d)[Def::Q],
                                                   const float (&c)[6][6], const uint2 (&cq)[6], float a0,
                                                   float ax, float ay, void* __restrict__ out, long long plane) {
-  (fused_collide_orbit<Def, BF, Ks, R2>(d, c, cq, a0, ax, ay, out, plane), ...);
+  (fused_collide_orbit<Def, BF, Ks, R2>(d, c[orbit_group<Def, Ks>()], cq[orbit_group<Def, Ks>()], a0, ax, ay, out,
+                                        plane),
+   ...);
 }
 
 // Per-population forms of the two loops (the stencil's reflection orbits are
@@ -547,16 +557,16 @@ __device__ __forceinline__ void fused_acc_pop(const float (&d)[Def::Q], float (&
 }
 
 template <class Def, bool BF, int I>
-__device__ __forceinline__ void fused_collide_pop(const float (&d)[Def::Q], const float (&c)[6][6],
-                                                  const uint2 (&cq)[6], float a0, float ax, float ay,
+__device__ __forceinline__ void fused_collide_pop(const float (&d)[Def::Q], const float (&c)[6], uint2 cq,
+                                                  float a0, float ax, float ay,
                                                   void* __restrict__ out, long long plane) {
-  constexpr int g = Def::F.grp[I], nx = Def::F.nx[I], ny = Def::F.ny[I], mult = Def::F.mult[I];
-  float e = c[g][0];
-  if constexpr (nx != 0) e = fmaf((float)nx, c[g][1], e);
-  if constexpr (ny != 0) e = fmaf((float)ny, c[g][2], e);
-  if constexpr (nx != 0) e = fmaf((float)(nx * nx), c[g][3], e);
-  if constexpr (ny != 0) e = fmaf((float)(ny * ny), c[g][4], e);
-  if constexpr (nx != 0 && ny != 0) e = fmaf((float)(nx * ny), c[g][5], e);
+  constexpr int nx = Def::F.nx[I], ny = Def::F.ny[I], mult = Def::F.mult[I];
+  float e = c[0];
+  if constexpr (nx != 0) e = fmaf((float)nx, c[1], e);
+  if constexpr (ny != 0) e = fmaf((float)ny, c[2], e);
+  if constexpr (nx != 0) e = fmaf((float)(nx * nx), c[3], e);
+  if constexpr (ny != 0) e = fmaf((float)(ny * ny), c[4], e);
+  if constexpr (nx != 0 && ny != 0) e = fmaf((float)(nx * ny), c[5], e);
   if constexpr (mult != 1) e *= (float)mult;
   fused_relax<Def, BF, I>(d, e, cq, a0, ax, ay, out, plane);
 }
@@ -573,6 +583,16 @@ struct FusedForms {
   static constexpr bool coeffs2 = BF ? true : EXL ? (Q == 39 || Q == 49) : (Q != 73);
   static constexpr bool relax2 = BF ? (Q == 39 || Q == 49) : EXL ? false : (Q == 39 || Q == 73);
   static constexpr bool magic_div = Q == 73 || (EXL && (Q == 39 || Q == 49));
+  // Extended sums: populations kept in shared memory, with the collision of
+  // late_collide_all; so the kernels fit six blocks (level 1 of the two small
+  // stencils) or five of 128 threads an SM.  Measured, 2048^2 us a step, without /
+  // with: level 1 G1-G6 275 / 249, S2 320 / 295, E5 469 / 461, M1 358 / 359;
+  // level 2 M1 412 / 390, G1-G6 298 / 285, S2 392 / 331, E5 not faster.  The plain
+  // FP32 and the BF16 kernels run 1-5 % slower that way: they are bound by
+  // bandwidth and by instruction issue, not by the warps in flight.
+  static constexpr int keep = EXL == 1 ? (Q == 49 ? 40 : Q == 39 ? 32 : Q == 73 ? 12 : Q == 58 ? 6 : 0)
+                            : EXL == 2 ? (Q == 49 ? 20 : Q == 39 ? 12 : Q == 58 ? 12 : 0)
+                                       : 0;
 };
 
 // Orbit form or per-population form, chosen per kernel from measurements on
@@ -594,7 +614,7 @@ template <class Def, bool BF, int... Is>
 __device__ __forceinline__ void fused_collide_pop_all(std::integer_sequence<int, Is...>, const float (&d)[Def::Q],
                                                       const float (&c)[6][6], const uint2 (&cq)[6], float a0,
                                                       float ax, float ay, void* __restrict__ out, long long plane) {
-  (fused_collide_pop<Def, BF, Is>(d, c, cq, a0, ax, ay, out, plane), ...);
+  (fused_collide_pop<Def, BF, Is>(d, c[pop_group<Def, Is>()], cq[pop_group<Def, Is>()], a0, ax, ay, out, plane), ...);
 }
 
 // dR(Td) from the R(zeta) table, for temperatures outside the lattice's dR
@@ -731,73 +751,169 @@ __device__ __forceinline__ SplitSite split_solve(const P& p, const float (&M)[9]
 // c2 n_y + c3 n_x^2 + c4 n_y^2 + c5 n_x n_y) of each group) from the split
 // site state: the App. B projections in deviation form, without their
 // normalisations (those and the App. A constants are folded into p.gf).
-template <bool C2 = false>
-__device__ __forceinline__ void fused_coeffs(const FusedParams& p, const SplitSite& ss, float (&c)[6][6]) {
+struct Proj {
+  float r0, r1, r2, r3, r4, r5, r6, r7, r8, r9, r78;
+};
+__device__ __forceinline__ Proj fused_projections(const FusedParams& p, const SplitSite& ss) {
   const float dg = ss.dg, Ux = ss.Ux, Uy = ss.Uy, n = ss.n, nd = ss.nd;
   const float Td = ss.Td, dR = ss.dR, R = ss.R, T = ss.T;
   const float mr32 = fmaf(p.mb, R, 4.0f * T);          // mbar K3/K2(zeta)
-  const float r0 = fmaf(p.nr.hi, dR, fmaf(p.nr.lo, dR, nd * R));   // n R - n_r R_r
-  const float r1 = n * (dg - p.k21 * dR);
-  const float r2 = n * Ux, r3 = n * Uy;
+  Proj w;
+  w.r0 = fmaf(p.nr.hi, dR, fmaf(p.nr.lo, dR, nd * R));   // n R - n_r R_r
+  w.r1 = n * (dg - p.k21 * dR);
+  w.r2 = n * Ux;
+  w.r3 = n * Uy;
   const float F = fmaf(p.mY, dR, 3.0f * Td);
   const float G = fmaf(p.mb, dR, 4.0f * Td);
-  const float r4 = n * (F + dg * fmaf(2.0f, mr32, p.cb00_1) + dg * dg * mr32);
+  w.r4 = n * (F + dg * fmaf(2.0f, mr32, p.cb00_1) + dg * dg * mr32);
   const float h = fmaf(mr32, dg, G);
-  const float r5 = n * h * Ux, r6 = n * h * Uy;
+  w.r5 = n * h * Ux;
+  w.r6 = n * h * Uy;
   const float nm = n * mr32;
-  const float r7 = nm * Uy * Uy, r8 = nm * (Uy * Uy - 2.0f * Ux * Ux), r9 = nm * Ux * Uy;
+  w.r7 = nm * Uy * Uy;
+  w.r8 = nm * (Uy * Uy - 2.0f * Ux * Ux);
+  w.r9 = nm * Ux * Uy;
+  w.r78 = w.r7 - w.r8;
+  return w;
+}
+
+// Coefficients of the groups 2j, 2j + 1 (C2: as packed pairs, each lane the
+// scalar form).
+template <bool C2>
+__device__ __forceinline__ void fused_coeffs_pair(const FusedParams& p, const Proj& w, int j, float (&c)[2][6]) {
   if constexpr (C2) {
-    // groups (2j, 2j + 1) as packed pairs; each lane is the scalar form below
-    const float r78 = r7 - r8;
-    const float2 R0 = make_float2(r0, r0), R1 = make_float2(r1, r1), R2 = make_float2(r2, r2);
-    const float2 R3 = make_float2(r3, r3), R4 = make_float2(r4, r4), R5 = make_float2(r5, r5);
-    const float2 R6 = make_float2(r6, r6), R7 = make_float2(r7, r7), R8 = make_float2(r8, r8);
-    const float2 R9 = make_float2(r9, r9), R78 = make_float2(r78, r78);
+    const float2 R0 = make_float2(w.r0, w.r0), R1 = make_float2(w.r1, w.r1), R2 = make_float2(w.r2, w.r2);
+    const float2 R3 = make_float2(w.r3, w.r3), R4 = make_float2(w.r4, w.r4), R5 = make_float2(w.r5, w.r5);
+    const float2 R6 = make_float2(w.r6, w.r6), R7 = make_float2(w.r7, w.r7), R8 = make_float2(w.r8, w.r8);
+    const float2 R9 = make_float2(w.r9, w.r9), R78 = make_float2(w.r78, w.r78);
+    const float2(*a)[2] = p.gf2[j];   // a[q][0]: hi pair, a[q][1]: lo pair
+    float2 al = __ffma2_rn(a[0][0], R0, __fmul2_rn(a[0][1], R0));
+    al = __ffma2_rn(a[1][0], R1, __ffma2_rn(a[1][1], R1, al));
+    al = __ffma2_rn(a[2][0], R4, __ffma2_rn(a[2][1], R4, al));
+    al = __ffma2_rn(a[3][0], R7, __ffma2_rn(a[3][1], R7, al));
+    al = __ffma2_rn(a[4][0], R8, __ffma2_rn(a[4][1], R8, al));
+    const float2 h5 = __ffma2_rn(a[6][0], R5, __fmul2_rn(a[6][1], R5));
+    const float2 h6 = __ffma2_rn(a[6][0], R6, __fmul2_rn(a[6][1], R6));
+    const float2 b1 = __ffma2_rn(a[5][0], R2, __ffma2_rn(a[5][1], R2, h5));
+    const float2 b2 = __ffma2_rn(a[5][0], R3, __ffma2_rn(a[5][1], R3, h6));
+    const float2 q3 = __ffma2_rn(a[7][0], R78, __fmul2_rn(a[7][1], R78));
+    const float2 q4 = __ffma2_rn(a[8][0], R7, __fmul2_rn(a[8][1], R7));
+    const float2 q5 = __ffma2_rn(a[9][0], R9, __fmul2_rn(a[9][1], R9));
+    const float2 cc[6] = {al, b1, b2, q3, q4, q5};
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const float2(*a)[2] = p.gf2[j];   // a[q][0]: hi pair, a[q][1]: lo pair
-      float2 al = __ffma2_rn(a[0][0], R0, __fmul2_rn(a[0][1], R0));
-      al = __ffma2_rn(a[1][0], R1, __ffma2_rn(a[1][1], R1, al));
-      al = __ffma2_rn(a[2][0], R4, __ffma2_rn(a[2][1], R4, al));
-      al = __ffma2_rn(a[3][0], R7, __ffma2_rn(a[3][1], R7, al));
-      al = __ffma2_rn(a[4][0], R8, __ffma2_rn(a[4][1], R8, al));
-      const float2 h5 = __ffma2_rn(a[6][0], R5, __fmul2_rn(a[6][1], R5));
-      const float2 h6 = __ffma2_rn(a[6][0], R6, __fmul2_rn(a[6][1], R6));
-      const float2 b1 = __ffma2_rn(a[5][0], R2, __ffma2_rn(a[5][1], R2, h5));
-      const float2 b2 = __ffma2_rn(a[5][0], R3, __ffma2_rn(a[5][1], R3, h6));
-      const float2 q3 = __ffma2_rn(a[7][0], R78, __fmul2_rn(a[7][1], R78));
-      const float2 q4 = __ffma2_rn(a[8][0], R7, __fmul2_rn(a[8][1], R7));
-      const float2 q5 = __ffma2_rn(a[9][0], R9, __fmul2_rn(a[9][1], R9));
-      const float2 cc[6] = {al, b1, b2, q3, q4, q5};
-#pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        c[2 * j][k] = cc[k].x;
-        c[2 * j + 1][k] = cc[k].y;
-      }
+    for (int k = 0; k < 6; ++k) {
+      c[0][k] = cc[k].x;
+      c[1][k] = cc[k].y;
     }
   } else {
 #pragma unroll
-    for (int g = 0; g < 6; ++g) {
-      const HL* a = p.gf[g];
-      float al = hl(a[0], r0);
-      al = hl_fma(a[1], r1, al);
-      al = hl_fma(a[2], r4, al);
-      al = hl_fma(a[3], r7, al);
-      al = hl_fma(a[4], r8, al);
-      c[g][0] = al;
-      c[g][1] = hl_fma(a[5], r2, hl(a[6], r5));
-      c[g][2] = hl_fma(a[5], r3, hl(a[6], r6));
-      c[g][3] = hl(a[7], r7 - r8);
-      c[g][4] = hl(a[8], r7);
-      c[g][5] = hl(a[9], r9);
+    for (int i = 0; i < 2; ++i) {
+      const HL* a = p.gf[2 * j + i];
+      float al = hl(a[0], w.r0);
+      al = hl_fma(a[1], w.r1, al);
+      al = hl_fma(a[2], w.r4, al);
+      al = hl_fma(a[3], w.r7, al);
+      al = hl_fma(a[4], w.r8, al);
+      c[i][0] = al;
+      c[i][1] = hl_fma(a[5], w.r2, hl(a[6], w.r5));
+      c[i][2] = hl_fma(a[5], w.r3, hl(a[6], w.r6));
+      c[i][3] = hl(a[7], w.r78);
+      c[i][4] = hl(a[8], w.r7);
+      c[i][5] = hl(a[9], w.r9);
     }
   }
+}
+
+// All six groups.
+template <bool C2 = false>
+__device__ __forceinline__ void fused_coeffs(const FusedParams& p, const SplitSite& ss, float (&c)[6][6]) {
+  const Proj w = fused_projections(p, ss);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    float t[2][6];
+    fused_coeffs_pair<C2>(p, w, j, t);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      c[2 * j][k] = t[0][k];
+      c[2 * j + 1][k] = t[1][k];
+    }
+  }
+}
+
+// Populations that wait for the collision in shared memory instead of in
+// registers: those of the last reflection orbits, which the collision takes up
+// last, FusedForms::keep of them or the next whole orbit.
+template <class Def, int KEEP>
+__host__ __device__ constexpr int keep_from_orbit() {
+  int n = 0, k = Def::O.K;
+  while (k > 0 && n < KEEP) {
+    --k;
+    n += Def::O.kind[k] == 4 ? 4 : Def::O.kind[k] == 1 ? 1 : 2;
+  }
+  return k;
+}
+template <class Def, int KEEP>
+__host__ __device__ constexpr int keep_slots() {
+  int n = 0;
+  for (int k = keep_from_orbit<Def, KEEP>(); k < Def::O.K; ++k)
+    n += Def::O.kind[k] == 4 ? 4 : Def::O.kind[k] == 1 ? 1 : 2;
+  return n;
+}
+// first slot of orbit K
+template <class Def, int KEEP>
+__host__ __device__ constexpr int keep_slot_of(int K) {
+  int n = 0;
+  for (int k = keep_from_orbit<Def, KEEP>(); k < K; ++k) n += Def::O.kind[k] == 4 ? 4 : Def::O.kind[k] == 1 ? 1 : 2;
+  return n;
+}
+// Orbit K's values to (PUT) or from their slots, a column of kKeepTB threads;
+// volatile, or the compiler would hand them over in registers.
+constexpr int kKeepTB = 128;
+template <class Def, int KEEP, int K, bool PUT>
+__device__ __forceinline__ void keep_orbit(float (&d)[Def::Q], volatile float* col) {
+  if constexpr (K >= keep_from_orbit<Def, KEEP>()) {
+    constexpr int kind = Def::O.kind[K], s0 = keep_slot_of<Def, KEEP>(K);
+    constexpr int i0 = Def::O.idx[K][0], i1 = Def::O.idx[K][1], i2 = Def::O.idx[K][2], i3 = Def::O.idx[K][3];
+    constexpr int n = kind == 4 ? 4 : kind == 1 ? 1 : 2;
+    constexpr int id[4] = {i0, kind == 3 ? i2 : i1, i2, i3};
+#pragma unroll
+    for (int j = 0; j < n; ++j) {
+      if constexpr (PUT) col[(s0 + j) * kKeepTB] = d[id[j]];
+      else d[id[j]] = col[(s0 + j) * kKeepTB];
+    }
+  }
+}
+template <class Def, int KEEP, int... Ks>
+__device__ __forceinline__ void keep_put_all(std::integer_sequence<int, Ks...>, float (&d)[Def::Q],
+                                             volatile float* col) {
+  (keep_orbit<Def, KEEP, Ks, true>(d, col), ...);
+}
+
+// Collision that takes the coefficients two groups at a time, so that 12 of them
+// live instead of 36, and the kept populations from their slots.
+template <class Def, int EXL, int K>
+__device__ __forceinline__ void late_collide_step(float (&d)[Def::Q], const FusedParams& p, const Proj& w,
+                                                  float (&c)[2][6], float a0, float ax, float ay, void* out,
+                                                  volatile float* col) {
+  using Forms = FusedForms<Def, false, EXL>;
+  constexpr int g = Def::O.grp[K];
+  keep_orbit<Def, Forms::keep, K, false>(d, col);
+  if constexpr (K == 0 || Def::O.grp[K > 0 ? K - 1 : 0] / 2 != g / 2) fused_coeffs_pair<Forms::coeffs2>(p, w, g / 2, c);
+  fused_collide_orbit<Def, false, K, Forms::relax2>(d, c[g & 1], make_uint2(0u, 0u), a0, ax, ay, out, p.plane);
+}
+template <class Def, int EXL, int... Ks>
+__device__ __forceinline__ void late_collide_all(std::integer_sequence<int, Ks...>, float (&d)[Def::Q],
+                                                 const FusedParams& p, const Proj& w, float a0, float ax, float ay,
+                                                 void* out, volatile float* col) {
+  float c[2][6];
+  (late_collide_step<Def, EXL, Ks>(d, p, w, c, a0, ax, ay, out, col), ...);
 }
 
 // One site update (see the header comment); p describes the lattice.
 template <class Def, bool BF, int EXL = 0, int LD = LD_RO>
 __device__ __forceinline__ void fused_site(const FusedParams& p, const void* __restrict__ fin,
-                                           void* __restrict__ fout, int site, unsigned& fl) {
+                                           void* __restrict__ fout, int site, unsigned& fl,
+                                           volatile float* col = nullptr) {
   static_assert(!(BF && EXL), "extended moment sums are for FP32 storage");
   constexpr int Q = Def::Q;
   using Seq = std::make_integer_sequence<int, Q>;
@@ -825,6 +941,7 @@ __device__ __forceinline__ void fused_site(const FusedParams& p, const void* __r
                                   p.Ny);
     }
     using Orb = std::make_integer_sequence<int, Def::O.K>;
+    constexpr int KEEP = FusedForms<Def, BF, EXL>::keep;
     // deviation moments N0 Nx Ny T00 T0x T0y Txx Txy Tyy (reference excluded)
     float M[9];
     SplitSite ss;
@@ -842,6 +959,7 @@ __device__ __forceinline__ void fused_site(const FusedParams& p, const void* __r
       M[6] = em.Txx;
       M[7] = em.Txy;
       M[8] = em.Tyy;
+      if constexpr (KEEP > 0) keep_put_all<Def, KEEP>(Orb{}, d, col);
       ss = split_solve<true>(p, M, fl, &em);
     } else {
       float s[6][6];
@@ -876,9 +994,14 @@ __device__ __forceinline__ void fused_site(const FusedParams& p, const void* __r
       ss = split_solve(p, M, fl);
     }
     const float U0 = ss.U0, Ux = ss.Ux, Uy = ss.Uy;
+    const float a0 = U0 * p.inv_tau, ax = p.v0 * Ux * p.inv_tau, ay = p.v0 * Uy * p.inv_tau;
+    if constexpr (KEEP > 0) {
+      late_collide_all<Def, EXL>(Orb{}, d, p, fused_projections(p, ss), a0, ax, ay, static_cast<float*>(fout) + here,
+                                 col);
+      return;
+    }
     float c[6][6];
     fused_coeffs<FusedForms<Def, BF, EXL>::coeffs2>(p, ss, c);
-    const float a0 = U0 * p.inv_tau, ax = p.v0 * Ux * p.inv_tau, ay = p.v0 * Uy * p.inv_tau;
     uint2 cq[6];
     if constexpr (BF) {
       // this site's reference coefficients, rounded once and stored for the readers
@@ -905,6 +1028,7 @@ __device__ __forceinline__ void fused_site(const FusedParams& p, const void* __r
 // registers), where fewer registers would spill.
 template <class Def, bool BF, int EXL = 0>
 constexpr int fused_min_blocks() {
+  if (FusedForms<Def, BF, EXL>::keep > 0) return EXL == 1 && Def::Q < 50 ? 6 : 5;
   return Def::Q <= 40 ? ((BF || EXL) ? 5 : 6) : ((Def::Q <= 64 && !BF && EXL < 2) ? 5 : 4);
 }
 
@@ -915,8 +1039,11 @@ __global__ void __launch_bounds__(128, fused_min_blocks<Def, BF, EXL>()) fused_f
                                                         void* __restrict__ fout) {
   const int site = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned fl = 0;
+  constexpr int KEEP = FusedForms<Def, BF, EXL>::keep;
+  __shared__ float kept[KEEP > 0 ? keep_slots<Def, KEEP>() * kKeepTB : 1];
   if constexpr (CHAIN) pdl_wait();
-  if (site < p.Nx * p.Ny) fused_site<Def, BF, EXL, CHAIN ? LD_CHAIN : LD_RO>(p, fin, fout, site, fl);
+  if (site < p.Nx * p.Ny)
+    fused_site<Def, BF, EXL, CHAIN ? LD_CHAIN : LD_RO>(p, fin, fout, site, fl, kept + (KEEP > 0 ? threadIdx.x : 0));
   report(fl, p.err);
 }
 

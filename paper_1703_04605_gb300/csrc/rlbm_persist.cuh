@@ -45,6 +45,8 @@ template <class Def, bool BF, int EXL>
 __global__ void __launch_bounds__(128, fused_min_blocks<Def, BF, EXL>())
     persist_kernel(const __grid_constant__ PersistParams pp) {
   __shared__ FusedParams sp;
+  constexpr int KEEP = FusedForms<Def, BF, EXL>::keep;
+  __shared__ float kept[KEEP > 0 ? keep_slots<Def, KEEP>() * kKeepTB : 1];
   __shared__ int s_lat, s_tile, s_step, s_go;
   const unsigned total = (unsigned)pp.units_per_step * (unsigned)pp.nsteps;
   for (;;) {
@@ -93,7 +95,7 @@ __global__ void __launch_bounds__(128, fused_min_blocks<Def, BF, EXL>())
     unsigned fl = 0;
     for (int j = 0; j < pp.spt; ++j) {
       const int site = (tile * pp.spt + j) * 128 + (int)threadIdx.x;
-      if (site < L.nsite) fused_site<Def, BF, EXL, LD_CG>(sp, fin, fout, site, fl);
+      if (site < L.nsite) fused_site<Def, BF, EXL, LD_CG>(sp, fin, fout, site, fl, kept + (KEEP > 0 ? threadIdx.x : 0));
     }
     report(fl, sp.err);
     __syncthreads();   // every store of the unit is issued
