@@ -60,8 +60,8 @@ __device__ __forceinline__ void write_planes64(const MomentOut& mo, long long N,
 }
 
 // Values of the members of orbit K to put (pairs: the partners of a BF16 word).
-template <class Def, int K, class Put, typename T>
-__device__ __forceinline__ void emit_orbit(const Put& put, T E, T X, T Y, T Z) {
+template <class Def, int K, class Put>
+__device__ __forceinline__ void emit_orbit(const Put& put, double E, double X, double Y, double Z) {
   constexpr int kind = Def::O.kind[K];
   constexpr int i0 = Def::O.idx[K][0], i1 = Def::O.idx[K][1], i2 = Def::O.idx[K][2], i3 = Def::O.idx[K][3];
   if constexpr (kind == 1) {
@@ -71,7 +71,7 @@ __device__ __forceinline__ void emit_orbit(const Put& put, T E, T X, T Y, T Z) {
   } else if constexpr (kind == 3) {
     put.template pair<Def, i0, i2>(E + Y, E - Y);
   } else {
-    const T EP = E + Z, EM = E - Z, XP = X + Y, XM = X - Y;
+    const double EP = E + Z, EM = E - Z, XP = X + Y, XM = X - Y;
     put.template pair<Def, i0, i3>(EP + XP, EP - XP);
     put.template pair<Def, i1, i2>(EM - XM, EM + XM);
   }

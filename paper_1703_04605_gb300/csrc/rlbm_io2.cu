@@ -45,70 +45,70 @@ __device__ __forceinline__ double pull64(const PullBF& q) {
   return (double)s + (double)e;
 }
 
+// The bfloat16 nearest to a double, in integer arithmetic: the FP64 pipe, which
+// bounds the init, has no part in it.  The double is cut to an FP32 bit pattern
+// whose last bit stands for anything cut off (round to odd), so that the second
+// rounding is the only one.  Outside FP32's normal range the conversion decides.
+__device__ __forceinline__ unsigned short bf16_nearest(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const unsigned e = ((hi >> 20) & 0x7ffu) - 896u;   // FP32 exponent field
+  if (e - 1u >= 253u) return __bfloat16_as_ushort(__double2bfloat16(v));
+  const unsigned f = (hi & 0x80000000u) | (e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29) | ((lo & 0x1fffffffu) != 0u);
+  return __bfloat16_as_ushort(__float2bfloat16_rn(__uint_as_float(f)));
+}
+
 // Puts deviations from the site's own reference.
 struct PutBF {
   unsigned* out;   // the site's word of word plane 0
   size_t plane;
   template <class Def, int I>
-  __device__ __forceinline__ void one(float v) const {
+  __device__ __forceinline__ void one(double v) const {
     constexpr int word = Def::B.word[I], half = Def::B.half[I];
     unsigned short* w = reinterpret_cast<unsigned short*>(out + plane * word);
-    __stcs(w + half, __bfloat16_as_ushort(__float2bfloat16_rn(v)));
+    __stcs(w + half, bf16_nearest(v));
   }
   template <class Def, int I, int J>
-  __device__ __forceinline__ void pair(float a, float b) const {
+  __device__ __forceinline__ void pair(double a, double b) const {
     static_assert(Def::B.word[I] == Def::B.word[J] && Def::B.half[I] == 0, "orbit partners share a word");
     constexpr int word = Def::B.word[I];
-    __stcs(out + plane * word, bf_pack(a, b));
+    __stcs(out + plane * word, (unsigned)bf16_nearest(a) | ((unsigned)bf16_nearest(b) << 16));
   }
 };
 
-// c: the group's equilibrium coefficients; BF16-deviation storage also e: their
-// deviations from the reference's (rounded) coefficients, formed in FP64, from
-// which the deviations of the populations follow without cancellation in FP32.
-struct GroupCoeffs {
-  double c[6];
-  float e[6];
-};
-
+// c: the group's equilibrium coefficients, for BF16-deviation storage less those
+// of the reference (rounded to bfloat16), so that the orbits' values are the
+// deviations themselves.
 template <class Def, int K, class Put>
-__device__ __forceinline__ void init_orbit(const Io2Params& p, const double (&r)[10], GroupCoeffs& u, const Put& put,
+__device__ __forceinline__ void init_orbit(const Io2Params& p, const double (&r)[10], double (&c)[6], const Put& put,
                                            uint2* cout) {
   constexpr int g = Def::O.grp[K], ax = Def::O.ax[K], ay = Def::O.ay[K];
-  constexpr bool BF = std::is_same<Put, PutBF>::value;
-  using T = typename std::conditional<BF, float, double>::type;
-  constexpr T m = (T)Def::O.mult[K];
+  constexpr double m = (double)Def::O.mult[K];
   if constexpr (orbit_starts_group<Def, K>()) {
-    double(&c)[6] = u.c;
     group_coeffs64(p.b.gf[g], r, c);
-    if constexpr (BF) {
+    if constexpr (std::is_same<Put, PutBF>::value) {
       uint2 cq;
       cq.x = bf_pack((float)c[0], (float)c[1]);
       cq.y = bf_pack((float)c[2], (float)(0.5 * (c[3] + c[4])));
       __stcs(cout + put.plane * g, cq);
       const double q = (double)bf_hi(cq.y);
-      u.e[0] = (float)(c[0] - (double)bf_lo(cq.x));
-      u.e[1] = (float)(c[1] - (double)bf_hi(cq.x));
-      u.e[2] = (float)(c[2] - (double)bf_lo(cq.y));
-      u.e[3] = (float)(c[3] - q);
-      u.e[4] = (float)(c[4] - q);
-      u.e[5] = (float)c[5];
+      c[0] -= (double)bf_lo(cq.x);
+      c[1] -= (double)bf_hi(cq.x);
+      c[2] -= (double)bf_lo(cq.y);
+      c[3] -= q;
+      c[4] -= q;
     }
   }
-  const T* c;
-  if constexpr (BF) c = u.e;
-  else c = u.c;
-  T E = m * c[0];
-  if constexpr (ax != 0) E += m * (T)(ax * ax) * c[3];
-  if constexpr (ay != 0) E += m * (T)(ay * ay) * c[4];
-  emit_orbit<Def, K, Put, T>(put, E, (m * (T)ax) * c[1], (m * (T)ay) * c[2], (m * (T)(ax * ay)) * c[5]);
+  double E = m == 1.0 ? c[0] : m * c[0];
+  if constexpr (ax != 0) E = fma(m * (double)(ax * ax), c[3], E);
+  if constexpr (ay != 0) E = fma(m * (double)(ay * ay), c[4], E);
+  emit_orbit<Def, K>(put, E, (m * (double)ax) * c[1], (m * (double)ay) * c[2], (m * (double)(ax * ay)) * c[5]);
 }
 
 template <class Def, class Put, int... Ks>
 __device__ __forceinline__ void init_all(std::integer_sequence<int, Ks...>, const Io2Params& p, const double (&r)[10],
                                          const Put& put, uint2* cout) {
-  GroupCoeffs u;
-  (init_orbit<Def, Ks>(p, r, u, put, cout), ...);
+  double c[6];
+  (init_orbit<Def, Ks>(p, r, c, put, cout), ...);
 }
 
 template <class Def, bool BF>
