@@ -18,7 +18,7 @@
 //
 // Measured (M1, FP64): 256^2 272 -> 107 us a step against the table-driven
 // step_f64_kernel, which other six-group stencils still take; third order
-// (Q = 100) 504 -> 240 us against step_o3_kernel.  Lattices of few warps:
+// (Q = 100) 504 -> 228 us against step_o3_kernel.  Lattices of few warps:
 // rlbm_lanes64.cu.
 // The populations are pulled twice (the second pull hits L1/L2) instead of
 // being held in 116 registers: 128 registers, eight blocks of 64 threads an SM

@@ -8,20 +8,14 @@
 namespace rlbm {
 namespace {
 
-template <class Def, int K>
-__device__ __forceinline__ void collide64_orbit(const FusedO364Params& p, const double (&e)[kO3Mono], double n,
-                                                const Pull64& q, const Relax64& rx) {
-  double E, X, Y, Z;
-  orbit_equilibrium_o3<Def, K>(p.ow[K], e, n, E, X, Y, Z);
-  relax64_orbit<Def, K>(q, rx, E, X, Y, Z);
-}
-
-template <class Def, int... Ks>
-__device__ __forceinline__ void collide64_all(std::integer_sequence<int, Ks...>, const FusedO364Params& p,
-                                              const double (&e)[kO3Mono], double n, const Pull64& q,
-                                              const Relax64& rx) {
-  (collide64_orbit<Def, Ks>(p, e, n, q, rx), ...);
-}
+struct RelaxUse {
+  const Pull64& q;
+  const Relax64& rx;
+  template <class Def, int K>
+  __device__ __forceinline__ void at(double E, double X, double Y, double Z) const {
+    relax64_orbit<Def, K>(q, rx, E, X, Y, Z);
+  }
+};
 
 template <class Def>
 __global__ void __launch_bounds__(64, 6) fused_f64_o3_kernel(const __grid_constant__ FusedO364Params p,
@@ -43,7 +37,7 @@ __global__ void __launch_bounds__(64, 6) fused_f64_o3_kernel(const __grid_consta
     const double wv = p.v0 * p.inv_tau;
     const Relax64 rx{o.U0 * p.inv_tau, wv * o.Ux, wv * o.Uy, fout + ((unsigned)y * (unsigned)p.pitch + (unsigned)x),
                      (size_t)p.plane};
-    collide64_all<Def>(Orb{}, p, e, o.n, q, rx);
+    all_orbits_o3<Def>(Orb{}, p, e, o.n, RelaxUse{q, rx});
   }
   report(fl, p.err);
 }

@@ -29,12 +29,6 @@
 namespace rlbm {
 namespace {
 
-// Parity classes of the centred monomials (kO3Mono order; rlbm_internal.h).
-using kEE = std::integer_sequence<int, 0, 1, 6, 7, 9, 10, 11, 17>;   // even in p_x and p_y
-using kOE = std::integer_sequence<int, 2, 4, 13, 15, 18>;            // odd in p_x only
-using kEO = std::integer_sequence<int, 3, 5, 14, 16, 19>;            // odd in p_y only
-using kOO = std::integer_sequence<int, 8, 12>;                       // odd in both
-
 template <class Def, int K>
 __host__ __device__ constexpr bool last_of_group() {
   return K + 1 == Def::O.K || Def::O.grp[K + 1] != Def::O.grp[K];
@@ -151,41 +145,61 @@ __device__ __forceinline__ void o3_relax(const Pops& d, float e, float a0, float
   __stcs(out + (size_t)(unsigned)plane * I, fmaf(om, e - v, v));   // plane < 2^32 elements
 }
 
-template <int... L>
-__device__ __forceinline__ float class_sum(std::integer_sequence<int, L...>, const HL* w, const float (&e)[kO3Mono],
+// acc + sum of w[1 + W_k] e[E_k]
+template <int... W, int... E>
+__device__ __forceinline__ float class_sum(MonoList<W...>, MonoList<E...>, const HL* w, const float (&e)[kO3Mono],
                                            float acc) {
-  ((acc = hl_fma(w[1 + L], e[L], acc)), ...);
+  ((acc = hl_fma(w[1 + W], e[E], acc)), ...);
   return acc;
 }
 
-// Equilibrium and relaxation of the members of reflection orbit K.
+// Relaxation of the members of reflection orbit K with equilibrium parts E (even
+// in n_x and n_y), X, Y (odd in one) and Z (odd in both).
 template <class Def, int K, class Pops>
-__device__ __forceinline__ void o3_collide_orbit(const Pops& d, const float (&e)[kO3Mono], float nd,
-                                                 float a0, float ax, float ay, float* __restrict__ out,
-                                                 long long plane, const FusedO3Params& p) {
+__device__ __forceinline__ void o3_relax_orbit(const Pops& d, float E, float X, float Y, float Z, float a0, float ax,
+                                               float ay, float* __restrict__ out, long long plane) {
   constexpr int kind = Def::O.kind[K];
   constexpr int i0 = Def::O.idx[K][0], i1 = Def::O.idx[K][1], i2 = Def::O.idx[K][2], i3 = Def::O.idx[K][3];
-  const HL* w = p.ow[K];
-  const float E = class_sum(kEE{}, w, e, hl(w[0], nd));
   if constexpr (kind == 1) {
     o3_relax<Def, i0, Pops>(d, E, a0, ax, ay, out, plane);
   } else if constexpr (kind == 2) {
-    const float X = class_sum(kOE{}, w, e, 0.0f);
     o3_relax<Def, i0, Pops>(d, E + X, a0, ax, ay, out, plane);
     o3_relax<Def, i1, Pops>(d, E - X, a0, ax, ay, out, plane);
   } else if constexpr (kind == 3) {
-    const float Y = class_sum(kEO{}, w, e, 0.0f);
     o3_relax<Def, i0, Pops>(d, E + Y, a0, ax, ay, out, plane);
     o3_relax<Def, i2, Pops>(d, E - Y, a0, ax, ay, out, plane);
   } else {
-    const float X = class_sum(kOE{}, w, e, 0.0f);
-    const float Y = class_sum(kEO{}, w, e, 0.0f);
-    const float Z = class_sum(kOO{}, w, e, 0.0f);
     const float EP = E + Z, EM = E - Z, XP = X + Y, XM = X - Y;
     o3_relax<Def, i0, Pops>(d, EP + XP, a0, ax, ay, out, plane);   // (+, +)
     o3_relax<Def, i1, Pops>(d, EM - XM, a0, ax, ay, out, plane);   // (-, +)
     o3_relax<Def, i2, Pops>(d, EM + XM, a0, ax, ay, out, plane);   // (+, -)
     o3_relax<Def, i3, Pops>(d, EP - XP, a0, ax, ay, out, plane);   // (-, -)
+  }
+}
+
+// Equilibrium and relaxation of the orbits (a_x, a_y), a_x >= a_y, and of their
+// exchanged ones (rlbm_o3.cuh).
+template <class Def, int K, class Pops>
+__device__ __forceinline__ void o3_collide_orbit(const Pops& d, const float (&e)[kO3Mono], float nd,
+                                                 float a0, float ax, float ay, float* __restrict__ out,
+                                                 long long plane, const FusedO3Params& p) {
+  constexpr int nx = Def::O.ax[K], ny = Def::O.ay[K];
+  if constexpr (nx >= ny) {
+    constexpr int KX = exchanged_orbit<Def, K>();
+    static_assert(KX >= 0, "full-symmetric groups are closed under exchange");
+    const HL* w = p.ow[K];
+    const float both = class_sum(O3Both{}, O3Both{}, w, e, hl(w[0], nd));
+    float X = 0.0f, Y = 0.0f, Z = 0.0f;
+    if constexpr (nx != 0 && ny != 0) Z = class_sum(O3OddXY{}, O3OddXY{}, w, e, 0.0f);
+    if constexpr (nx != 0) X = class_sum(O3OddX{}, O3OddX{}, w, e, 0.0f);
+    if constexpr (ny != 0) Y = class_sum(O3OddY{}, O3OddY{}, w, e, 0.0f);
+    o3_relax_orbit<Def, K, Pops>(d, class_sum(O3Even{}, O3Even{}, w, e, both), X, Y, Z, a0, ax, ay, out, plane);
+    if constexpr (KX != K) {
+      X = Y = 0.0f;
+      if constexpr (ny != 0) X = class_sum(O3OddY{}, O3OddX{}, w, e, 0.0f);
+      if constexpr (nx != 0) Y = class_sum(O3OddX{}, O3OddY{}, w, e, 0.0f);
+      o3_relax_orbit<Def, KX, Pops>(d, class_sum(O3EvenX{}, O3Even{}, w, e, both), X, Y, Z, a0, ax, ay, out, plane);
+    }
   }
 }
 
@@ -227,7 +241,9 @@ __device__ __forceinline__ void o3_collide_all(std::integer_sequence<int, Ks...>
 //   Q = 133: 0 x 3 1238; 60 x 4 1045; 80 x 4 1048; 96 x 4 1057; 80 x 5 1270
 //   Q = 149: 0 x 3 1271; 60 x 4 1187; 80 x 4 1147; 96 x 4 1137; 80 x 5 1460
 // One pass (all values in registers, four blocks, 70-90 bytes spilled) was 4 %
-// slower than 0 x 4.  Results are the same bit for bit.
+// slower than 0 x 4.  Results are the same bit for bit.  With the constants of
+// exchanged orbits shared (o3_collide_orbit): Q = 100 731 -> 705, Q = 99 719 -> 715,
+// Q = 133 1048 -> 1001, Q = 149 1143 -> 1098; 0.66-0.70 of the copy bandwidth.
 constexpr bool O3_TWO_PASS = true;
 
 template <class Def>

@@ -6,18 +6,14 @@
 namespace rlbm {
 namespace {
 
-template <class Def, int K, class Put>
-__device__ __forceinline__ void init_orbit(const IoO3Params& p, const double (&e)[kO3Mono], double dn, const Put& put) {
-  double E, X, Y, Z;
-  orbit_equilibrium_o3<Def, K>(p.b.ow[K], e, dn, E, X, Y, Z);
-  emit_orbit<Def, K>(put, E, X, Y, Z);
-}
-
-template <class Def, class Put, int... Ks>
-__device__ __forceinline__ void init_all(std::integer_sequence<int, Ks...>, const IoO3Params& p,
-                                         const double (&e)[kO3Mono], double dn, const Put& put) {
-  (init_orbit<Def, Ks>(p, e, dn, put), ...);
-}
+template <class Put>
+struct EmitUse {
+  const Put& put;
+  template <class Def, int K>
+  __device__ __forceinline__ void at(double E, double X, double Y, double Z) const {
+    emit_orbit<Def, K>(put, E, X, Y, Z);
+  }
+};
 
 template <class Def, typename S>
 __global__ void __launch_bounds__(128) init_o3c_kernel(const __grid_constant__ IoO3Params p, FieldPtrs fd,
@@ -31,7 +27,7 @@ __global__ void __launch_bounds__(128) init_o3c_kernel(const __grid_constant__ I
     double e[kO3Mono];
     deviations64(p.b, o, e);
     const PutPlain<S> put{cur + ((unsigned)y * (unsigned)p.b.pitch + (unsigned)x), (size_t)p.b.plane};
-    init_all<Def>(std::make_integer_sequence<int, Def::O.K>{}, p, e, o.n - p.nref, put);
+    all_orbits_o3<Def>(std::make_integer_sequence<int, Def::O.K>{}, p.b, e, o.n - p.nref, EmitUse<PutPlain<S>>{put});
   }
   report(fl, p.b.err);
 }

@@ -12,6 +12,8 @@
 // and FP32 evaluation has no cancellation.
 #pragma once
 
+#include <utility>
+
 #include "rlbm_internal.h"
 
 namespace rlbm {
@@ -60,6 +62,27 @@ template <typename R_t>
 __device__ __forceinline__ void o3_deviations(R_t m, R_t c, R_t n, R_t U0, R_t Ux, R_t Uy, R_t dU, R_t dR,
                                               R_t dT, R_t T, R_t R, R_t (&e)[kO3Mono]) {
   o3_deviations<R_t>(m, c, n, U0, Ux, Uy, dU, dR, dT, T, R, e, o3_rcp(m));
+}
+
+// Parity classes of the monomials (kO3Mono order), and the same lists with x and
+// y exchanged: the dual basis of the orbit (a_y, a_x) is that of (a_x, a_y) with
+// the exchanged monomials, so one row of constants serves both and the part of
+// the even class that the exchange leaves alone is summed once.
+template <int... L>
+using MonoList = std::integer_sequence<int, L...>;
+using O3Both = MonoList<0, 1, 9, 17>;            // even in p_x and p_y: 1, t, pz^2, t pz^2,
+using O3Even = MonoList<6, 7, 10, 11>;           // px^2, py^2, t px^2, t py^2
+using O3EvenX = MonoList<7, 6, 11, 10>;
+using O3OddX = MonoList<2, 4, 13, 15, 18>;       // odd in p_x only
+using O3OddY = MonoList<3, 5, 16, 14, 19>;       // odd in p_y only (exchange of O3OddX)
+using O3OddXY = MonoList<8, 12>;                 // odd in both
+
+// The orbit of the exchanged representative (K itself where a_x = a_y).
+template <class Def, int K>
+__host__ __device__ constexpr int exchanged_orbit() {
+  for (int j = 0; j < Def::O.K; ++j)
+    if (Def::O.grp[j] == Def::O.grp[K] && Def::O.ax[j] == Def::O.ay[K] && Def::O.ay[j] == Def::O.ax[K]) return j;
+  return -1;
 }
 
 }  // namespace rlbm
