@@ -273,8 +273,8 @@ def cpu_baseline_o3(seconds=10.0, side=24, procs=None):
 # (profiles/fp64_kernels_alu_1024.md).  The peak is measured (fp64_peak); GB300's
 # nominal FP64 rate is reported beside it and used only if the probe fails.
 FP64_PEAK_TFLOPS = 1.25
-FP64_FLOP_PER_SITE = {"step_f64_kernel/5,12,14,17,21,26": 3271.0,
-                      "step_o3_kernel/1,2,5,6,7,9,10,11,12,13,15": 7352.0}
+FP64_FLOP_PER_SITE = {"fused_f64_kernel/5,12,14,17,21,26": 1121.4,
+                      "fused_f64_o3_kernel/1,2,5,6,7,9,10,11,12,13,15": 2378.5}
 
 
 _FP64_PEAK = []
@@ -309,7 +309,7 @@ def fp64_alu(mlups, key):
 def kernel_name(dtype, variant):
     stencil = {1: "5,12,14,17,21,26", 2: "1,2,3,4,5,6", 3: "1,14,49,51,60,70", 4: "3,9,10,14,17,21"}.get(variant)
     if dtype == "f64":
-        return "step_f64_kernel<64>"
+        return "fused_f64_kernel<StencilDef<5,12,14,17,21,26>>"
     if stencil is None:
         return "step_f32_kernel<64>"
     return "fused_f32_kernel<StencilDef<%s>, %s>" % (stencil, "true" if dtype == "bf16dev" else "false")
@@ -373,7 +373,8 @@ O3_SOURCES = ["paper_1703_04605_gb300/csrc/rlbm_fused_o3.cu", "paper_1703_04605_
               "paper_1703_04605_gb300/csrc/rlbm_fused.cuh",
               "paper_1703_04605_gb300/csrc/rlbm_internal.h", "paper_1703_04605_gb300/csrc/rlbm_stencils.h",
               "paper_1703_04605_gb300/csrc/rlbm_kernels.cuh"]
-F3D_SOURCES = ["paper_1703_04605_gb300/csrc/rlbm_fused3d.cu", "paper_1703_04605_gb300/csrc/rlbm_fused.cuh",
+F3D_SOURCES = ["paper_1703_04605_gb300/csrc/rlbm_fused3d.cu", "paper_1703_04605_gb300/csrc/rlbm_octants.cuh",
+               "paper_1703_04605_gb300/csrc/rlbm_solve3.cuh", "paper_1703_04605_gb300/csrc/rlbm_fused.cuh",
                "paper_1703_04605_gb300/csrc/rlbm_internal.h", "paper_1703_04605_gb300/csrc/rlbm_stencils.h",
                "paper_1703_04605_gb300/csrc/rlbm_kernels.cuh"]
 FUSED_SOURCES = ["paper_1703_04605_gb300/csrc/rlbm_fused.cuh", "paper_1703_04605_gb300/csrc/rlbm_internal.h",
@@ -833,7 +834,7 @@ def run_third_order(args):
             "f64": {"MLUPS": sites / (ms64 / 1e3) / 1e6, "ms_per_step": ms64, "steps": k64,
                     "frac_hbm": info64["bytes_per_site"] * sites / (ms64 / 1e3) / 1e9 / peak,
                     "alu": fp64_alu(sites / (ms64 / 1e3) / 1e6,
-                                    "step_o3_kernel/" + ",".join(str(g) for g in sorted(st["groups"])))},
+                                    "fused_f64_o3_kernel/" + ",".join(str(g) for g in sorted(st["groups"])))},
             "error_vs_f64": err, "gpu_launches": args.steps, "clocks": clk.summary()}
     if not args.no_cpu_baseline and rank == 0:
         line["cpu_baseline"] = cpu_baseline_o3()
@@ -965,7 +966,7 @@ def main():
                 l2.step(nsteps - (args.warmup + k))
                 rec["error_vs_f64"] = dict(errs(l2.moments(), rm), steps=nsteps)
             else:
-                rec["alu"] = fp64_alu(rec["MLUPS"], "step_f64_kernel/" + ",".join(str(g) for g in st["groups"]))
+                rec["alu"] = fp64_alu(rec["MLUPS"], "fused_f64_kernel/" + ",".join(str(g) for g in st["groups"]))
             by_dtype[dt] = rec
             l2.close()
 

@@ -4,7 +4,7 @@
 // An FP64 instruction of a warp holds its SM sub-partition's FP64 unit for 64
 // cycles (half a lane a clock) however few warps there are, so a lattice with
 // fewer warps than the GPU has sub-partitions (4 an SM) takes as long as one
-// warp's FP64 instructions: 870 x 64 cycles in fused_f64_kernel, 27 us.  Here
+// warp's FP64 instructions: 741 x 64 cycles in fused_f64_kernel, 23 us.  Here
 // the populations of a site are spread over L lanes (table rows in place of
 // compile-time constants), their moments summed by shuffles, the site solve
 // repeated on every lane: about 308 FP64 instructions a warp at L = 16, 391 at

@@ -71,3 +71,13 @@ def test_lane_counts(shape):
     got, _ = run_gpu(st, 0.8, f, "f64", 2)
     e = errors(got, run_oracle(st, 0.8, f, 2))
     assert max(e.values()) < 1e-12, e
+
+
+@pytest.mark.parametrize("shape", [(50, 16), (96, 77)])
+def test_other_group_set(shape):
+    # no compiled kernel: several lanes a site, and the table-driven kernel above that
+    st = dict(groups=[1, 2, 3, 6, 7, 11], m=5.0, v0=0.3095)
+    f = smooth_fields(shape[0], shape[1], seed=4, dn=0.05, dT=0.05, du=0.05)
+    got, info = run_gpu(st, 0.9, f, "f64", 3)
+    e = errors(got, run_oracle(st, 0.9, f, 3))
+    assert max(e.values()) < 1e-12, e
