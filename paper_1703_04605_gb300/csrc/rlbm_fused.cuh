@@ -1051,8 +1051,10 @@ __global__ void __launch_bounds__(128, fused_min_blocks<Def, BF, EXL>()) fused_f
 // 512^2 M1 FP32 22.0 / 24.6, BF16 29.8 / 31.5, G1-G6 15.4 / 18.3, S2 19.0 / 20.7;
 // 2048^2 M1 297 / 301, S2 BF16 334 / 349; 4096^2 M1 1179 / 1191.  The one kernel
 // that loses on large lattices is E5's FP32 one, which is at the bandwidth and
-// whose loads are slower off the read-only path (2048^2 403 / 391, 512^2
-// 29.9 / 32.8): chained up to 2^20 sites, where the launch saved still counts.
+// whose loads are slower off the read-only path: 255^2 9.5 / 12.1, 383^2 16.8 /
+// 18.5, 512^2 31.6 / 32.8, 601^2 47.0 / 47.9, but 727^2 67.2 / 66.1, 853^2 87.4 /
+// 86.1, 1023^2 124.8 / 123.6, 2048^2 403 / 391.  It is chained up to 3 2^17 sites
+// (627^2), where the launch saved still counts for more.
 // Entry point of the step kernel of a stencil, for CUDA graph kernel nodes
 // (rlbm_batch_step); the node's grid is (Nx Ny + 127)/128 blocks of 128.
 // mode: 0 FP32, 1 BF16 deviation, 2 / 3 FP32 with extended moment sums of
@@ -1073,7 +1075,7 @@ cudaError_t launch_fused_impl(const FusedParams& p, const void* fin, void* fout,
   if (mode == 2) return launch_pdl(fused_f32_kernel<Def, false, 1>, grid, 128, s, p, fin, fout);
   if (mode == 3) return launch_pdl(fused_f32_kernel<Def, false, 2>, grid, 128, s, p, fin, fout);
   if constexpr (Def::Q == 73) {
-    if (nsite > (1LL << 20)) {
+    if (nsite > (3LL << 17)) {
       fused_f32_kernel<Def, false, 0, false><<<grid, 128, 0, s>>>(p, fin, fout);
       return cudaGetLastError();
     }
