@@ -45,6 +45,18 @@ struct Cfg3<Stencil3G16> {
   static constexpr bool KEEP_PLANE = true;
 };
 
+// Lattices of at most 200 sites an SM (152 SMs): blocks of 64 threads, so that the
+// sites are on all of the SMs.  Such a step is bound by the latency of one pass, and
+// by the loads that an SM's warps share.  us a step, Cfg3's block / 64 threads:
+// 17^3 M1 10.3 / 8.2, E5 12.3 / 11.5; 23^3 M1 10.3 / 8.2; 27^3 G16 8.2 / 6.2, S2 9.3 /
+// 8.2; 31^3 S2 10.3 / 9.3, E5 14.4 / 12.8 (32 threads: 12.3, but 17^3 12.3).  Above, at
+// 33^3, M1 loses (10.3 / 12.3) and the others are even.
+template <class C>
+struct Small3 : C {
+  static constexpr int TB = 64, BLOCKS = C::BLOCKS * C::TB / 64;
+};
+constexpr long long kSmall3 = 152 * 200;
+
 // The projections of App. B at a site, without their normalisations (in p.gf).
 struct Proj3 {
   float r0, r1, r5, r9, r10, r11, r12, r13, h;
@@ -169,7 +181,7 @@ __global__ void __launch_bounds__(Cfg::TB, Cfg::BLOCKS) fused3d_kernel(const __g
 }
 
 template <class Cfg>
-cudaError_t launch_fused3d_impl(const Fused3Params& p, const void* fin, void* fout, cudaStream_t s) {
+cudaError_t launch_fused3d_cfg(const Fused3Params& p, const void* fin, void* fout, cudaStream_t s) {
   constexpr int smem = Cfg::KEEP * Cfg::TB * (int)sizeof(float);
   static const cudaError_t attr =
       cudaFuncSetAttribute(fused3d_kernel<Cfg>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -177,6 +189,12 @@ cudaError_t launch_fused3d_impl(const Fused3Params& p, const void* fin, void* fo
   const unsigned grid = (unsigned)(((long long)p.Nx * p.Ny * p.Nz + Cfg::TB - 1) / Cfg::TB);
   fused3d_kernel<Cfg><<<grid, Cfg::TB, smem, s>>>(p, static_cast<const float*>(fin), static_cast<float*>(fout));
   return cudaGetLastError();
+}
+
+template <class Cfg>
+cudaError_t launch_fused3d_impl(const Fused3Params& p, const void* fin, void* fout, cudaStream_t s) {
+  if ((long long)p.Nx * p.Ny * p.Nz <= kSmall3) return launch_fused3d_cfg<Small3<Cfg>>(p, fin, fout, s);
+  return launch_fused3d_cfg<Cfg>(p, fin, fout, s);
 }
 
 }  // namespace
