@@ -1114,11 +1114,11 @@ __device__ __forceinline__ void f32_init_pops(std::integer_sequence<int, Is...>,
       ...);
 }
 
-// S_{-1} is not written: the read-out of the freshly initialised state reads
-// S_0 in place (f32_moments_kernel<Def, false>).
+// S_{-1} is not written: other is marked, and the read-out of the freshly
+// initialised state reads S_0 in place.
 template <class Def>
 __global__ void __launch_bounds__(128) f32_init_kernel(const __grid_constant__ FusedParams p, FieldPtrs fd,
-                                                       float* __restrict__ cur) {
+                                                       float* __restrict__ cur, float* __restrict__ other) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned fl = 0;
   if (s < p.Nx * p.Ny) {
@@ -1148,6 +1148,7 @@ __global__ void __launch_bounds__(128) f32_init_kernel(const __grid_constant__ F
     float c[6][6];
     fused_coeffs(p, ss, c);
     f32_init_pops<Def>(std::make_integer_sequence<int, Def::Q>{}, c, cur, p.plane, p.pitch, x, y);
+    if (s == 0) mark_unwritten(other);
   }
   report(fl, p.err);
 }
@@ -1158,12 +1159,13 @@ __global__ void __launch_bounds__(128) f32_init_kernel(const __grid_constant__ F
 // reference in FP32, the EOS finished by an FP64 Newton step), so n and T
 // carry FP32 rounding of their deviations from the reference only.  The
 // moment planes are assembled in FP64 from the float-float sums.
-// PULL: the state at t is the pull of S_{t-1} in prev; otherwise (right
-// after f32_init_kernel) it is S_0 in prev read in place.
-template <class Def, bool PULL>
+// The state at t is the pull of S_{t-1} in prev; where prev carries the mark
+// (right after f32_init_kernel) it is S_0 in cur read in place.
+template <class Def>
 __global__ void __launch_bounds__(128) f32_moments_kernel(const __grid_constant__ FusedParams fp,
                                                           const __grid_constant__ StepParams<double> p,
-                                                          const float* __restrict__ prev, MomentOut mo) {
+                                                          const float* __restrict__ prev,
+                                                          const float* __restrict__ cur, MomentOut mo) {
   const int site = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned fl = 0;
   const long long N = (long long)p.Nx * p.Ny;
@@ -1171,14 +1173,14 @@ __global__ void __launch_bounds__(128) f32_moments_kernel(const __grid_constant_
     int x, y;
     site_of(site, p.Nx, x, y);
     float d[Def::Q];
-    if constexpr (PULL) {
+    if (!is_unwritten(prev)) {
       fused_load_all<Def, false>(std::make_integer_sequence<int, Def::Q>{}, d, prev, nullptr, p.plane, p.pitch, x,
                                  y, p.Nx, p.Ny);
     } else {
       const unsigned here = (unsigned)y * (unsigned)p.pitch + (unsigned)x;
       const size_t pl = (unsigned)p.plane;
 #pragma unroll
-      for (int i = 0; i < Def::Q; ++i) d[i] = __ldg(prev + here + pl * i);
+      for (int i = 0; i < Def::Q; ++i) d[i] = __ldg(cur + here + pl * i);
     }
     ExMoments em;
     em.N0 = em.Nx = em.Ny = em.K0 = em.Kx = em.Ky = FF{0.0f, 0.0f};
@@ -1225,17 +1227,14 @@ __global__ void __launch_bounds__(128) f32_moments_kernel(const __grid_constant_
   report(fl, p.err);
 }
 
-// what: 0 init of S_0 into buf, 1 read-out of the pull of buf, 2 read-out of
-// S_0 in buf, in place.
 template <class Def>
-cudaError_t launch_f32_io_impl(int what, const FusedParams& fp, const StepParams<double>& p, FieldPtrs fd, void* buf,
-                               MomentOut mo, cudaStream_t s) {
+cudaError_t launch_f32_io_impl(bool init, const FusedParams& fp, const StepParams<double>& p, FieldPtrs fd, void* cur,
+                               void* other, MomentOut mo, cudaStream_t s) {
   const long long nsite = (long long)p.Nx * p.Ny;
   const unsigned grid = (unsigned)((nsite + 127) / 128);
-  float* b = static_cast<float*>(buf);
-  if (what == 0) f32_init_kernel<Def><<<grid, 128, 0, s>>>(fp, fd, b);
-  else if (what == 1) f32_moments_kernel<Def, true><<<grid, 128, 0, s>>>(fp, p, b, mo);
-  else f32_moments_kernel<Def, false><<<grid, 128, 0, s>>>(fp, p, b, mo);
+  float *c = static_cast<float*>(cur), *o = static_cast<float*>(other);
+  if (init) f32_init_kernel<Def><<<grid, 128, 0, s>>>(fp, fd, c, o);
+  else f32_moments_kernel<Def><<<grid, 128, 0, s>>>(fp, p, o, c, mo);
   return cudaGetLastError();
 }
 

@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(64, 8) fused_f64_kernel(const __grid_constant_
   if (s < p.Nx * p.Ny) {
     int x, y;
     site_of(s, p.Nx, x, y);
-    const Pull64 q{fin, (size_t)p.plane, (unsigned)p.pitch, x, y, p.Nx, p.Ny, p.dxm, p.dym};
+    const Pull64 q{fin, (size_t)p.plane, (unsigned)p.pitch, x, y, p.Nx, p.Ny, p.dxm, p.dym, -1};
     using Orb = std::make_integer_sequence<int, Def::O.K>;
     double M[9];
     acc64_all<Def>(Orb{}, q, p.gm, M);

@@ -208,19 +208,21 @@ __host__ __device__ constexpr bool orbit_ends_group() {
   return K + 1 == Def::O.K || Def::O.grp[K + 1] != Def::O.grp[K];
 }
 
-// Where a site's populations are pulled from.
+// Where a site's populations are pulled from; mask 0: from the site itself (S_0
+// read in place), -1: from x - n_i.
 struct Pull64 {
   const double* fin;
   size_t plane;
   unsigned pitch;
   int x, y, Nx, Ny;
   const int *dxm, *dym;
+  int mask;
 };
 
 template <class Def, int I>
 __device__ __forceinline__ double pull64(const Pull64& q) {
-  const unsigned xs = (unsigned)wrap_sub(q.x, q.dxm[Def::F.nx[I] + kMaxDisp], q.Nx);
-  const unsigned ys = (unsigned)wrap_sub(q.y, q.dym[Def::F.ny[I] + kMaxDisp], q.Ny);
+  const unsigned xs = (unsigned)wrap_sub(q.x, q.dxm[Def::F.nx[I] + kMaxDisp] & q.mask, q.Nx);
+  const unsigned ys = (unsigned)wrap_sub(q.y, q.dym[Def::F.ny[I] + kMaxDisp] & q.mask, q.Ny);
   return __ldg(q.fin + (ys * q.pitch + xs) + q.plane * I);
 }
 
@@ -231,11 +233,12 @@ struct Pull32 {
   unsigned pitch;
   int x, y, Nx, Ny;
   const int *dxm, *dym;
+  int mask;
 };
 template <class Def, int I>
 __device__ __forceinline__ double pull64(const Pull32& q) {
-  const unsigned xs = (unsigned)wrap_sub(q.x, q.dxm[Def::F.nx[I] + kMaxDisp], q.Nx);
-  const unsigned ys = (unsigned)wrap_sub(q.y, q.dym[Def::F.ny[I] + kMaxDisp], q.Ny);
+  const unsigned xs = (unsigned)wrap_sub(q.x, q.dxm[Def::F.nx[I] + kMaxDisp] & q.mask, q.Nx);
+  const unsigned ys = (unsigned)wrap_sub(q.y, q.dym[Def::F.ny[I] + kMaxDisp] & q.mask, q.Ny);
   return (double)__ldg(q.fin + (ys * q.pitch + xs) + q.plane * I);
 }
 

@@ -16,9 +16,9 @@ __device__ __forceinline__ bool site_of3(const P& p, int& x, int& y, int& z, int
 }
 
 template <class P, typename S>
-__device__ __forceinline__ Pull3<S> pull_of(const P& p, const S* fin, int x, int y, int z) {
+__device__ __forceinline__ Pull3<S> pull_of(const P& p, const S* fin, int x, int y, int z, int mask = -1) {
   return Pull3<S>{fin, (size_t)p.plane, (unsigned)p.zstride, (unsigned)p.pitch, x, y, z, p.Nx, p.Ny, p.Nz,
-                  p.dxm, p.dym, p.dzm};
+                  p.dxm, p.dym, p.dzm, mask};
 }
 
 struct Relax3 {
@@ -103,7 +103,8 @@ __device__ __forceinline__ void put_octants(std::integer_sequence<int, Ks...>, c
 }
 
 template <class D, class P, typename S>
-__global__ void __launch_bounds__(64, 8) init3c_kernel(const __grid_constant__ P p, Field3Ptrs f, S* __restrict__ cur) {
+__global__ void __launch_bounds__(64, 8) init3c_kernel(const __grid_constant__ P p, Field3Ptrs f, S* __restrict__ cur,
+                                                      S* __restrict__ other) {
   int x, y, z, s;
   unsigned fl = 0;
   if (site_of3(p, x, y, z, s)) {
@@ -112,19 +113,22 @@ __global__ void __launch_bounds__(64, 8) init3c_kernel(const __grid_constant__ P
     eq.prepare(p, o);
     put_octants<D>(std::make_integer_sequence<int, D::O.K>{}, p, eq,
                    cur + ((unsigned)z * (unsigned)p.zstride + (unsigned)y * (unsigned)p.pitch + (unsigned)x));
+    if (s == 0) mark_unwritten(other);
   }
   report(fl, p.err);
 }
 
 template <class D, class P, typename S>
 __global__ void __launch_bounds__(64, 8) moments3c_kernel(const __grid_constant__ P p, const S* __restrict__ prev,
-                                                          MomentOut mo) {
+                                                          const S* __restrict__ cur, MomentOut mo) {
   int x, y, z, s;
   unsigned fl = 0;
   if (site_of3(p, x, y, z, s)) {
     const long long N = (long long)p.Nx * p.Ny * p.Nz;
     double m[14];
-    acc_octants<D>(std::make_integer_sequence<int, D::O.K>{}, pull_of(p, prev, x, y, z), p.gm, m);
+    const bool here = is_unwritten(prev);
+    acc_octants<D>(std::make_integer_sequence<int, D::O.K>{}, pull_of(p, here ? cur : prev, x, y, z, here ? 0 : -1),
+                   p.gm, m);
 #pragma unroll
     for (int k = 0; k < 14; ++k) m[k] += p.mref[k];
     const Mac3 o = solve3_seeded(m, p.sc, p.rt64, p.rt32, fl);
@@ -161,16 +165,22 @@ cudaError_t step3c(const P& p, const void* fin, void* fout, cudaStream_t s) {
 }
 
 template <class D, class P>
-cudaError_t init3c(bool f64, const P& p, Field3Ptrs f, void* cur, cudaStream_t s) {
-  if (f64) init3c_kernel<D, P, double><<<grid64(p), 64, 0, s>>>(p, f, static_cast<double*>(cur));
-  else init3c_kernel<D, P, float><<<grid64(p), 64, 0, s>>>(p, f, static_cast<float*>(cur));
+cudaError_t init3c(bool f64, const P& p, Field3Ptrs f, void* cur, void* other, cudaStream_t s) {
+  if (f64)
+    init3c_kernel<D, P, double><<<grid64(p), 64, 0, s>>>(p, f, static_cast<double*>(cur), static_cast<double*>(other));
+  else
+    init3c_kernel<D, P, float><<<grid64(p), 64, 0, s>>>(p, f, static_cast<float*>(cur), static_cast<float*>(other));
   return cudaGetLastError();
 }
 
 template <class D, class P>
-cudaError_t moments3c(bool f64, const P& p, const void* prev, MomentOut mo, cudaStream_t s) {
-  if (f64) moments3c_kernel<D, P, double><<<grid64(p), 64, 0, s>>>(p, static_cast<const double*>(prev), mo);
-  else moments3c_kernel<D, P, float><<<grid64(p), 64, 0, s>>>(p, static_cast<const float*>(prev), mo);
+cudaError_t moments3c(bool f64, const P& p, const void* prev, const void* cur, MomentOut mo, cudaStream_t s) {
+  if (f64)
+    moments3c_kernel<D, P, double><<<grid64(p), 64, 0, s>>>(p, static_cast<const double*>(prev),
+                                                            static_cast<const double*>(cur), mo);
+  else
+    moments3c_kernel<D, P, float><<<grid64(p), 64, 0, s>>>(p, static_cast<const float*>(prev),
+                                                           static_cast<const float*>(cur), mo);
   return cudaGetLastError();
 }
 
@@ -188,28 +198,30 @@ cudaError_t launch_step3c(const C3Params3& p, const void* fin, void* fout, cudaS
   return step3c<Stencil3O3M5>(p, fin, fout, s);
 }
 
-cudaError_t launch_init3c(int kind, bool f64, const C3Params2& p, Field3Ptrs f, void* cur, cudaStream_t s) {
+cudaError_t launch_init3c(int kind, bool f64, const C3Params2& p, Field3Ptrs f, void* cur, void* other, cudaStream_t s) {
   switch (kind) {
-    case 1: return init3c<Stencil3M1>(f64, p, f, cur, s);
-    case 2: return init3c<Stencil3G16>(f64, p, f, cur, s);
-    case 3: return init3c<Stencil3E5>(f64, p, f, cur, s);
-    default: return init3c<Stencil3S2>(f64, p, f, cur, s);
+    case 1: return init3c<Stencil3M1>(f64, p, f, cur, other, s);
+    case 2: return init3c<Stencil3G16>(f64, p, f, cur, other, s);
+    case 3: return init3c<Stencil3E5>(f64, p, f, cur, other, s);
+    default: return init3c<Stencil3S2>(f64, p, f, cur, other, s);
   }
 }
-cudaError_t launch_init3c(bool f64, const C3Params3& p, Field3Ptrs f, void* cur, cudaStream_t s) {
-  return init3c<Stencil3O3M5>(f64, p, f, cur, s);
+cudaError_t launch_init3c(bool f64, const C3Params3& p, Field3Ptrs f, void* cur, void* other, cudaStream_t s) {
+  return init3c<Stencil3O3M5>(f64, p, f, cur, other, s);
 }
 
-cudaError_t launch_moments3c(int kind, bool f64, const C3Params2& p, const void* prev, MomentOut mo, cudaStream_t s) {
+cudaError_t launch_moments3c(int kind, bool f64, const C3Params2& p, const void* prev, const void* cur, MomentOut mo,
+                             cudaStream_t s) {
   switch (kind) {
-    case 1: return moments3c<Stencil3M1>(f64, p, prev, mo, s);
-    case 2: return moments3c<Stencil3G16>(f64, p, prev, mo, s);
-    case 3: return moments3c<Stencil3E5>(f64, p, prev, mo, s);
-    default: return moments3c<Stencil3S2>(f64, p, prev, mo, s);
+    case 1: return moments3c<Stencil3M1>(f64, p, prev, cur, mo, s);
+    case 2: return moments3c<Stencil3G16>(f64, p, prev, cur, mo, s);
+    case 3: return moments3c<Stencil3E5>(f64, p, prev, cur, mo, s);
+    default: return moments3c<Stencil3S2>(f64, p, prev, cur, mo, s);
   }
 }
-cudaError_t launch_moments3c(bool f64, const C3Params3& p, const void* prev, MomentOut mo, cudaStream_t s) {
-  return moments3c<Stencil3O3M5>(f64, p, prev, mo, s);
+cudaError_t launch_moments3c(bool f64, const C3Params3& p, const void* prev, const void* cur, MomentOut mo,
+                             cudaStream_t s) {
+  return moments3c<Stencil3O3M5>(f64, p, prev, cur, mo, s);
 }
 
 }  // namespace rlbm

@@ -166,7 +166,8 @@ __host__ __device__ constexpr int octant_comps() {
   return (D::O.ax[K] ? 1 : 0) | (D::O.ay[K] ? 2 : 0) | (D::O.az[K] ? 4 : 0);
 }
 
-// A site's place; dxm, dym, dzm: displacements reduced modulo the lattice.
+// A site's place; dxm, dym, dzm: displacements reduced modulo the lattice; mask 0:
+// read in place, -1: pulled.
 template <typename S>
 struct Pull3 {
   const S* fin;
@@ -174,13 +175,14 @@ struct Pull3 {
   unsigned zs, pitch;
   int x, y, z, Nx, Ny, Nz;
   const int *dxm, *dym, *dzm;
+  int mask;
 };
 
 template <class D, int I, typename S>
 __device__ __forceinline__ double pull3d(const Pull3<S>& q) {
-  const unsigned xs = (unsigned)wrap_sub(q.x, q.dxm[D::U.nx[I] + kMaxDisp], q.Nx);
-  const unsigned ys = (unsigned)wrap_sub(q.y, q.dym[D::U.ny[I] + kMaxDisp], q.Ny);
-  const unsigned zs = (unsigned)wrap_sub(q.z, q.dzm[D::U.nz[I] + kMaxDisp], q.Nz);
+  const unsigned xs = (unsigned)wrap_sub(q.x, q.dxm[D::U.nx[I] + kMaxDisp] & q.mask, q.Nx);
+  const unsigned ys = (unsigned)wrap_sub(q.y, q.dym[D::U.ny[I] + kMaxDisp] & q.mask, q.Ny);
+  const unsigned zs = (unsigned)wrap_sub(q.z, q.dzm[D::U.nz[I] + kMaxDisp] & q.mask, q.Nz);
   return (double)__ldg(q.fin + (zs * q.zs + ys * q.pitch + xs) + q.plane * I);
 }
 

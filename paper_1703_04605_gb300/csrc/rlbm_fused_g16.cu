@@ -9,9 +9,9 @@ cudaError_t launch_fused<StencilG16>(const FusedParams& p, const void* fin, void
   return launch_fused_impl<StencilG16>(p, fin, fout, mode, s);
 }
 template <>
-cudaError_t launch_f32_io<StencilG16>(int what, const FusedParams& fp, const StepParams<double>& p, FieldPtrs fd, void* buf,
-                                   MomentOut mo, cudaStream_t s) {
-  return launch_f32_io_impl<StencilG16>(what, fp, p, fd, buf, mo, s);
+cudaError_t launch_f32_io<StencilG16>(bool init, const FusedParams& fp, const StepParams<double>& p, FieldPtrs fd,
+                                    void* cur, void* other, MomentOut mo, cudaStream_t s) {
+  return launch_f32_io_impl<StencilG16>(init, fp, p, fd, cur, other, mo, s);
 }
 template <>
 const void* fused_kernel_fn<StencilG16>(int mode) {

@@ -48,16 +48,15 @@ const void* persist_kernel_fn<StencilS2>(int);
 // fin, float* fout), for graph kernel nodes; grid (Nx Ny + 127)/128, block
 // 128, no dynamic shared memory (rlbm_fused_o3.cu).
 const void* fused_o3_kernel_fn(int kind);
-// Init and read-out of FP32 storage on a compiled stencil: what = 0 init of S_0
-// into buf, 1 read-out of the pull of buf, 2 read-out of S_0 in buf in place
-// (right after the init).  BF16-deviation storage: rlbm_io2.cu.
+// Init and read-out of FP32 storage on a compiled stencil, cur and other as cur
+// and other / prev of launch_init2 and launch_moments2 (BF16-deviation storage).
 template <class Def>
-cudaError_t launch_f32_io(int what, const FusedParams& fp, const StepParams<double>& p, FieldPtrs fd, void* buf,
-                          MomentOut mo, cudaStream_t s);
+cudaError_t launch_f32_io(bool init, const FusedParams& fp, const StepParams<double>& p, FieldPtrs fd, void* cur,
+                          void* other, MomentOut mo, cudaStream_t s);
 #define RLBM_DECL_F32_IO(S)                                                                                \
   template <>                                                                                              \
-  cudaError_t launch_f32_io<S>(int, const FusedParams&, const StepParams<double>&, FieldPtrs, void*, MomentOut, \
-                               cudaStream_t);
+  cudaError_t launch_f32_io<S>(bool, const FusedParams&, const StepParams<double>&, FieldPtrs, void*, void*, \
+                               MomentOut, cudaStream_t);
 RLBM_DECL_F32_IO(StencilM1)
 RLBM_DECL_F32_IO(StencilG16)
 RLBM_DECL_F32_IO(StencilE5)

@@ -9,9 +9,9 @@ cudaError_t launch_fused<StencilS2>(const FusedParams& p, const void* fin, void*
   return launch_fused_impl<StencilS2>(p, fin, fout, mode, s);
 }
 template <>
-cudaError_t launch_f32_io<StencilS2>(int what, const FusedParams& fp, const StepParams<double>& p, FieldPtrs fd, void* buf,
-                                   MomentOut mo, cudaStream_t s) {
-  return launch_f32_io_impl<StencilS2>(what, fp, p, fd, buf, mo, s);
+cudaError_t launch_f32_io<StencilS2>(bool init, const FusedParams& fp, const StepParams<double>& p, FieldPtrs fd,
+                                    void* cur, void* other, MomentOut mo, cudaStream_t s) {
+  return launch_f32_io_impl<StencilS2>(init, fp, p, fd, cur, other, mo, s);
 }
 template <>
 const void* fused_kernel_fn<StencilS2>(int mode) {

@@ -42,7 +42,6 @@ struct rlbm_ctx {
   size_t device_bytes = 0;
   bool initialised = false;
   bool host_init = false;   // rlbm_init in progress (it sets the reference itself)
-  bool fresh = false;       // compiled init: S_0 written in place, not stepped yet (S_{-1} not written)
   std::unique_ptr<StepParams<double>> p64;
   std::unique_ptr<StepParams<float>> p32;
   int fused = 0;                 // 1: M1, 2: G1..G6, 3: E5, 4: S2; 0: generic kernel
@@ -481,17 +480,6 @@ static void fill_lanes(rlbm_ctx* c) {
   f.err = c->d_err;
 }
 
-// The read-out parameters with the displacements that pull the state (or none).
-template <class P>
-static P in_place(const P& p, bool fresh) {
-  P q = p;
-  if (fresh) {
-    std::memset(q.b.dxm, 0, sizeof q.b.dxm);
-    std::memset(q.b.dym, 0, sizeof q.b.dym);
-  }
-  return q;
-}
-
 // Context of a third-order (eleven-group) stencil: FP64 or FP32 storage,
 // generic kernels over a device table (rlbm_kernels_o3.cu).
 static rlbm_status create_o3(const rlbm_stencil* st, double m, double tau, int Nx, int Ny, rlbm_dtype dtype,
@@ -778,17 +766,18 @@ rlbm_status rlbm_init_device(rlbm_ctx* c, const double* n, const double* ux, con
   if (!c->host_init) set_reference(c, 1.0);
   cudaError_t e;
   if (c->io3) {
-    e = launch_init_o3c(c->kind64, c->dtype == RLBM_F64, *c->io3, fp, c->buf[0], c->stream);
+    e = launch_init_o3c(c->kind64, c->dtype == RLBM_F64, *c->io3, fp, c->buf[0], c->buf[1], c->stream);
   } else if (c->order == 3) {
     e = launch_init_o3(c->dtype, *c->o3, fp, c->buf[0], c->buf[1], c->stream);
   } else if (c->io2) {
-    e = launch_init2(c->kind64, c->dtype == RLBM_BF16_DEV, *c->io2, fp, c->buf[0], c->coef[0], c->stream);
+    const bool bf = c->dtype == RLBM_BF16_DEV;
+    e = launch_init2(c->kind64, bf, *c->io2, fp, c->buf[0], c->coef[0], bf ? c->coef[1] : c->buf[1], c->stream);
   } else if (c->dtype == RLBM_F32 && c->fused) {
     MomentOut none{nullptr, 0};
-    if (c->fused == 1) e = launch_f32_io<StencilM1>(0, *c->fp, *c->p64, fp, c->buf[0], none, c->stream);
-    else if (c->fused == 2) e = launch_f32_io<StencilG16>(0, *c->fp, *c->p64, fp, c->buf[0], none, c->stream);
-    else if (c->fused == 3) e = launch_f32_io<StencilE5>(0, *c->fp, *c->p64, fp, c->buf[0], none, c->stream);
-    else e = launch_f32_io<StencilS2>(0, *c->fp, *c->p64, fp, c->buf[0], none, c->stream);
+    if (c->fused == 1) e = launch_f32_io<StencilM1>(true, *c->fp, *c->p64, fp, c->buf[0], c->buf[1], none, c->stream);
+    else if (c->fused == 2) e = launch_f32_io<StencilG16>(true, *c->fp, *c->p64, fp, c->buf[0], c->buf[1], none, c->stream);
+    else if (c->fused == 3) e = launch_f32_io<StencilE5>(true, *c->fp, *c->p64, fp, c->buf[0], c->buf[1], none, c->stream);
+    else e = launch_f32_io<StencilS2>(true, *c->fp, *c->p64, fp, c->buf[0], c->buf[1], none, c->stream);
   } else {
     e = launch_init(c->dtype, *c->p64, fp, c->buf[0], c->buf[1], c->stream);
   }
@@ -796,7 +785,6 @@ rlbm_status rlbm_init_device(rlbm_ctx* c, const double* n, const double* ux, con
   c->cur = 0;
   c->t = 0;
   c->initialised = true;
-  c->fresh = c->io2 || c->io3 || (c->order == 2 && c->dtype == RLBM_F32 && c->fused);
   return RLBM_OK;
 }
 
@@ -874,7 +862,6 @@ rlbm_status rlbm_step(rlbm_ctx* c, int nsteps) {
     if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
     c->cur = 1 - c->cur;
     ++c->t;
-    c->fresh = false;
   }
   return RLBM_OK;
 }
@@ -908,23 +895,24 @@ rlbm_status rlbm_moments(rlbm_ctx* c, double* out, unsigned mask) {
   }
   MomentOut mo{direct ? direct : c->d_out, mask};
   cudaError_t e;
-  // the state at t is the pull of S_{t-1}; right after a compiled init, S_0 read in place
-  const void* src = c->fresh ? c->buf[c->cur] : c->buf[1 - c->cur];
+  // the state at t is the pull of S_{t-1}; where that buffer carries the mark of a
+  // compiled init, S_0 in the other read in place
+  const void* src = c->buf[1 - c->cur];
+  const void* cur = c->buf[c->cur];
   if (c->io3) {
-    e = launch_moments_o3c(c->kind64, c->dtype == RLBM_F64, in_place(*c->io3, c->fresh), src, mo, c->stream);
+    e = launch_moments_o3c(c->kind64, c->dtype == RLBM_F64, *c->io3, src, cur, mo, c->stream);
   } else if (c->order == 3) {
     e = launch_moments_o3(c->dtype, *c->o3, src, mo, c->stream);
   } else if (c->io2) {
-    e = launch_moments2(c->kind64, c->dtype == RLBM_BF16_DEV, in_place(*c->io2, c->fresh), src,
-                        c->fresh ? c->coef[c->cur] : c->coef[1 - c->cur], mo, c->stream);
+    e = launch_moments2(c->kind64, c->dtype == RLBM_BF16_DEV, *c->io2, src, c->coef[1 - c->cur], cur,
+                        c->coef[c->cur], mo, c->stream);
   } else if (c->dtype == RLBM_F32 && c->fused) {
     FieldPtrs none{nullptr, nullptr, nullptr, nullptr};
-    void* pv = const_cast<void*>(src);
-    const int what = c->fresh ? 2 : 1;
-    if (c->fused == 1) e = launch_f32_io<StencilM1>(what, *c->fp, *c->p64, none, pv, mo, c->stream);
-    else if (c->fused == 2) e = launch_f32_io<StencilG16>(what, *c->fp, *c->p64, none, pv, mo, c->stream);
-    else if (c->fused == 3) e = launch_f32_io<StencilE5>(what, *c->fp, *c->p64, none, pv, mo, c->stream);
-    else e = launch_f32_io<StencilS2>(what, *c->fp, *c->p64, none, pv, mo, c->stream);
+    void *o = c->buf[1 - c->cur], *k = c->buf[c->cur];
+    if (c->fused == 1) e = launch_f32_io<StencilM1>(false, *c->fp, *c->p64, none, k, o, mo, c->stream);
+    else if (c->fused == 2) e = launch_f32_io<StencilG16>(false, *c->fp, *c->p64, none, k, o, mo, c->stream);
+    else if (c->fused == 3) e = launch_f32_io<StencilE5>(false, *c->fp, *c->p64, none, k, o, mo, c->stream);
+    else e = launch_f32_io<StencilS2>(false, *c->fp, *c->p64, none, k, o, mo, c->stream);
   } else {
     e = launch_moments(c->dtype, *c->p64, src, mo, c->stream);
   }
@@ -1158,7 +1146,6 @@ void advance_all(const std::vector<rlbm_ctx*>& v, int k) {
   for (rlbm_ctx* c : v) {
     c->cur ^= (k & 1);
     c->t += k;
-    if (k > 0) c->fresh = false;
   }
 }
 

@@ -56,7 +56,6 @@ struct rlbm_ctx3 {
   int kind = 0;                          // second order: 1..4
   std::unique_ptr<C3Params2> c2;
   std::unique_ptr<C3Params3> c3;
-  bool fresh = false;                    // S_0 written in place by such an init, not stepped yet
   std::unique_ptr<StencilBuild3O3> s3;
   DevMem mem;                  // device allocator (rlbm_set_allocator at creation)
   std::string last_error;
@@ -168,24 +167,13 @@ void fill_c3o3(rlbm_ctx3* c, const StencilBuild3O3& s3) {
   }
 }
 
-// The reference state of the FP32 storage, and the displacements of a read-out.
+// The reference state of the FP32 storage.
 template <class P>
 void set_reference_c3(const rlbm_ctx3* c, P* f) {
   if (!f) return;
   f->nref = c->p.nref;
   f->ref = c->p.nref * c->sb.mref1[0] * c->sb.sb.sc.Rr;
   for (int k = 0; k < 14; ++k) f->mref[k] = c->p.mref[k];
-}
-
-template <class P>
-P in_place3(const P& p, bool fresh) {
-  P q = p;
-  if (fresh) {
-    std::memset(q.dxm, 0, sizeof q.dxm);
-    std::memset(q.dym, 0, sizeof q.dym);
-    std::memset(q.dzm, 0, sizeof q.dzm);
-  }
-  return q;
 }
 
 // Parameters of the stencil-specialised 3D kernel at reference density nref.
@@ -478,15 +466,14 @@ rlbm_status rlbm3_init(rlbm_ctx3* c, const double* n, const double* ux, const do
   Field3Ptrs fp{c->d_fields, c->d_fields + N, c->d_fields + 2 * N, c->d_fields + 3 * N, c->d_fields + 4 * N};
   c->q.b = c->p;
   const bool f64 = c->dtype == RLBM_F64;
-  cudaError_t e = c->c2           ? launch_init3c(c->kind, f64, *c->c2, fp, c->buf[0], c->stream)
-                  : c->c3         ? launch_init3c(f64, *c->c3, fp, c->buf[0], c->stream)
+  cudaError_t e = c->c2           ? launch_init3c(c->kind, f64, *c->c2, fp, c->buf[0], c->buf[1], c->stream)
+                  : c->c3         ? launch_init3c(f64, *c->c3, fp, c->buf[0], c->buf[1], c->stream)
                   : c->order == 3 ? launch_init3d_o3(c->dtype, c->q, fp, c->buf[0], c->buf[1], c->stream)
                                   : launch_init3d(c->dtype, c->p, fp, c->buf[0], c->buf[1], c->stream);
   if (e != cudaSuccess) return cuda_fail3(c, e, "init launch");
   c->cur = 0;
   c->t = 0;
   c->initialised = true;
-  c->fresh = c->c2 || c->c3;
   return check_error3(c);
 }
 
@@ -506,7 +493,6 @@ rlbm_status rlbm3_step(rlbm_ctx3* c, int nsteps) {
     if (e != cudaSuccess) return cuda_fail3(c, e, "step launch");
     c->cur = 1 - c->cur;
     ++c->t;
-    c->fresh = false;
   }
   return RLBM_OK;
 }
@@ -540,11 +526,12 @@ rlbm_status rlbm3_moments(rlbm_ctx3* c, double* out, unsigned mask) {
   }
   MomentOut mo{direct ? direct : c->d_out, mask};
   // the pre-collision state at t is the pull of S_{t-1}, the buffer the last step
-  // read; right after a compiled init, S_0 read in place
-  const void* src = c->fresh ? c->buf[c->cur] : c->buf[1 - c->cur];
+  // read; where that carries the mark of a compiled init, S_0 in the other read in place
+  const void* src = c->buf[1 - c->cur];
+  const void* cur = c->buf[c->cur];
   const bool f64 = c->dtype == RLBM_F64;
-  cudaError_t e = c->c2   ? launch_moments3c(c->kind, f64, in_place3(*c->c2, c->fresh), src, mo, c->stream)
-                  : c->c3 ? launch_moments3c(f64, in_place3(*c->c3, c->fresh), src, mo, c->stream)
+  cudaError_t e = c->c2   ? launch_moments3c(c->kind, f64, *c->c2, src, cur, mo, c->stream)
+                  : c->c3 ? launch_moments3c(f64, *c->c3, src, cur, mo, c->stream)
                           : launch_moments3d(c->dtype, c->p, src, mo, c->stream);
   if (e == cudaSuccess && !direct)
     e = cudaMemcpyAsync(out, c->d_out, need * sizeof(double), cudaMemcpyDeviceToHost, c->stream);

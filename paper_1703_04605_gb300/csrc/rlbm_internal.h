@@ -191,17 +191,20 @@ struct Fused64Params {
 cudaError_t launch_fused_f64(int kind, const Fused64Params& p, const void* fin, void* fout, cudaStream_t s);
 
 // Init and read-out of compiled second-order stencils in FP64 and
-// BF16-deviation storage (rlbm_io2.cu): the FP64 step's parameters (dxm, dym all
-// zero: read in place), n R and the moments of the reference state that the
-// storage subtracts (zero for FP64 storage).
+// BF16-deviation storage (rlbm_io2.cu): the FP64 step's parameters, n R and the
+// moments of the reference state that the storage subtracts (zero for FP64 storage).
 struct Io2Params {
   Fused64Params b;
   double ref;
   double mref[9];
 };
-cudaError_t launch_init2(int kind, bool bf, const Io2Params& p, FieldPtrs f, void* cur, void* ccur, cudaStream_t s);
-cudaError_t launch_moments2(int kind, bool bf, const Io2Params& p, const void* prev, const void* cprev, MomentOut mo,
-                            cudaStream_t s);
+// The init writes S_0 into cur (ccur) and marks other, the buffer that the first step
+// writes (BF16-deviation storage: its coefficients); the read-out pulls prev, or,
+// where prev (cprev) carries the mark, reads cur in place.
+cudaError_t launch_init2(int kind, bool bf, const Io2Params& p, FieldPtrs f, void* cur, void* ccur, void* other,
+                         cudaStream_t s);
+cudaError_t launch_moments2(int kind, bool bf, const Io2Params& p, const void* prev, const void* cprev,
+                            const void* cur, const void* ccur, MomentOut mo, cudaStream_t s);
 
 // FP64 step of small lattices, several lanes a site (rlbm_lanes64.cu).  tab:
 // second order rows of kRowLanes2 (0..8 momentum products, 10..19 w_i J_k,
@@ -339,9 +342,10 @@ struct IoO3Params {
   double nref;
   double mref[9];
 };
-cudaError_t launch_init_o3c(int kind, bool f64, const IoO3Params& p, FieldPtrs f, void* cur, cudaStream_t s);
-cudaError_t launch_moments_o3c(int kind, bool f64, const IoO3Params& p, const void* prev, MomentOut mo,
-                               cudaStream_t s);
+cudaError_t launch_init_o3c(int kind, bool f64, const IoO3Params& p, FieldPtrs f, void* cur, void* other,
+                            cudaStream_t s);
+cudaError_t launch_moments_o3c(int kind, bool f64, const IoO3Params& p, const void* prev, const void* cur,
+                               MomentOut mo, cudaStream_t s);
 
 // kind 5, 6, 7: groups {1,2,5,6,7,9,10,11,12,13,15}, {2,3,5,6,7,8,9,10,11,13,15},
 // {1,2,3,6,7,8,9,10,11,13,15}; 8, 9, 10: {8,15,20,24,26,27,28,30,36,37,42},

@@ -3,8 +3,8 @@
 // evaluate the equilibrium and the moment sums once a reflection orbit
 // (rlbm_fused64.cuh), so that the FP64 pipe, which bounds them, has about a
 // third to a fifth of the work; and the init writes S_0 alone: a read-out right
-// after it reads S_0 in place (displacement tables of zeros) instead of pulling
-// a shifted copy S_{-1}.
+// after it reads S_0 in place (mark_unwritten) instead of pulling a shifted copy
+// S_{-1}.
 #pragma once
 
 #include "rlbm_fused64.cuh"

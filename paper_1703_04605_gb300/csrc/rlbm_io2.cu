@@ -16,14 +16,15 @@ struct PullBF {
   unsigned pitch;
   int x, y, Nx, Ny;
   const int *dxm, *dym;
+  int mask;
 };
 
 template <class Def, int I>
 __device__ __forceinline__ double pull64(const PullBF& q) {
   constexpr int nx = Def::F.nx[I], ny = Def::F.ny[I], g = Def::F.grp[I], mult = Def::F.mult[I];
   constexpr int word = Def::B.word[I], half = Def::B.half[I];
-  const unsigned xs = (unsigned)wrap_sub(q.x, q.dxm[nx + kMaxDisp], q.Nx);
-  const unsigned ys = (unsigned)wrap_sub(q.y, q.dym[ny + kMaxDisp], q.Ny);
+  const unsigned xs = (unsigned)wrap_sub(q.x, q.dxm[nx + kMaxDisp] & q.mask, q.Nx);
+  const unsigned ys = (unsigned)wrap_sub(q.y, q.dym[ny + kMaxDisp] & q.mask, q.Ny);
   const unsigned idx = ys * q.pitch + xs;
   const uint2 c = __ldg(q.cin + idx + q.plane * g);
   const unsigned h = __ldg(q.fin + 2 * (size_t)idx + half + 2 * q.plane * word);
@@ -113,7 +114,8 @@ __device__ __forceinline__ void init_all(std::integer_sequence<int, Ks...>, cons
 
 template <class Def, bool BF>
 __global__ void __launch_bounds__(128) init2_kernel(const __grid_constant__ Io2Params p, FieldPtrs fd,
-                                                    void* __restrict__ cur, uint2* __restrict__ ccur) {
+                                                    void* __restrict__ cur, uint2* __restrict__ ccur,
+                                                    void* __restrict__ other) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned fl = 0;
   if (s < p.b.Nx * p.b.Ny) {
@@ -127,9 +129,11 @@ __global__ void __launch_bounds__(128) init2_kernel(const __grid_constant__ Io2P
     if constexpr (BF) {
       const PutBF put{static_cast<unsigned*>(cur) + here, (size_t)p.b.plane};
       init_all<Def>(Orb{}, p, r, put, ccur + here);
+      if (s == 0) mark_unwritten(static_cast<uint2*>(other));
     } else {
       const PutPlain<double> put{static_cast<double*>(cur) + here, (size_t)p.b.plane};
       init_all<Def>(Orb{}, p, r, put, nullptr);
+      if (s == 0) mark_unwritten(static_cast<double*>(other));
     }
   }
   report(fl, p.b.err);
@@ -138,7 +142,9 @@ __global__ void __launch_bounds__(128) init2_kernel(const __grid_constant__ Io2P
 template <class Def, bool BF>
 __global__ void __launch_bounds__(64, 8) moments2_kernel(const __grid_constant__ Io2Params p,
                                                          const void* __restrict__ prev,
-                                                         const uint2* __restrict__ cprev, MomentOut mo) {
+                                                         const uint2* __restrict__ cprev,
+                                                         const void* __restrict__ cur,
+                                                         const uint2* __restrict__ ccur, MomentOut mo) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned fl = 0;
   const long long N = (long long)p.b.Nx * p.b.Ny;
@@ -147,16 +153,20 @@ __global__ void __launch_bounds__(64, 8) moments2_kernel(const __grid_constant__
     site_of(s, p.b.Nx, x, y);
     double m[9];
     using Orb = std::make_integer_sequence<int, Def::O.K>;
-    if constexpr (BF)
+    if constexpr (BF) {
+      const bool here = is_unwritten(cprev);
       acc64_all<Def>(Orb{},
-                     PullBF{static_cast<const unsigned short*>(prev), cprev, (size_t)p.b.plane, (unsigned)p.b.pitch, x,
-                            y, p.b.Nx, p.b.Ny, p.b.dxm, p.b.dym},
+                     PullBF{static_cast<const unsigned short*>(here ? cur : prev), here ? ccur : cprev,
+                            (size_t)p.b.plane, (unsigned)p.b.pitch, x, y, p.b.Nx, p.b.Ny, p.b.dxm, p.b.dym,
+                            here ? 0 : -1},
                      p.b.gm, m);
-    else
+    } else {
+      const bool here = is_unwritten(static_cast<const double*>(prev));
       acc64_all<Def>(Orb{},
-                     Pull64{static_cast<const double*>(prev), (size_t)p.b.plane, (unsigned)p.b.pitch, x, y, p.b.Nx,
-                            p.b.Ny, p.b.dxm, p.b.dym},
+                     Pull64{static_cast<const double*>(here ? cur : prev), (size_t)p.b.plane, (unsigned)p.b.pitch, x,
+                            y, p.b.Nx, p.b.Ny, p.b.dxm, p.b.dym, here ? 0 : -1},
                      p.b.gm, m);
+    }
 #pragma unroll
     for (int k = 0; k < 9; ++k) m[k] += p.mref[k];
     const Macro<double> o = solve_site_f64_seeded(m, p.b.sc, p.b.rt64, p.b.rt32, fl);
@@ -166,36 +176,39 @@ __global__ void __launch_bounds__(64, 8) moments2_kernel(const __grid_constant__
 }
 
 template <class Def>
-cudaError_t init2(bool bf, const Io2Params& p, FieldPtrs f, void* cur, void* ccur, cudaStream_t s) {
+cudaError_t init2(bool bf, const Io2Params& p, FieldPtrs f, void* cur, void* ccur, void* other, cudaStream_t s) {
   const unsigned grid = (unsigned)(((long long)p.b.Nx * p.b.Ny + 127) / 128);
-  if (bf) init2_kernel<Def, true><<<grid, 128, 0, s>>>(p, f, cur, static_cast<uint2*>(ccur));
-  else init2_kernel<Def, false><<<grid, 128, 0, s>>>(p, f, cur, nullptr);
+  if (bf) init2_kernel<Def, true><<<grid, 128, 0, s>>>(p, f, cur, static_cast<uint2*>(ccur), other);
+  else init2_kernel<Def, false><<<grid, 128, 0, s>>>(p, f, cur, nullptr, other);
   return cudaGetLastError();
 }
 
 template <class Def>
-cudaError_t moments2(bool bf, const Io2Params& p, const void* prev, const void* cprev, MomentOut mo, cudaStream_t s) {
+cudaError_t moments2(bool bf, const Io2Params& p, const void* prev, const void* cprev, const void* cur,
+                     const void* ccur, MomentOut mo, cudaStream_t s) {
   const unsigned grid = (unsigned)(((long long)p.b.Nx * p.b.Ny + 63) / 64);
-  if (bf) moments2_kernel<Def, true><<<grid, 64, 0, s>>>(p, prev, static_cast<const uint2*>(cprev), mo);
-  else moments2_kernel<Def, false><<<grid, 64, 0, s>>>(p, prev, nullptr, mo);
+  if (bf) moments2_kernel<Def, true><<<grid, 64, 0, s>>>(p, prev, static_cast<const uint2*>(cprev), cur,
+                                                           static_cast<const uint2*>(ccur), mo);
+  else moments2_kernel<Def, false><<<grid, 64, 0, s>>>(p, prev, nullptr, cur, nullptr, mo);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_init2(int kind, bool bf, const Io2Params& p, FieldPtrs f, void* cur, void* ccur, cudaStream_t s) {
-  if (kind == 1) return init2<StencilM1>(bf, p, f, cur, ccur, s);
-  if (kind == 2) return init2<StencilG16>(bf, p, f, cur, ccur, s);
-  if (kind == 3) return init2<StencilE5>(bf, p, f, cur, ccur, s);
-  return init2<StencilS2>(bf, p, f, cur, ccur, s);
+cudaError_t launch_init2(int kind, bool bf, const Io2Params& p, FieldPtrs f, void* cur, void* ccur, void* other,
+                         cudaStream_t s) {
+  if (kind == 1) return init2<StencilM1>(bf, p, f, cur, ccur, other, s);
+  if (kind == 2) return init2<StencilG16>(bf, p, f, cur, ccur, other, s);
+  if (kind == 3) return init2<StencilE5>(bf, p, f, cur, ccur, other, s);
+  return init2<StencilS2>(bf, p, f, cur, ccur, other, s);
 }
 
-cudaError_t launch_moments2(int kind, bool bf, const Io2Params& p, const void* prev, const void* cprev, MomentOut mo,
-                            cudaStream_t s) {
-  if (kind == 1) return moments2<StencilM1>(bf, p, prev, cprev, mo, s);
-  if (kind == 2) return moments2<StencilG16>(bf, p, prev, cprev, mo, s);
-  if (kind == 3) return moments2<StencilE5>(bf, p, prev, cprev, mo, s);
-  return moments2<StencilS2>(bf, p, prev, cprev, mo, s);
+cudaError_t launch_moments2(int kind, bool bf, const Io2Params& p, const void* prev, const void* cprev,
+                            const void* cur, const void* ccur, MomentOut mo, cudaStream_t s) {
+  if (kind == 1) return moments2<StencilM1>(bf, p, prev, cprev, cur, ccur, mo, s);
+  if (kind == 2) return moments2<StencilG16>(bf, p, prev, cprev, cur, ccur, mo, s);
+  if (kind == 3) return moments2<StencilE5>(bf, p, prev, cprev, cur, ccur, mo, s);
+  return moments2<StencilS2>(bf, p, prev, cprev, cur, ccur, mo, s);
 }
 
 }  // namespace rlbm

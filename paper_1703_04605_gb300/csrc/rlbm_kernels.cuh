@@ -380,6 +380,33 @@ __device__ __forceinline__ void report(unsigned fl, unsigned* err) {
   if (any && (threadIdx.x & 31) == 0) atomicOr(err, any);
 }
 
+// ------------------------------------------------------- S_0 alone in memory
+// The state at t is the pull of S_{t-1}, the buffer that the last step read.  An
+// init that writes S_0 alone marks the other buffer instead, and a read-out that
+// finds the mark reads S_0 in place.  The first step overwrites the mark with its
+// own output, so what is read follows what has run on the device, in whatever
+// order graphs with init and steps in them are captured and replayed; a flag kept
+// by the calls on the host would not.  The mark is a signalling NaN in population
+// 0 of site 0 (BF16-deviation storage: in that site's first coefficient word),
+// which no arithmetic or conversion returns.
+constexpr unsigned kMark32 = 0x7fa5c3e1u;
+constexpr unsigned long long kMark64 = 0x7ff4a5c37fa5c3e1ull;
+
+__device__ __forceinline__ void mark_unwritten(double* p) { *reinterpret_cast<unsigned long long*>(p) = kMark64; }
+__device__ __forceinline__ void mark_unwritten(float* p) { *reinterpret_cast<unsigned*>(p) = kMark32; }
+__device__ __forceinline__ void mark_unwritten(uint2* p) { *p = make_uint2(kMark32, kMark32); }
+
+__device__ __forceinline__ bool is_unwritten(const double* p) {
+  return __ldg(reinterpret_cast<const unsigned long long*>(p)) == kMark64;
+}
+__device__ __forceinline__ bool is_unwritten(const float* p) {
+  return __ldg(reinterpret_cast<const unsigned*>(p)) == kMark32;
+}
+__device__ __forceinline__ bool is_unwritten(const uint2* p) {
+  const uint2 v = __ldg(p);
+  return v.x == kMark32 && v.y == kMark32;
+}
+
 // ------------------------------------------------------------ step kernels
 // FP64 storage and arithmetic.
 template <int QB>

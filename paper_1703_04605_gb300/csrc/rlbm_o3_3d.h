@@ -62,9 +62,10 @@ struct Fused3O3Params {
 cudaError_t launch_fused3d_o3(const Fused3O3Params& p, const void* fin, void* fout, cudaStream_t s);
 
 // FP64 arithmetic of the compiled 3D stencils (rlbm_fused64_3d.cu): the FP64
-// step, and init and read-out of both storages.  dxm, dym, dzm: displacement D at
-// [D + 6] reduced modulo the lattice (all zero: read in place); mref, ref (n R)
-// and nref: the reference state that FP32 storage subtracts.
+// step, and init and read-out of both storages (cur, other and prev as for
+// launch_init2 and launch_moments2).  dxm, dym, dzm: displacement D at [D + 6]
+// reduced modulo the lattice; mref, ref (n R) and nref: the reference state that
+// FP32 storage subtracts.
 struct C3Params {
   int Nx, Ny, Nz;
   long long pitch, zstride, plane;   // elements; zstride = pitch * Ny
@@ -87,10 +88,13 @@ struct C3Params3 : C3Params {   // third order: dual basis of the octant represe
 };
 cudaError_t launch_step3c(int kind, const C3Params2& p, const void* fin, void* fout, cudaStream_t s);
 cudaError_t launch_step3c(const C3Params3& p, const void* fin, void* fout, cudaStream_t s);
-cudaError_t launch_init3c(int kind, bool f64, const C3Params2& p, Field3Ptrs f, void* cur, cudaStream_t s);
-cudaError_t launch_init3c(bool f64, const C3Params3& p, Field3Ptrs f, void* cur, cudaStream_t s);
-cudaError_t launch_moments3c(int kind, bool f64, const C3Params2& p, const void* prev, MomentOut mo, cudaStream_t s);
-cudaError_t launch_moments3c(bool f64, const C3Params3& p, const void* prev, MomentOut mo, cudaStream_t s);
+cudaError_t launch_init3c(int kind, bool f64, const C3Params2& p, Field3Ptrs f, void* cur, void* other,
+                          cudaStream_t s);
+cudaError_t launch_init3c(bool f64, const C3Params3& p, Field3Ptrs f, void* cur, void* other, cudaStream_t s);
+cudaError_t launch_moments3c(int kind, bool f64, const C3Params2& p, const void* prev, const void* cur, MomentOut mo,
+                             cudaStream_t s);
+cudaError_t launch_moments3c(bool f64, const C3Params3& p, const void* prev, const void* cur, MomentOut mo,
+                             cudaStream_t s);
 
 cudaError_t launch_step3d_o3(rlbm_dtype dt, const Step3O3Params& p, const void* fin, void* fout, cudaStream_t s);
 cudaError_t launch_init3d_o3(rlbm_dtype dt, const Step3O3Params& p, Field3Ptrs f, void* cur, void* prev,
