@@ -9,9 +9,9 @@
 //    with one group momentum a sum: about 4 FP64 instructions a population
 //    where nine products a population take 9;
 //  * the site solve starts from FP32 iterates (Landau frame and temperature);
-//    two FP64 corrections with the FP64 residual and an FP32 inverse slope
-//    then square the FP32 error twice over, to below FP64 rounding.  FP64
-//    divisions and square roots are an FP32 seed and two Newton corrections;
+//    corrections with the FP64 residual and an FP32 inverse slope, mostly two,
+//    go on until what is left is below FP64 rounding.  FP64 divisions and
+//    square roots are an FP32 seed and two Newton corrections;
 //  * where that does not settle (or a seed is not finite) the site falls back
 //    to the all-FP64 iterations of solve_site_f64, so every state is treated,
 //    and every error bit set, as there.
@@ -99,6 +99,17 @@ __device__ __forceinline__ bool eos_seeded(double y, const SiteConsts& sc, const
   return ok;
 }
 
+// Whether FP64 corrections of the Landau frame have settled, from the lengths of
+// the last two.  Their inverse Jacobian is fixed, and off by up to about 1e-5 times
+// gamma^2, so each is shorter than the one before by about that factor and d1 (d1/d0)
+// is left: below 1e-17, a tenth of the rounding of v.  Or the last one is as short as
+// the all-FP64 iterations ask for.  (NaN: not settled.)  A limit on d1 alone left up
+// to 2e-13 at gamma = 8, where rounding leaves 2e-14.  At gamma below 1.2 one site
+// in 200 takes a third correction.
+__device__ __forceinline__ bool landau_settled(float d0, float d1) {
+  return d1 < 1e-15f || d1 * d1 < 1e-17f * d0;
+}
+
 // Site solve of FP64 storage: m = N0 Nx Ny T00 T0x T0y Txx Txy Tyy.
 __device__ __forceinline__ Macro<double> solve_site_f64_seeded(const double (&m)[9], const SiteConsts& sc,
                                                                const double* __restrict__ rt64,
@@ -141,18 +152,22 @@ __device__ __forceinline__ Macro<double> solve_site_f64_seeded(const double (&m)
     }
   }
   double Vx = vx, Vy = vy, e;
-  float d1 = 1.0f;
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
+  float d0, d1 = 0.0f;   // lengths of the last two corrections
+  auto correct = [&] {
     e = t[0] - t[1] * Vx - t[2] * Vy;
     const float Fx = (float)(t[1] - t[3] * Vx - t[4] * Vy - e * Vx);
     const float Fy = (float)(t[2] - t[4] * Vx - t[5] * Vy - e * Vy);
     const float dx = j11 * Fx + j12 * Fy, dy = j21 * Fx + j22 * Fy;
     Vx -= (double)dx;
     Vy -= (double)dy;
+    d0 = d1;
     d1 = fabsf(dx) + fabsf(dy);
-  }
-  ok = ok && d1 < 1e-10f;   // the next correction would be below 1e-15 (NaN: not ok)
+  };
+  correct();
+  correct();
+#pragma unroll 1
+  for (int it = 0; it < 4 && !landau_settled(d0, d1); ++it) correct();
+  ok = ok && landau_settled(d0, d1);
   const double v2 = Vx * Vx + Vy * Vy;
   const double s = 1.0 - v2;
   ok = ok && s > 1e-6;
