@@ -75,23 +75,27 @@ __device__ __forceinline__ Mac3 solve3_seeded(const double (&m)[14], const SiteC
     }
   }
   double V[3] = {v[0], v[1], v[2]}, e;
-  float len = 1.0f;
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
+  float d0, d1 = 0.0f;   // lengths of the last two corrections
+  auto correct = [&] {
     e = t[0] - t[1] * V[0] - t[2] * V[1] - t[3] * V[2];
     float F[3];
     F[0] = (float)(t[1] - t[4] * V[0] - t[5] * V[1] - t[6] * V[2] - e * V[0]);
     F[1] = (float)(t[2] - t[5] * V[0] - t[7] * V[1] - t[8] * V[2] - e * V[1]);
     F[2] = (float)(t[3] - t[6] * V[0] - t[8] * V[1] - t[9] * V[2] - e * V[2]);
-    len = 0.0f;
+    d0 = d1;
+    d1 = 0.0f;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const float d = J[a][0] * F[0] + J[a][1] * F[1] + J[a][2] * F[2];
       V[a] -= (double)d;
-      len += fabsf(d);
+      d1 += fabsf(d);
     }
-  }
-  ok = ok && len < 1e-10f;
+  };
+  correct();
+  correct();
+#pragma unroll 1
+  for (int it = 0; it < 4 && !landau_settled(d0, d1); ++it) correct();
+  ok = ok && landau_settled(d0, d1);
   const double v2 = V[0] * V[0] + V[1] * V[1] + V[2] * V[2];
   const double s = 1.0 - v2, hs = 0.5 * s;
   ok = ok && s > 1e-6;

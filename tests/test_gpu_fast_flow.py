@@ -1,7 +1,7 @@
 """FP64 site solve in fast flows, where the Landau frame is ill conditioned: the
 velocity of a read-out against the frame of its own moments T^ab, solved in
 extended precision.  Tolerance 1e-15 gamma^2: rounding of the residual's six
-products (6 2^-53 T^00) through the inverse Jacobian (T^00 <= (e + P) gamma^2),
+products (6 2^-53 T^00; eight in 3D) through the inverse Jacobian (T^00 <= (e + P) gamma^2),
 and of the velocity itself."""
 import numpy as np
 import pytest
@@ -53,4 +53,23 @@ def test_frame_2d(name):
     S = [[t["Txx"], t["Txy"]], [t["Txy"], t["Tyy"]]]
     ref = _frame(T00, T0, S, [m["ux"], m["uy"]])
     err = sum(np.abs((m[k] - r).astype(float)) for k, r in zip(("ux", "uy"), ref))
+    assert np.max(err / g ** 2) < 1e-15
+
+
+@pytest.mark.parametrize("name", ["M1", "O3"])
+def test_frame_3d(name):
+    from paper_1703_04605_gb300 import Lattice3D
+    st = {"M1": W.STENCIL_M1, "O3": W.STENCIL_O3}[name]
+    shape = (32, 36, 44)
+    rng = np.random.default_rng(12)
+    g, d = rng.uniform(3, 9, shape), rng.normal(size=(3,) + shape)
+    v = np.sqrt(1 - 1 / g ** 2) * d / np.sqrt((d * d).sum(0))
+    names = ("ux", "uy", "uz")
+    with Lattice3D(st["groups"], st["m"], 0.9, shape[2], shape[1], shape[0], dtype="f64", v0=st["v0"]) as lat:
+        lat.init(n=rng.uniform(0.5, 2, shape), T=rng.uniform(0.3, 3, shape), **dict(zip(names, v)))
+        m = lat.moments(A.M_UX | A.M_UY | A.M_UZ | A.M_TMN)
+    t = {k: x.astype(np.longdouble) for k, x in m.items()}
+    S = [[t["T" + "".join(sorted(a + b))] for b in "xyz"] for a in "xyz"]
+    ref = _frame(t["T00"], [t["T0" + a] for a in "xyz"], S, [m[k] for k in names])
+    err = sum(np.abs((m[k] - r).astype(float)) for k, r in zip(names, ref))
     assert np.max(err / g ** 2) < 1e-15
