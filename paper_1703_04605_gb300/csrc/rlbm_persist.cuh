@@ -41,8 +41,21 @@ __device__ __forceinline__ unsigned ld_relaxed_gpu(const unsigned* p) {
   return v;
 }
 
+// Resident blocks: those of the single-lattice kernel, but one fewer where the claim
+// loop's registers on top of the extended sums make that count spill (E5 level 1
+// 164 bytes, M1 level 2 92).  Batches of 64^2, 256^2 and 1024^2 lattices, us a step,
+// the single-lattice kernel's blocks / one fewer: E5 level 1 21.4, 76.2, 612 / 17.1,
+// 62.0, 497; M1 level 2 17.7, 59.4, 473 / 16.7, 58.1, 460; the others lose on the two
+// larger: S2 level 1 14.5, 43.8, 350 / 13.6, 45.5, 352; G1-G6 level 1 12.0, 35.0,
+// 274 / 12.0, 38.9, 296, M1 level 1 15.3, 52.4, 414 / 14.8, 54.2, 430.
 template <class Def, bool BF, int EXL>
-__global__ void __launch_bounds__(128, fused_min_blocks<Def, BF, EXL>())
+constexpr int persist_min_blocks() {
+  constexpr bool fewer = (EXL == 1 && Def::Q == 73) || (EXL == 2 && Def::Q == 58);
+  return fused_min_blocks<Def, BF, EXL>() - (fewer ? 1 : 0);
+}
+
+template <class Def, bool BF, int EXL>
+__global__ void __launch_bounds__(128, persist_min_blocks<Def, BF, EXL>())
     persist_kernel(const __grid_constant__ PersistParams pp) {
   __shared__ FusedParams sp;
   constexpr int KEEP = FusedForms<Def, BF, EXL>::keep;
