@@ -181,13 +181,12 @@ __global__ void __launch_bounds__(Cfg::TB, Cfg::BLOCKS) fused3d_kernel(const __g
 }
 
 template <class Cfg>
+constexpr int smem_of = Cfg::KEEP * Cfg::TB * (int)sizeof(float);
+
+template <class Cfg>
 cudaError_t launch_fused3d_cfg(const Fused3Params& p, const void* fin, void* fout, cudaStream_t s) {
-  constexpr int smem = Cfg::KEEP * Cfg::TB * (int)sizeof(float);
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(fused3d_kernel<Cfg>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (attr != cudaSuccess) return attr;
   const unsigned grid = (unsigned)(((long long)p.Nx * p.Ny * p.Nz + Cfg::TB - 1) / Cfg::TB);
-  fused3d_kernel<Cfg><<<grid, Cfg::TB, smem, s>>>(p, static_cast<const float*>(fin), static_cast<float*>(fout));
+  fused3d_kernel<Cfg><<<grid, Cfg::TB, smem_of<Cfg>, s>>>(p, static_cast<const float*>(fin), static_cast<float*>(fout));
   return cudaGetLastError();
 }
 
@@ -197,7 +196,30 @@ cudaError_t launch_fused3d_impl(const Fused3Params& p, const void* fin, void* fo
   return launch_fused3d_cfg<Cfg>(p, fin, fout, s);
 }
 
+// The opt-in to more shared memory than a kernel gets by default (48 KB: only M1's
+// blocks of 256 threads need it).  It belongs to the current device, so every
+// context asks for it when it is created; nothing is remembered between contexts.
+template <class Cfg>
+cudaError_t prepare_cfg() {
+  if (smem_of<Cfg> <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(fused3d_kernel<Cfg>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_of<Cfg>);
+}
+template <class Cfg>
+cudaError_t prepare_impl() {
+  const cudaError_t e = prepare_cfg<Small3<Cfg>>();
+  return e != cudaSuccess ? e : prepare_cfg<Cfg>();
+}
+
 }  // namespace
+
+cudaError_t prepare_fused3d(int kind) {
+  switch (kind) {
+    case 1: return prepare_impl<Cfg3<Stencil3M1>>();
+    case 2: return prepare_impl<Cfg3<Stencil3G16>>();
+    case 3: return prepare_impl<Cfg3<Stencil3E5>>();
+    default: return prepare_impl<Cfg3<Stencil3S2>>();
+  }
+}
 
 cudaError_t launch_fused3d(int kind, const Fused3Params& p, const void* fin, void* fout, cudaStream_t s) {
   switch (kind) {

@@ -431,6 +431,10 @@ rlbm_status rlbm3_create(const rlbm_stencil* st, double m, double tau, int Nx, i
     c->c2.reset(new C3Params2);
     fill_c2(c.get());
     if (dtype == RLBM_F32 && halo_wide(c.get())) c->fused = c->kind;
+    if (c->fused && (e = prepare_fused3d(c->fused)) != cudaSuccess) {
+      release3(c.get());
+      return fail3(nullptr, RLBM_ECUDA, std::string("step kernel: ") + cudaGetErrorString(e));
+    }
   }
   set_reference3(c.get(), 1.0);
   *out = c.release();

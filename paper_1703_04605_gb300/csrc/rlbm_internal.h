@@ -416,6 +416,8 @@ struct Fused3Params {
 };
 
 // kind 1..4: groups {5,12,14,17,21,26}, {1..6}, {1,14,49,51,60,70}, {3,9,10,14,17,21}
+// Once for every context, on its device, before the first launch_fused3d.
+cudaError_t prepare_fused3d(int kind);
 cudaError_t launch_fused3d(int kind, const Fused3Params& p, const void* fin, void* fout, cudaStream_t s);
 
 cudaError_t launch_step3d(rlbm_dtype dt, const Step3Params& p, const void* fin, void* fout, cudaStream_t s);
