@@ -45,8 +45,8 @@ struct Cfg3<Stencil3G16> {
   static constexpr bool KEEP_PLANE = true;
 };
 
-// Lattices of at most 200 sites an SM (152 SMs): blocks of 64 threads, so that the
-// sites are on all of the SMs.  Such a step is bound by the latency of one pass, and
+// Lattices of at most 200 sites an SM: blocks of 64 threads, so that the sites are
+// on all of the SMs.  Such a step is bound by the latency of one pass, and
 // by the loads that an SM's warps share.  us a step, Cfg3's block / 64 threads:
 // 17^3 M1 10.3 / 8.2, E5 12.3 / 11.5; 23^3 M1 10.3 / 8.2; 27^3 G16 8.2 / 6.2, S2 9.3 /
 // 8.2; 31^3 S2 10.3 / 9.3, E5 14.4 / 12.8 (32 threads: 12.3, but 17^3 12.3).  Above, at
@@ -55,7 +55,7 @@ template <class C>
 struct Small3 : C {
   static constexpr int TB = 64, BLOCKS = C::BLOCKS * C::TB / 64;
 };
-constexpr long long kSmall3 = 152 * 200;
+constexpr long long kSmall3 = 200;   // sites an SM
 
 // The projections of App. B at a site, without their normalisations (in p.gf).
 struct Proj3 {
@@ -191,8 +191,8 @@ cudaError_t launch_fused3d_cfg(const Fused3Params& p, const void* fin, void* fou
 }
 
 template <class Cfg>
-cudaError_t launch_fused3d_impl(const Fused3Params& p, const void* fin, void* fout, cudaStream_t s) {
-  if ((long long)p.Nx * p.Ny * p.Nz <= kSmall3) return launch_fused3d_cfg<Small3<Cfg>>(p, fin, fout, s);
+cudaError_t launch_fused3d_impl(bool small, const Fused3Params& p, const void* fin, void* fout, cudaStream_t s) {
+  if (small) return launch_fused3d_cfg<Small3<Cfg>>(p, fin, fout, s);
   return launch_fused3d_cfg<Cfg>(p, fin, fout, s);
 }
 
@@ -205,28 +205,29 @@ cudaError_t prepare_cfg() {
   return cudaFuncSetAttribute(fused3d_kernel<Cfg>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_of<Cfg>);
 }
 template <class Cfg>
-cudaError_t prepare_impl() {
-  const cudaError_t e = prepare_cfg<Small3<Cfg>>();
-  return e != cudaSuccess ? e : prepare_cfg<Cfg>();
+cudaError_t prepare_impl(bool small) {
+  return small ? prepare_cfg<Small3<Cfg>>() : prepare_cfg<Cfg>();
 }
 
 }  // namespace
 
-cudaError_t prepare_fused3d(int kind) {
+bool fused3d_small(long long nsite) { return nsite <= kSmall3 * sm_count(); }
+
+cudaError_t prepare_fused3d(int kind, bool small) {
   switch (kind) {
-    case 1: return prepare_impl<Cfg3<Stencil3M1>>();
-    case 2: return prepare_impl<Cfg3<Stencil3G16>>();
-    case 3: return prepare_impl<Cfg3<Stencil3E5>>();
-    default: return prepare_impl<Cfg3<Stencil3S2>>();
+    case 1: return prepare_impl<Cfg3<Stencil3M1>>(small);
+    case 2: return prepare_impl<Cfg3<Stencil3G16>>(small);
+    case 3: return prepare_impl<Cfg3<Stencil3E5>>(small);
+    default: return prepare_impl<Cfg3<Stencil3S2>>(small);
   }
 }
 
-cudaError_t launch_fused3d(int kind, const Fused3Params& p, const void* fin, void* fout, cudaStream_t s) {
+cudaError_t launch_fused3d(int kind, bool small, const Fused3Params& p, const void* fin, void* fout, cudaStream_t s) {
   switch (kind) {
-    case 1: return launch_fused3d_impl<Cfg3<Stencil3M1>>(p, fin, fout, s);
-    case 2: return launch_fused3d_impl<Cfg3<Stencil3G16>>(p, fin, fout, s);
-    case 3: return launch_fused3d_impl<Cfg3<Stencil3E5>>(p, fin, fout, s);
-    default: return launch_fused3d_impl<Cfg3<Stencil3S2>>(p, fin, fout, s);
+    case 1: return launch_fused3d_impl<Cfg3<Stencil3M1>>(small, p, fin, fout, s);
+    case 2: return launch_fused3d_impl<Cfg3<Stencil3G16>>(small, p, fin, fout, s);
+    case 3: return launch_fused3d_impl<Cfg3<Stencil3E5>>(small, p, fin, fout, s);
+    default: return launch_fused3d_impl<Cfg3<Stencil3S2>>(small, p, fin, fout, s);
   }
 }
 

@@ -131,7 +131,7 @@ static void fill_params(rlbm_ctx* c, StepParams<CT>* p) {
   fill_pop_table<CT>(c->sb, c->Nx, c->Ny, &p->pt);
 }
 
-static int sm_count() {
+int rlbm::sm_count() {
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return 1;

@@ -44,6 +44,7 @@ struct rlbm_ctx3 {
   Step3Params p{};
   int fused = 0;               // 0 generic kernel; 1..4: {5,12,14,17,21,26}, {1..6},
                                // {1,14,49,51,60,70}, {3,9,10,14,17,21} (FP32)
+  bool small = false;          // the compiled kernel in blocks for a small lattice
   Fused3Params fp{};
   // third-order (eleven-group) stencils: the dual-basis tables and the
   // kernel parameters (q.b mirrors p at every launch)
@@ -431,7 +432,8 @@ rlbm_status rlbm3_create(const rlbm_stencil* st, double m, double tau, int Nx, i
     c->c2.reset(new C3Params2);
     fill_c2(c.get());
     if (dtype == RLBM_F32 && halo_wide(c.get())) c->fused = c->kind;
-    if (c->fused && (e = prepare_fused3d(c->fused)) != cudaSuccess) {
+    c->small = fused3d_small((long long)nsite);
+    if (c->fused && (e = prepare_fused3d(c->fused, c->small)) != cudaSuccess) {
       release3(c.get());
       return fail3(nullptr, RLBM_ECUDA, std::string("step kernel: ") + cudaGetErrorString(e));
     }
@@ -492,7 +494,7 @@ rlbm_status rlbm3_step(rlbm_ctx3* c, int nsteps) {
     else if (c->c3 && c->dtype == RLBM_F64) e = launch_step3c(*c->c3, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
     else if (c->c2 && c->dtype == RLBM_F64) e = launch_step3c(c->kind, *c->c2, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
     else if (c->order == 3) e = launch_step3d_o3(c->dtype, c->q, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
-    else if (c->fused) e = launch_fused3d(c->fused, c->fp, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
+    else if (c->fused) e = launch_fused3d(c->fused, c->small, c->fp, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
     else e = launch_step3d(c->dtype, c->p, c->buf[c->cur], c->buf[1 - c->cur], c->stream);
     if (e != cudaSuccess) return cuda_fail3(c, e, "step launch");
     c->cur = 1 - c->cur;

@@ -415,10 +415,15 @@ struct Fused3Params {
   unsigned* err;
 };
 
-// kind 1..4: groups {5,12,14,17,21,26}, {1..6}, {1,14,49,51,60,70}, {3,9,10,14,17,21}
-// Once for every context, on its device, before the first launch_fused3d.
-cudaError_t prepare_fused3d(int kind);
-cudaError_t launch_fused3d(int kind, const Fused3Params& p, const void* fin, void* fout, cudaStream_t s);
+// kind 1..4: groups {5,12,14,17,21,26}, {1..6}, {1,14,49,51,60,70}, {3,9,10,14,17,21};
+// small: in blocks of 64 threads (fused3d_small of the lattice's sites).
+// prepare_fused3d once for every context, on its device, before the first launch.
+bool fused3d_small(long long nsite);
+cudaError_t prepare_fused3d(int kind, bool small);
+cudaError_t launch_fused3d(int kind, bool small, const Fused3Params& p, const void* fin, void* fout, cudaStream_t s);
+
+// SMs of the current device (1 if it cannot be asked).
+int sm_count();
 
 cudaError_t launch_step3d(rlbm_dtype dt, const Step3Params& p, const void* fin, void* fout, cudaStream_t s);
 cudaError_t launch_init3d(rlbm_dtype dt, const Step3Params& p, Field3Ptrs f, void* cur, void* prev,

@@ -18,3 +18,10 @@ def test_attributes_are_not_set_once_for_the_process():
             assert "static" not in statement and "call_once" not in statement, (path, statement)
             calls += 1
     assert calls > 0
+
+
+def test_size_rules_ask_for_the_sm_count():
+    """Rules on sites an SM take the count of the device, not that of one chip."""
+    for path in glob.glob(os.path.join(CSRC, "*")):
+        code = re.sub(r"//[^\n]*", "", open(path).read())
+        assert not re.search(r"\b(148|152)\s*\*|\*\s*(148|152)\b", code), path
