@@ -306,10 +306,18 @@ def fp64_alu(mlups, key):
             "flop_source": "ncu FP64 instruction counts (profiles/fp64_kernels_alu_1024.md)"}
 
 
-def kernel_name(dtype, variant):
-    stencil = {1: "5,12,14,17,21,26", 2: "1,2,3,4,5,6", 3: "1,14,49,51,60,70", 4: "3,9,10,14,17,21"}.get(variant)
+COMPILED = {1: "5,12,14,17,21,26", 2: "1,2,3,4,5,6", 3: "1,14,49,51,60,70", 4: "3,9,10,14,17,21"}
+
+
+def kernel_name(dtype, variant, groups, sites, sms=None):
+    """Step kernel of a second-order 2D lattice (variant: info()["kernel"], which FP64 lattices leave 0)."""
     if dtype == "f64":
-        return "fused_f64_kernel<StencilDef<5,12,14,17,21,26>>"
+        import torch
+        if sites <= 32 * (sms or torch.cuda.get_device_properties(0).multi_processor_count):
+            return "lanes64_kernel"
+        g = ",".join(str(k) for k in sorted(groups))
+        return "fused_f64_kernel<StencilDef<%s>>" % g if g in COMPILED.values() else "step_f64_kernel"
+    stencil = COMPILED.get(variant)
     if stencil is None:
         return "step_f32_kernel<64>"
     return "fused_f32_kernel<StencilDef<%s>, %s>" % (stencil, "true" if dtype == "bf16dev" else "false")
@@ -651,7 +659,7 @@ def run_blast(args):
                          "frac": achieved / peak, "peak_kind": peak_kind,
                          "traffic": (profiled_traffic("fused_bf16_kernel_blast_8192.md", FUSED_E5_SOURCES)
                                      if N == 8192 and info["kernel"] == 3 else None),
-                         "kernel": kernel_name("bf16dev", info["kernel"]),
+                         "kernel": kernel_name("bf16dev", info["kernel"], st["groups"], sites),
                          "bytes_per_site": info["bytes_per_site"],
                          "frac_incl_coefficients": (info["bytes_per_site"] + info["extra_bytes_per_site"]) * sites
                          / (ms / 1e3) / 1e9 / peak},
@@ -1022,7 +1030,7 @@ def main():
                      "frac": achieved / peak,
                      "traffic": (profiled_traffic("fused_f32_kernel_random_flow_4096.md", FUSED_SOURCES)
                                  if args.dtype == "f32" and side == N_SIDE else None),
-                     "kernel": kernel_name(args.dtype, info["kernel"]), "peak_kind": peak_kind,
+                     "kernel": kernel_name(args.dtype, info["kernel"], st["groups"], sites), "peak_kind": peak_kind,
                      "bytes_per_site": info["bytes_per_site"]},
         "gpu_launches": args.steps,
         "clocks": clk.summary(),
