@@ -81,18 +81,14 @@ __device__ __forceinline__ void o3_acc_orbit(const float (&d)[Def::Q], float (&s
   }
 }
 
-// the pulled values of the collision pass: kept in registers since the
-// moment pass, or pulled again (two-pass form; L1/L2 hits)
+// where the collision pass takes the values from: shared memory, or pulled again
+// (L1/L2 hits)
 struct O3Repull {
   const float* keep;   // the thread's column of kept values
   const float* fin;
   long long plane, pitch;
   int x, y, Nx, Ny;
 };
-template <class Def, int I>
-__device__ __forceinline__ float o3_pop(const float (&d)[Def::Q]) {
-  return d[I];
-}
 // Populations that stay in shared memory between the passes: o3_keep of those
 // with n_x and n_y nonzero (their addresses cost most), the others are pulled
 // again.  Slot of population i, -1: pulled again.
@@ -134,8 +130,8 @@ __device__ __forceinline__ float o3_pop(const O3Repull& r) {
 
 // d_i + (p_i.U/(p_i^0 tau)) (e - d_i), stored at the site; the weight is
 // (U0 - v0 (n_x U_x + n_y U_y))/tau.
-template <class Def, int I, class Pops>
-__device__ __forceinline__ void o3_relax(const Pops& d, float e, float a0, float ax, float ay,
+template <class Def, int I>
+__device__ __forceinline__ void o3_relax(const O3Repull& d, float e, float a0, float ax, float ay,
                                          float* __restrict__ out, long long plane) {
   constexpr int nx = Def::F.nx[I], ny = Def::F.ny[I];
   float om = a0;
@@ -155,32 +151,32 @@ __device__ __forceinline__ float class_sum(MonoList<W...>, MonoList<E...>, const
 
 // Relaxation of the members of reflection orbit K with equilibrium parts E (even
 // in n_x and n_y), X, Y (odd in one) and Z (odd in both).
-template <class Def, int K, class Pops>
-__device__ __forceinline__ void o3_relax_orbit(const Pops& d, float E, float X, float Y, float Z, float a0, float ax,
+template <class Def, int K>
+__device__ __forceinline__ void o3_relax_orbit(const O3Repull& d, float E, float X, float Y, float Z, float a0, float ax,
                                                float ay, float* __restrict__ out, long long plane) {
   constexpr int kind = Def::O.kind[K];
   constexpr int i0 = Def::O.idx[K][0], i1 = Def::O.idx[K][1], i2 = Def::O.idx[K][2], i3 = Def::O.idx[K][3];
   if constexpr (kind == 1) {
-    o3_relax<Def, i0, Pops>(d, E, a0, ax, ay, out, plane);
+    o3_relax<Def, i0>(d, E, a0, ax, ay, out, plane);
   } else if constexpr (kind == 2) {
-    o3_relax<Def, i0, Pops>(d, E + X, a0, ax, ay, out, plane);
-    o3_relax<Def, i1, Pops>(d, E - X, a0, ax, ay, out, plane);
+    o3_relax<Def, i0>(d, E + X, a0, ax, ay, out, plane);
+    o3_relax<Def, i1>(d, E - X, a0, ax, ay, out, plane);
   } else if constexpr (kind == 3) {
-    o3_relax<Def, i0, Pops>(d, E + Y, a0, ax, ay, out, plane);
-    o3_relax<Def, i2, Pops>(d, E - Y, a0, ax, ay, out, plane);
+    o3_relax<Def, i0>(d, E + Y, a0, ax, ay, out, plane);
+    o3_relax<Def, i2>(d, E - Y, a0, ax, ay, out, plane);
   } else {
     const float EP = E + Z, EM = E - Z, XP = X + Y, XM = X - Y;
-    o3_relax<Def, i0, Pops>(d, EP + XP, a0, ax, ay, out, plane);   // (+, +)
-    o3_relax<Def, i1, Pops>(d, EM - XM, a0, ax, ay, out, plane);   // (-, +)
-    o3_relax<Def, i2, Pops>(d, EM + XM, a0, ax, ay, out, plane);   // (+, -)
-    o3_relax<Def, i3, Pops>(d, EP - XP, a0, ax, ay, out, plane);   // (-, -)
+    o3_relax<Def, i0>(d, EP + XP, a0, ax, ay, out, plane);   // (+, +)
+    o3_relax<Def, i1>(d, EM - XM, a0, ax, ay, out, plane);   // (-, +)
+    o3_relax<Def, i2>(d, EM + XM, a0, ax, ay, out, plane);   // (+, -)
+    o3_relax<Def, i3>(d, EP - XP, a0, ax, ay, out, plane);   // (-, -)
   }
 }
 
 // Equilibrium and relaxation of the orbits (a_x, a_y), a_x >= a_y, and of their
 // exchanged ones (rlbm_o3.cuh).
-template <class Def, int K, class Pops>
-__device__ __forceinline__ void o3_collide_orbit(const Pops& d, const float (&e)[kO3Mono], float nd,
+template <class Def, int K>
+__device__ __forceinline__ void o3_collide_orbit(const O3Repull& d, const float (&e)[kO3Mono], float nd,
                                                  float a0, float ax, float ay, float* __restrict__ out,
                                                  long long plane, const FusedO3Params& p) {
   constexpr int nx = Def::O.ax[K], ny = Def::O.ay[K];
@@ -193,12 +189,12 @@ __device__ __forceinline__ void o3_collide_orbit(const Pops& d, const float (&e)
     if constexpr (nx != 0 && ny != 0) Z = class_sum(O3OddXY{}, O3OddXY{}, w, e, 0.0f);
     if constexpr (nx != 0) X = class_sum(O3OddX{}, O3OddX{}, w, e, 0.0f);
     if constexpr (ny != 0) Y = class_sum(O3OddY{}, O3OddY{}, w, e, 0.0f);
-    o3_relax_orbit<Def, K, Pops>(d, class_sum(O3Even{}, O3Even{}, w, e, both), X, Y, Z, a0, ax, ay, out, plane);
+    o3_relax_orbit<Def, K>(d, class_sum(O3Even{}, O3Even{}, w, e, both), X, Y, Z, a0, ax, ay, out, plane);
     if constexpr (KX != K) {
       X = Y = 0.0f;
       if constexpr (ny != 0) X = class_sum(O3OddY{}, O3OddX{}, w, e, 0.0f);
       if constexpr (nx != 0) Y = class_sum(O3OddX{}, O3OddY{}, w, e, 0.0f);
-      o3_relax_orbit<Def, KX, Pops>(d, class_sum(O3EvenX{}, O3Even{}, w, e, both), X, Y, Z, a0, ax, ay, out, plane);
+      o3_relax_orbit<Def, KX>(d, class_sum(O3EvenX{}, O3Even{}, w, e, both), X, Y, Z, a0, ax, ay, out, plane);
     }
   }
 }
@@ -223,11 +219,11 @@ __device__ __forceinline__ void o3_acc_all(std::integer_sequence<int, Ks...>, co
   (o3_acc_orbit<Def, Ks>(d, s, M, p), ...);
 }
 
-template <class Def, class Pops, int... Ks>
-__device__ __forceinline__ void o3_collide_all(std::integer_sequence<int, Ks...>, const Pops& d,
+template <class Def, int... Ks>
+__device__ __forceinline__ void o3_collide_all(std::integer_sequence<int, Ks...>, const O3Repull& d,
                                                const float (&e)[kO3Mono], float nd, float a0, float ax, float ay,
                                                float* __restrict__ out, long long plane, const FusedO3Params& p) {
-  (o3_collide_orbit<Def, Ks, Pops>(d, e, nd, a0, ax, ay, out, plane, p), ...);
+  (o3_collide_orbit<Def, Ks>(d, e, nd, a0, ax, ay, out, plane, p), ...);
 }
 
 // Two passes over the populations: the moment pass pulls each value and folds it
@@ -240,12 +236,10 @@ __device__ __forceinline__ void o3_collide_all(std::integer_sequence<int, Ks...>
 //   Q = 99:  0 x 4 803; 40 x 5 724; 48 x 5 717; 56 x 5 729
 //   Q = 133: 0 x 3 1238; 60 x 4 1045; 80 x 4 1048; 96 x 4 1057; 80 x 5 1270
 //   Q = 149: 0 x 3 1271; 60 x 4 1187; 80 x 4 1147; 96 x 4 1137; 80 x 5 1460
-// One pass (all values in registers, four blocks, 70-90 bytes spilled) was 4 %
-// slower than 0 x 4.  Results are the same bit for bit.  With the constants of
+// One pass over values held in registers (four blocks, 70-90 bytes spilled) was
+// 4 % slower than 0 x 4.  Results are the same bit for bit.  With the constants of
 // exchanged orbits shared (o3_collide_orbit): Q = 100 731 -> 705, Q = 99 719 -> 715,
 // Q = 133 1048 -> 1001, Q = 149 1143 -> 1098; 0.66-0.70 of the copy bandwidth.
-constexpr bool O3_TWO_PASS = true;
-
 template <class Def>
 constexpr int o3_min_blocks() {
   return Def::Q <= 104 ? 5 : 4;
@@ -266,29 +260,24 @@ __global__ void __launch_bounds__(128, o3_min_blocks<Def>()) fused_o3_kernel(con
 #pragma unroll
     for (int k = 0; k < 9; ++k) M[k] = 0.0f;
     using Orb = std::make_integer_sequence<int, Def::O.K>;
-    constexpr bool two_pass = O3_TWO_PASS;
-    float d[two_pass ? 1 : Def::Q];
-    if constexpr (two_pass) {
-      float dd[Def::Q];
-      o3_load_all<Def>(std::make_integer_sequence<int, Def::Q>{}, dd, fin, p.plane, p.pitch, x, y, p.Nx, p.Ny);
-      o3_keep_all<Def>(std::make_integer_sequence<int, Def::Q>{}, dd, kept + threadIdx.x);
-      o3_acc_all<Def>(Orb{}, dd, s, M, p);
-    } else {
-      o3_load_all<Def>(std::make_integer_sequence<int, Def::Q>{}, d, fin, p.plane, p.pitch, x, y, p.Nx, p.Ny);
+    {
+      using Seq = std::make_integer_sequence<int, Def::Q>;
+      float d[Def::Q];
+      o3_load_all<Def>(Seq{}, d, fin, p.plane, p.pitch, x, y, p.Nx, p.Ny);
+      o3_keep_all<Def>(Seq{}, d, kept + threadIdx.x);
       o3_acc_all<Def>(Orb{}, d, s, M, p);
     }
     const SplitSite ss = split_solve(p, M, fl);
     // e_l = n dmu_l in the small quantities dU, dT, dR, U_x, U_y (no cancellation)
     float e[kO3Mono];
     o3_deviations<float>(p.mb, p.c, ss.n, ss.U0, ss.Ux, ss.Uy, ss.dg, ss.dR, ss.Td, ss.T, ss.R, e);
+    // the second pass pulls again: hide that its addresses are the first's
     asm volatile("" : "+r"(x), "+r"(y) : : "memory");
     const float Ux = ss.Ux, Uy = ss.Uy;
     const float a0 = ss.U0 * p.inv_tau, ax = p.v0 * Ux * p.inv_tau, ay = p.v0 * Uy * p.inv_tau;
     float* out = fout + (long long)y * p.pitch + x;
-    if constexpr (two_pass)
-      o3_collide_all<Def>(Orb{}, O3Repull{kept + threadIdx.x, fin, p.plane, p.pitch, x, y, p.Nx, p.Ny}, e, ss.nd, a0, ax, ay, out,
-                          p.plane, p);
-    else o3_collide_all<Def>(Orb{}, d, e, ss.nd, a0, ax, ay, out, p.plane, p);
+    o3_collide_all<Def>(Orb{}, O3Repull{kept + threadIdx.x, fin, p.plane, p.pitch, x, y, p.Nx, p.Ny}, e, ss.nd, a0, ax,
+                        ay, out, p.plane, p);
   }
   report(fl, p.err);
 }
