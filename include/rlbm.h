@@ -59,7 +59,9 @@ typedef enum {
                         compiled maximum)                                      */
 } rlbm_status;
 
-/* Population storage.  Arithmetic: F64 computes everything in FP64.  F32
+/* Population storage.  Arithmetic: F64 computes everything in FP64 (on
+ * compiled stencils the site solve starts from FP32 iterates and is corrected
+ * with FP64 residuals until what is left is below FP64 rounding).  F32
  * and BF16_DEV accumulate the moments in FP32, solve the Landau frame in
  * FP32 and the EOS by FP32 Newton iterations finished by one FP64 Newton
  * step with the FP64 R(zeta) table (the only FP64 work of their step).
@@ -110,7 +112,9 @@ typedef struct {
                                {8,15,20,24,26,27,28,30,36,37,42},
                                {4,10,15,20,24,26,27,28,30,36,37},
                                {4,8,14,15,16,17,18,21,22,23,26} (FP32
-                               storage, lattice at least a halo wide)          */
+                               storage, lattice at least a halo wide; FP64
+                               lattices report 0, although the same stencils
+                               have compiled FP64 kernels)                     */
   int order;                /* expansion order of f^eq: 2 or 3               */
   int extended_sums;        /* level of extended-precision moment sums of the
                                FP32 step, 0..2 (rlbm_set_extended_sums)      */
@@ -300,9 +304,12 @@ rlbm_status rlbm_batch_tuning(rlbm_ctx* const* ctxs, int count, int* steps_per_g
  * stencil (every vector of the six Table I orbits, signed n_z), all three
  * velocity components and the 14 polynomials of App. A (any six-group
  * stencil): FP64 storage (f_i), or FP32 storage of
- * d_i = f_i - r_i with FP32 accumulation; the site solve (Landau frame by
- * Newton iteration on the three velocities, Eq. 20; EOS, Eq. 28) is FP64.
- * Fields are [Nz][Ny][Nx] arrays, x fastest.  A separate context type. */
+ * d_i = f_i - r_i with FP32 accumulation.  The site solve (Landau frame by
+ * Newton iteration on the three velocities, Eq. 20; EOS, Eq. 28) is FP64 for
+ * FP64 storage.  For FP32 storage the kernels compiled for a stencil solve the
+ * Landau frame in FP32 and the EOS by FP32 Newton iterations finished by one
+ * FP64 Newton step, as in two dimensions; the table-driven kernels finish
+ * both with an FP64 Newton step.  Fields are [Nz][Ny][Nx] arrays, x fastest.  A separate context type. */
 typedef struct rlbm_ctx3 rlbm_ctx3;
 
 typedef struct {
@@ -317,8 +324,11 @@ typedef struct {
   int kernel;               /* step kernel: 0 generic; 1..4 compiled for the
                                stencils {5,12,14,17,21,26}, {1..6},
                                {1,14,49,51,60,70}, {3,9,10,14,17,21} (FP32
-                               storage, lattice at least a halo wide); 0 for
-                               every third-order stencil                      */
+                               storage, lattice at least a halo wide); 0 also
+                               for FP64 lattices and for third-order stencils,
+                               although those four and the third-order set
+                               {1,2,5,6,7,9,10,11,12,13,15} have compiled
+                               kernels there                                  */
   int order;                /* expansion order of f^eq: 2 or 3 (eleven groups:
                                the thirty-monomial third-order equilibrium)   */
 } rlbm3_info;

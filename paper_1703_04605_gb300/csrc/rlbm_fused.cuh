@@ -589,7 +589,9 @@ struct FusedForms {
   // with: level 1 G1-G6 275 / 249, S2 320 / 295, E5 469 / 461, M1 358 / 359;
   // level 2 M1 412 / 390, G1-G6 298 / 285, S2 392 / 331, E5 not faster.  The plain
   // FP32 and the BF16 kernels run 1-5 % slower that way: they are bound by
-  // bandwidth and by instruction issue, not by the warps in flight.
+  // bandwidth and by instruction issue, not by the warps in flight.  The counts
+  // are the fastest measured of those that spill little; a stencil of another Q
+  // keeps none.
   static constexpr int keep = EXL == 1 ? (Q == 49 ? 40 : Q == 39 ? 32 : Q == 73 ? 12 : Q == 58 ? 6 : 0)
                             : EXL == 2 ? (Q == 49 ? 20 : Q == 39 ? 12 : Q == 58 ? 12 : 0)
                                        : 0;
@@ -1047,18 +1049,15 @@ __global__ void __launch_bounds__(128, fused_min_blocks<Def, BF, EXL>()) fused_f
   report(fl, p.err);
 }
 
-// Steps of one lattice are chained, measured (us a step, chained against not):
-// 512^2 M1 FP32 22.0 / 24.6, BF16 29.8 / 31.5, G1-G6 15.4 / 18.3, S2 19.0 / 20.7;
-// 2048^2 M1 297 / 301, S2 BF16 334 / 349; 4096^2 M1 1179 / 1191.  The one kernel
-// that loses on large lattices is E5's FP32 one, which is at the bandwidth and
-// whose loads are slower off the read-only path: 255^2 9.5 / 12.1, 383^2 16.8 /
-// 18.5, 512^2 31.6 / 32.8, 601^2 47.0 / 47.9, but 727^2 67.2 / 66.1, 853^2 87.4 /
-// 86.1, 1023^2 124.8 / 123.6, 2048^2 403 / 391.  It is chained up to 3 2^17 sites
-// (627^2), where the launch saved still counts for more.
 // Entry point of the step kernel of a stencil, for CUDA graph kernel nodes
 // (rlbm_batch_step); the node's grid is (Nx Ny + 127)/128 blocks of 128.
 // mode: 0 FP32, 1 BF16 deviation, 2 / 3 FP32 with extended moment sums of
-// level 1 / 2.
+// level 1 / 2.  The nodes have full edges, so a chained kernel's waits are empty
+// there; its coherent loads are the faster ones all the same, us a step of 8
+// lattices of 256^2 and 4 of 1024^2, coherent / read-only: M1 44.4, 302 / 45.7, 304;
+// G1-G6 35.7, 206 / 35.7, 214; S2 39.1, 263 / 40.5, 278; BF16 M1 60.4, 393 / 60.5,
+// 392, G1-G6 42.8, 282 / 43.4, 277, S2 52.1, 344 / 54.0, 356; level 1 M1 47.2, 365 /
+// 49.1, 379, S2 41.9, 298 / 43.8, 313.
 template <class Def>
 const void* fused_kernel_fn_impl(int mode) {
   return mode == 1 ? (const void*)&fused_f32_kernel<Def, true>
@@ -1067,6 +1066,14 @@ const void* fused_kernel_fn_impl(int mode) {
                      : (const void*)&fused_f32_kernel<Def, false, 0, Def::Q != 73>;
 }
 
+// Steps of one lattice are chained, measured (us a step, chained against not):
+// 512^2 M1 FP32 22.0 / 24.6, BF16 29.8 / 31.5, G1-G6 15.4 / 18.3, S2 19.0 / 20.7;
+// 2048^2 M1 297 / 301, S2 BF16 334 / 349; 4096^2 M1 1187 / 1191.  The one kernel
+// that loses on large lattices is E5's FP32 one, which is at the bandwidth and
+// whose loads are slower off the read-only path: 255^2 9.5 / 12.1, 383^2 16.8 /
+// 18.5, 512^2 31.6 / 32.8, 601^2 47.0 / 47.9, but 727^2 67.2 / 66.1, 853^2 87.4 /
+// 86.1, 1023^2 124.8 / 123.6, 2048^2 403 / 391.  It is chained up to 3 2^17 sites
+// (627^2), where the launch saved still counts for more.
 template <class Def>
 cudaError_t launch_fused_impl(const FusedParams& p, const void* fin, void* fout, int mode, cudaStream_t s) {
   const long long nsite = (long long)p.Nx * p.Ny;

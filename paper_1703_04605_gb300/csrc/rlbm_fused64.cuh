@@ -353,7 +353,7 @@ __device__ __forceinline__ void relax64_orbit(const Pull64& q, const Relax64& r,
   }
 }
 
-// ------------------------------------------------------ four lanes a site
+// ------------------------------------------------ equilibrium, second order
 // Equilibrium coefficients of one group from the projections r.
 __device__ __forceinline__ void group_coeffs64(const double* a, const double (&r)[10], double (&c)[6]) {
   c[0] = fma(a[0], r[0], fma(a[1], r[1], fma(a[2], r[4], fma(a[3], r[7], a[4] * r[8]))));
