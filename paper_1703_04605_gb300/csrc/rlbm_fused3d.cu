@@ -48,8 +48,8 @@ struct Cfg3<Stencil3G16> {
 // Lattices of at most 200 sites an SM: blocks of 64 threads, so that the sites are
 // on all of the SMs.  Such a step is bound by the latency of one pass, and
 // by the loads that an SM's warps share.  us a step, Cfg3's block / 64 threads:
-// 17^3 M1 10.3 / 8.2, E5 12.3 / 11.5; 23^3 M1 10.3 / 8.2; 27^3 G16 8.2 / 6.2, S2 9.3 /
-// 8.2; 31^3 S2 10.3 / 9.3, E5 14.4 / 12.8 (32 threads: 12.3, but 17^3 12.3).  Above, at
+// 17^3 M1 10.3 / 8.2, E5 12.3 / 11.9; 23^3 M1 10.3 / 8.2; 27^3 G16 8.2 / 6.2, S2 9.3 /
+// 8.2; 31^3 S2 10.3 / 9.3, E5 14.4 / 12.6 (32 threads: 12.3, but 17^3 12.3).  Above, at
 // 33^3, M1 loses (10.3 / 12.3) and the others are even.
 template <class C>
 struct Small3 : C {

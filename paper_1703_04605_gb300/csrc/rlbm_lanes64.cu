@@ -11,9 +11,9 @@
 // L = 8, 566 at L = 4 (Q = 58).  L is the largest of 32, 16, 8 and 4 that gives
 // no more warps than sub-partitions (lanes64_for); a lattice with more sites than
 // that holds at L = 4 is faster with a lane a site.  Measured, us a step, M1
-// (Q = 58): 64 sites 13.8, 800 20.1, 2432 25.2, 4864 28.7 against 30.8 for
+// (Q = 58): 64 sites 14.0, 800 19.7, 2432 24.5, 4864 28.1 against 30.8 for
 // fused_f64_kernel up to 9728 (800 x 1 on step_f64_kernel: 77); third order
-// (Q = 100) 64 sites 22.2, 800 23.4, 2432 33.9, 4864 48.2 against 57.5.  What is
+// (Q = 100) 64 sites 22.2, 800 23.3, 2432 33.7, 4864 48.1 against 55.3.  What is
 // left is the solve's serial FP64 chain and the latency of one pass over memory.
 #include "rlbm_fused64.cuh"
 #include "rlbm_o3.cuh"
